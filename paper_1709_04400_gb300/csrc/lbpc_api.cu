@@ -123,6 +123,40 @@ bool is_dirichlet_ok(int v) { return v == LBPC_T_NONE || v == LBPC_T_DIRICHLET; 
 double critical_T(const lbpc_params* p) { return 0.0778 * p->a / (0.45724 * p->b * p->R); }
 double kappa_of(double om) { return 0.37464 + 1.54226 * om - 0.26992 * om * om; }
 
+void fill_flow_rates(lbpc::FlowRates<float>& c, const lbpc_params* p) {
+  for (int k = 0; k < 9; ++k) {
+    c.s_f[k] = (float)p->s_f[k];
+    c.hf[k] = (float)(1.0 - 0.5 * p->s_f[k]);
+  }
+}
+template <class R> void fill_flow_rates(lbpc::FoldedFlowRates<R>& c, const lbpc_params* p) {
+  static const int moment[6] = {1, 2, 4, 6, 7, 8};
+  static const double scale[6] = {1.0 / 36, 1.0 / 36, 1.0 / 12, 1.0 / 12, 1.0 / 4, 1.0 / 4};
+  double B[6];
+  for (int k = 0; k < 6; ++k) {
+    const double s = p->s_f[moment[k]];
+    B[k] = s * scale[k];
+    c.A[k] = (R)((1.0 - s) * scale[k]);
+    c.H[k] = (R)((1.0 - 0.5 * s) * scale[k] * (moment[k] == 7 ? 2.0 : 1.0));
+  }
+  for (int k = 0; k < 4; ++k) c.B[k] = (R)B[k + 2];
+  for (int k = 0; k < 2; ++k) c.E[k] = (R)(3.0 * B[k]);
+  // m1_eq and m2_eq hold -2 rho and rho: x0 = u0 + 4 (u2 - u1), axes u0 - u1 - 2 u2, diagonals u0 + 2 u1 + u2
+  c.w0 = (R)(1.0 / 9 + 4.0 * (B[1] + 2.0 * B[0]));
+  c.wa = (R)(1.0 / 9 + 2.0 * (B[0] - B[1]));
+  c.wd = (R)(1.0 / 9 - 4.0 * B[0] + B[1]);
+  const double kappa = kappa_of(p->omega), kdiff = (1.0 / p->s_g[3] - 0.5) / 3.0;
+  c.kappa1 = (R)(1.0 + kappa);
+  c.kappa_Tc = (R)(kappa / critical_T(p));
+  c.G12 = (R)(-p->G / 12.0);
+  c.qG144 = (R)(12.0 * p->sigma / (1.0 / p->s_f[1] - 0.5) * p->G * p->G / 144.0);
+  c.inv_cV12 = (R)(1.0 / (12.0 * p->cV));
+  c.lambda2 = (R)(2.0 * p->lambda);
+  c.kdiff6 = (R)(kdiff / 6.0);
+  c.chi6 = (R)((p->chi - kdiff) / 6.0);
+  c.chi144 = (R)(p->chi / 144.0);
+}
+
 template <class R> void fill_coefs(lbpc::Coefs<R>& c, const lbpc_params* p) {
   for (int k = 0; k < 4; ++k) c.T_bc[k] = (R)p->T_bc[k];
   c.T_strip = (R)p->T_strip;
@@ -134,10 +168,9 @@ template <class R> void fill_coefs(lbpc::Coefs<R>& c, const lbpc_params* p) {
   c.G = (R)p->G;
   c.kappa = (R)kappa_of(p->omega);
   for (int k = 0; k < 9; ++k) {
-    c.s_f[k] = (R)p->s_f[k];
     c.s_g[k] = (R)p->s_g[k];
-    c.hf[k] = (R)(1.0 - 0.5 * p->s_f[k]);
   }
+  fill_flow_rates(c.flow, p);
   c.lambda = (R)p->lambda;
   c.chi = (R)p->chi;
   c.cV = (R)p->cV;
@@ -426,12 +459,12 @@ static cudaError_t launch_step(lbpc_ctx* c, cudaEvent_t* ev) {
 }
 
 static int step_kernel_count(const lbpc_ctx* c) {
-  return use_fused(c) ? (c->dp.buoyancy == 1 ? 2 : 1) : lbpc::split_kernel_count(c->dp);
+  return use_fused(c) ? (c->dp.buoyancy == 1 ? 2 : 1) : lbpc::split_kernel_count(c->dp, c->p.prec);
 }
 
 static const char* step_kernel_name(const lbpc_ctx* c, int k) {
   if (use_fused(c)) return k == 0 ? "k_fused" : (k == 1 ? "k_finish" : "");
-  return lbpc::split_kernel_name(k);
+  return lbpc::split_kernel_name(c->p.prec, k);
 }
 
 LBPC_API lbpc_status lbpc_set_path(lbpc_ctx* c, int32_t path) {

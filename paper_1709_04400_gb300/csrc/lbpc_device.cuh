@@ -25,16 +25,38 @@ __host__ __device__ constexpr int EY(int a) { return a == 2 || a == 5 || a == 6 
 
 // Real-valued parameters in the arithmetic type of a kernel, folded on the host, so that a kernel
 // never converts between FP64 and FP32 (on GB300 those conversions run at the FP64 rate).
+//
+// The flow relaxation in the form each arithmetic uses. Binary32 takes it in increments with the rates as
+// they are. Binary64 and double-word arithmetic, whose step is bound by the number of such operations, take
+// it with the back-transform's scale c of each moment folded in: c = (1/36, 1/36, 1/12, 1/12, 1/4, 1/4) for the
+// moments (e, eps, qx, qy, pxx, pxy).
+template <class R> struct FlowRates {
+  R s_f[9];
+  R hf[9];      // 1 - s_f[k]/2, the forcing weights of (I - Lambda/2) S_F
+};
+template <class R> struct FoldedFlowRates {
+  R A[6], H[6];  // (1 - s) c, (1 - s/2) c; H[4] (pxx) carries the factor 2 of its S_F
+  R B[4];        // s c of qx, qy, pxx, pxy
+  R E[2];        // 3 s c of e and eps: the weights of rho v^2 in their equilibria
+  R w0, wa, wd;  // weights of rho in f0, in f1..f4 and in f5..f8 that the zeroth moment and those equilibria add
+  // further constants of these steps, with the scales of the unscaled differences (12 grad, 6 lap) folded in
+  R kappa1, kappa_Tc;           // 1 + kappa, kappa / T_c
+  R G12, qG144, inv_cV12;       // -G/12, qG2/144, 1/(12 c_V)
+  R lambda2, kdiff6, chi6, chi144;  // 2 lambda, kdiff/6, (chi - kdiff)/6, chi/144
+};
+template <> struct FlowRates<double> : FoldedFlowRates<double> {};
+template <> struct FlowRates<dw> : FoldedFlowRates<dw> {};
+
 template <class R> struct Coefs {
   R T_bc[4], T_strip;
   R rho_bc_lo, rho_bc_hi;
   R a, b, R_gas, G, kappa;
-  R s_f[9], s_g[9];
+  R s_g[9];
+  FlowRates<R> flow;
   R lambda, chi, cV, kdiff;  // kdiff = (1/s_g3 - 1/2) c_s^2
   R gx, gy, G_wall;
   R c3, c5;     // (1 - s3/2) s4, (1 - s5/2) s6 of Eqs. 54-55
   R inv_Tc;     // 1 / T_c
-  R hf[9];      // 1 - s_f[k]/2, the forcing weights of (I - Lambda/2) S_F
   R qG2;        // 12 sigma / (1/s_e - 1/2) * G^2: Q = qcoef |F_int|^2 / psi^2 = qG2 |sum_a w psi e|^2
   R inv_cV;     // 1 / c_V
   R psi_scale;  // 2 / G: psi^2 = (2/G) (p - rho c_s^2)
@@ -176,6 +198,72 @@ template <class R, class PT> __device__ __forceinline__ void eos(R rho, R T, con
   dpdT = rho * C.R_gas * inv1 - C.a * dtheta * r2 * inv2;
 }
 
+// The same for binary64 and double-word arithmetic, arranged for the fewest operations (their step is bound by
+// the arithmetic pipe): psi^2, (dp/dT)_rho and 1/rho from one reciprocal and one reciprocal square root.
+// With u = rho R / (1 - b rho), A = a rho^2 / (1 + 2 b rho - b^2 rho^2) and h = 1 + kappa (1 - sqrt(T/T_c)):
+// p = u T - A h^2 and dp/dT = u + A h kappa / sqrt(T T_c).
+template <class R> __device__ __forceinline__ R inverse_of(R x) { return R(1) / x; }
+template <> __device__ __forceinline__ dw inverse_of<dw>(dw x) {  // binary32 reciprocal, corrected once
+  x = dw_norm(x);
+  const float r = __frcp_rn(x.hi);
+  const dw p = dw_two_prod(r, x.hi);
+  const float d = __fsub_rn(__fsub_rn(__fsub_rn(1.0f, p.hi), p.lo), __fmul_rn(r, x.lo));  // 1 - r x
+  return dw_fast_two_sum(r, __fmul_rn(d, r));
+}
+// Binary64 reciprocal and roots from the hardware's approximations (relative error below 2^-20) by one step
+// of the third-order iteration (Householder 1970; for the reciprocal, r (1 + e + e^2) with e = 1 - x r): the
+// error left is of the order of e^3, below binary64's rounding. 3 and 5 operations of the pipe that bounds the
+// step; the compiler's correctly rounded forms take more. Arguments are normal numbers here (a state outside
+// the equation of state's range is reported by classify, whatever these return for it).
+template <> __device__ __forceinline__ double inverse_of<double>(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+// 1/sqrt(x) and sqrt(x) of x > 0
+__device__ __forceinline__ void roots_of(double x, double& inv_root, double& root) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double s = x * y;
+  const double e = fma(-s, y, 1.0);
+  const double pe = fma(0.375, e, 0.5) * e;
+  inv_root = fma(pe, y, y);
+  root = fma(pe, s, s);
+}
+__device__ __forceinline__ void roots_of(dw x, dw& inv_root, dw& root) {
+  inv_root = rsqrt(x);
+  root = x * inv_root;
+}
+// psi = sqrt(max(psi^2, 0)), a NaN counting as 0; the tests of the binary64 form run on the integer pipe.
+template <class R> __device__ __forceinline__ R psi_of(R psi2) { return sqrt(fmax(psi2, R(0))); }
+template <> __device__ __forceinline__ double psi_of<double>(double psi2) {
+  const long long b = __double_as_longlong(psi2);
+  double inv_root, root;
+  roots_of(psi2, inv_root, root);
+  return b >= 0x0010000000000000LL && b < 0x7ff0000000000000LL ? root : (b == 0x7ff0000000000000LL ? psi2 : 0.0);
+}
+template <class R, class PT>
+__device__ __forceinline__ R eos_psi_squared(R rho, R T, const PT& P, R& dpdT, R& inv_rho) {
+  const Coefs<R>& C = coefs<R>(P);
+  const R t = T * C.inv_Tc;
+  R rs, sq;
+  roots_of(t, rs, sq);
+  const R h = C.flow.kappa1 - C.kappa * sq;
+  const R br = C.b * rho;
+  const R d1 = R(1) - br;
+  const R d2 = br * (R(2) - br) + R(1);
+  const R d12 = d1 * d2;
+  const R r = inverse_of(rho * d12);
+  inv_rho = d12 * r;
+  const R z = rho * (rho * r);  // rho / d12
+  const R u = (d2 * z) * C.R_gas;
+  const R Ah = ((C.a * rho) * (d1 * z)) * h;
+  dpdT = u + (Ah * rs) * C.flow.kappa_Tc;
+  const R p = u * T - Ah * h;
+  return C.psi_scale * (p - rho * R(1.0 / 3.0));
+}
+
 // ------------------------------------------------------------------------------------------------
 // zeroth moments and the pseudopotential in binary32
 // ------------------------------------------------------------------------------------------------
@@ -221,6 +309,19 @@ template <class R>
 __device__ __forceinline__ R psi_squared(R p, R dpdT, R Tlo, R rho, const Coefs<R>& C) {
   if constexpr (sizeof(R) == 4) return C.psi_scale * ((p + dpdT * Tlo) - rho * R(1.0 / 3.0));
   else return C.psi_scale * (p - rho * R(1.0 / 3.0));
+}
+
+// psi^2 and (dp/dT)_rho of a node in the form its arithmetic takes (Tlo: the residual of a binary32 T).
+template <class R, class PT>
+__device__ __forceinline__ R node_psi_squared(R rho, R T, R Tlo, const PT& P, R& dpdT) {
+  if constexpr (sizeof(R) == 4) {
+    R p;
+    eos(rho, T, P, p, dpdT);
+    return psi_squared(p, dpdT, Tlo, rho, coefs<R>(P));
+  } else {
+    R inv_rho;
+    return eos_psi_squared(rho, T, P, dpdT, inv_rho);
+  }
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -470,6 +571,66 @@ __device__ __forceinline__ void wall_force_store(double* wall, const PT& P, int 
 // ------------------------------------------------------------------------------------------------
 // collisions
 // ------------------------------------------------------------------------------------------------
+// Density, momentum and the non-conserved flow moments m = (e, eps, qx, qy, pxx, pxy) of f in binary64 and
+// double-word arithmetic: 24 additions, the sums and differences of opposite populations shared by all of them.
+template <class R> __device__ __forceinline__ R flow_moments(const R f[9], R& jx, R& jy, R m[6]) {
+  const R s13 = f[1] + f[3], s24 = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
+  const R d13 = f[1] - f[3], d24 = f[2] - f[4], a = f[5] - f[7], b = f[8] - f[6];
+  const R s14 = s13 + s24, s58 = s57 + s68;
+  const R c = a + b, d = a - b;
+  jx = d13 + c;
+  jy = d24 + d;
+  m[0] = s58 * 2 - s14 - f[0] * 4;
+  m[1] = f[0] * 4 - s14 * 2 + s58;
+  m[2] = c - d13 * 2;
+  m[3] = d - d24 * 2;
+  m[4] = s13 - s24;
+  m[5] = s57 - s68;
+  return f[0] + s14 + s58;
+}
+
+// Post-collision f from those moments: c_k m_k* = (1 - s) c_k m_k + s c_k m_k,eq + (1 - s/2) c_k S_F,k for the
+// six relaxed moments (FlowRates), m0* = rho and j* = j + F whatever the rates (S_F,0 = 0, m0_eq = rho,
+// m_eq,3 = j + F/2), and the back-transform. 57 binary64 instructions.
+template <class R>
+__device__ __forceinline__ void relax_flow(const R m[6], R jx, R jy, R rho, R vx, R vy, R Fx, R Fy, R Q, const Coefs<R>& C,
+                                           R f[9]) {
+  const auto& K = C.flow;
+  const R rvx = rho * vx, rvy = rho * vy;
+  const R rxx = rvx * vx, ryy = rvy * vy;
+  const R r3 = rxx + ryy;                      // rho v^2: m1_eq = 3 r3 - 2 rho, m2_eq = rho - 3 r3
+  const R xF = vx * Fx, yF = vy * Fy;
+  const R t = (xF + yF) * 6 + Q;               // S_F,1 = -S_F,2
+  // energy moments without the parts of their equilibria linear in rho, which w0, wa and wd carry
+  const R u1 = K.A[0] * m[0] + (K.E[0] * r3 + K.H[0] * t);
+  const R u2 = K.A[1] * m[1] - (K.E[1] * r3 + K.H[1] * t);
+  const R u4 = K.A[2] * m[2] - (K.B[0] * rvx + K.H[2] * Fx);
+  const R u6 = K.A[3] * m[3] - (K.B[1] * rvy + K.H[3] * Fy);
+  const R u7 = K.A[4] * m[4] + (K.B[2] * (rxx - ryy) + K.H[4] * (xF - yF));
+  const R u8 = K.A[5] * m[5] + (K.B[3] * (rvx * vy) + K.H[5] * (vx * Fy + vy * Fx));
+  const R ax = (K.wa * rho - u1) - u2 * 2;  // common to e1..e4
+  const R dg = (K.wd * rho + u2) + u1 * 2;  // common to e5..e8
+  R sx, sy, qx, qy;                         // j*/6 plus the fluxes, on the diagonals and on the axes
+  if constexpr (is_dw_t<R>::value) {        // a scale by 2 costs a double-word less than one by 3
+    const R w3 = (jx + Fx) * R(1.0 / 6.0), w5 = (jy + Fy) * R(1.0 / 6.0);
+    sx = w3 + u4; qx = w3 - u4 * 2;
+    sy = w5 + u6; qy = w5 - u6 * 2;
+  } else {
+    sx = (jx + Fx) * R(1.0 / 6.0) + u4; qx = sx - u4 * 3;
+    sy = (jy + Fy) * R(1.0 / 6.0) + u6; qy = sy - u6 * 3;
+  }
+  const R a1 = ax + u7, a2 = ax - u7, g5 = dg + u8, g6 = dg - u8, k5 = sx + sy, k6 = sy - sx;
+  f[0] = K.w0 * rho + (u2 - u1) * 4;
+  f[1] = a1 + qx;
+  f[2] = a2 + qy;
+  f[3] = a1 - qx;
+  f[4] = a2 - qy;
+  f[5] = g5 + k5;
+  f[6] = g6 + k6;
+  f[7] = g5 - k5;
+  f[8] = g6 - k6;
+}
+
 // Flow MRT collision with forcing (reading of the improved pseudopotential model, Refs. [13,29]):
 // m* = m - Lambda (m - m_eq) + (I - Lambda/2) S_F, S_F with the sigma term Q in the energy moments.
 //
@@ -478,14 +639,14 @@ __device__ __forceinline__ void wall_force_store(double* wall, const PT& P, int 
 // times at the scale of the populations, and the roundings of the opposite pair e_a, -e_a differ, which
 // moves momentum at random. The non-equilibrium parts m - m_eq of the energy and stress moments come
 // from the populations' exact deviations from their rest-state ratios (see density_of), not from moments
-// of size about 2 rho that cancel. Binary64 and double-word arithmetic rebuild f* from m*.
+// of size about 2 rho that cancel. Binary64 and double-word arithmetic rebuild f* from m* (relax_flow).
 template <class R, class PT>
 __device__ __forceinline__ void collide_flow(R f[9], R rho, R vx, R vy, R Fx, R Fy, R Q, const PT& P) {
   const Coefs<R>& C = coefs<R>(P);
-  const R vxx = vx * vx, vyy = vy * vy;
-  const R v2 = vxx + vyy;
-  const R vF = vx * Fx + vy * Fy;
   if constexpr (sizeof(R) == 4) {
+    const R vxx = vx * vx, vyy = vy * vy;
+    const R v2 = vxx + vyy;
+    const R vF = vx * Fx + vy * Fy;
     const R q = f[0] * 0.25f;
     const R d1 = f[1] - q, d2 = f[2] - q, d3 = f[3] - q, d4 = f[4] - q;
     const R d5 = fmaf(4.f, f[5], -q), d6 = fmaf(4.f, f[6], -q), d7 = fmaf(4.f, f[7], -q), d8 = fmaf(4.f, f[8], -q);
@@ -501,37 +662,50 @@ __device__ __forceinline__ void collide_flow(R f[9], R rho, R vx, R vy, R Fx, R 
     dm[0] = R(0);  // S_F,0 = 0 and m0_eq = rho
     dm[3] = Fx;    // j* = j + F whatever s_j (m_eq,3 = j + F/2)
     dm[5] = Fy;
-    dm[1] = C.hf[1] * (vF * 6 + Q) - C.s_f[1] * (e_dev - r3v2);  // m1 - m1_eq = (m1 + 2 rho) - 3 rho v^2
-    dm[2] = C.hf[2] * (vF * -6 - Q) - C.s_f[2] * (eps_dev + r3v2);  // m2 - m2_eq = (m2 - rho) + 3 rho v^2
-    dm[4] = C.hf[4] * -Fx - C.s_f[4] * (qx + rho * vx);
-    dm[6] = C.hf[6] * -Fy - C.s_f[6] * (qy + rho * vy);
-    dm[7] = C.hf[7] * ((vx * Fx - vy * Fy) * 2) - C.s_f[7] * (pxx - rho * (vxx - vyy));
-    dm[8] = C.hf[8] * (vx * Fy + vy * Fx) - C.s_f[8] * (pxy - rho * vx * vy);
+    dm[1] = C.flow.hf[1] * (vF * 6 + Q) - C.flow.s_f[1] * (e_dev - r3v2);  // m1 - m1_eq = (m1 + 2 rho) - 3 rho v^2
+    dm[2] = C.flow.hf[2] * (vF * -6 - Q) - C.flow.s_f[2] * (eps_dev + r3v2);  // m2 - m2_eq = (m2 - rho) + 3 rho v^2
+    dm[4] = C.flow.hf[4] * -Fx - C.flow.s_f[4] * (qx + rho * vx);
+    dm[6] = C.flow.hf[6] * -Fy - C.flow.s_f[6] * (qy + rho * vy);
+    dm[7] = C.flow.hf[7] * ((vx * Fx - vy * Fy) * 2) - C.flow.s_f[7] * (pxx - rho * (vxx - vyy));
+    dm[8] = C.flow.hf[8] * (vx * Fy + vy * Fx) - C.flow.s_f[8] * (pxy - rho * vx * vy);
     from_moments(dm, df);
 #pragma unroll
     for (int a = 0; a < 9; ++a) f[a] = f[a] + df[a];
-    return;
+  } else {
+    R m[6], jx, jy;
+    flow_moments(f, jx, jy, m);
+    relax_flow(m, jx, jy, rho, vx, vy, Fx, Fy, Q, C, f);
   }
-  R m[9];
-  to_moments(f, m);
-  // conserved moments: m0* = m0 = rho (S_F,0 = 0, m0_eq = rho; rho is the caller's sum of these f) and
-  // j* = j + F whatever s_j (m_eq,3 = j + F/2)
-  m[0] = rho;
-  m[3] += Fx;
-  m[5] += Fy;
-  R meq[9], SF[9];
-  meq[1] = rho * (R(-2) + v2 * 3); SF[1] = vF * 6 + Q;
-  meq[2] = rho * (R(1) - v2 * 3);  SF[2] = vF * -6 - Q;
-  meq[4] = -rho * vx;                 SF[4] = -Fx;
-  meq[6] = -rho * vy;                 SF[6] = -Fy;
-  meq[7] = rho * (vxx - vyy);         SF[7] = (vx * Fx - vy * Fy) * 2;
-  meq[8] = rho * vx * vy;             SF[8] = vx * Fy + vy * Fx;
-#pragma unroll
-  for (int k = 1; k < 9; ++k) {
-    if (k == 3 || k == 5) continue;
-    m[k] = m[k] - C.s_f[k] * (m[k] - meq[k]) + C.hf[k] * SF[k];
-  }
-  from_moments_conserving(m, f);
+}
+
+// The thermal moments n4, n6 (the fluxes qx, qy of g) in binary64 and double-word arithmetic.
+template <class R> __device__ __forceinline__ void heat_fluxes(const R g[9], R& n4, R& n6) {
+  const R a = g[5] - g[7], b = g[8] - g[6];
+  n4 = (a + b) - (g[1] - g[3]) * 2;
+  n6 = (a - b) - (g[2] - g[4]) * 2;
+}
+
+// Post-collision g of the improved model when every rate s_k, k >= 1, is 1, from n4 and n6 alone.
+template <class R>
+__device__ __forceinline__ void relax_heat_unit(R n4, R n6, R T, R vx, R vy, R S0, R g[9]) {
+  const R TS = T + S0;
+  const R Tvx = T * vx, Tvy = T * vy;
+  const R h4 = n4 * R(1.0 / 12.0), h6 = n6 * R(1.0 / 12.0);
+  const R X = Tvx * R(5.0 / 12.0) + h4, Xd = Tvx * R(1.0 / 6.0) + h4;
+  const R Y = Tvy * R(5.0 / 12.0) + h6, Yd = Tvy * R(1.0 / 6.0) + h6;
+  const R B = TS * R(1.0 / 9.0) - T * R(1.0 / 18.0);
+  const R P1 = B + Xd, P2 = B - Xd;
+  g[1] = B + X;
+  g[3] = B - X;
+  g[2] = B + Y;
+  g[4] = B - Y;
+  g[5] = P1 + Yd;
+  g[8] = P1 - Yd;
+  g[6] = P2 + Yd;
+  g[7] = P2 - Yd;
+  // binary32 keeps the heat of the node to one rounding (see from_moments_conserving)
+  if constexpr (sizeof(R) == 4) g[0] = TS - (((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8])));
+  else g[0] = B + T * 0.5f;
 }
 
 // Thermal MRT collision of the improved model: Eq. 45 with m_eq of Eq. 53 and S = (S0, 0, ..., 0)
@@ -557,26 +731,14 @@ __device__ __forceinline__ void collide_heat(R g[9], R T, R vx, R vy, R S0, cons
     // back-transform M^{-1} n* in closed form: the axes and the diagonals share the base
     // B = (T + S0)/9 - T/18, the axes add +-X (+-Y) with X = 5 T vx/12 + n4/12, the diagonals +-X' +-Y'
     // with X' = T vx/6 + n4/12, and the rest population is B + T/2.
-    const R TS = T + S0;
-    const R Tvx = T * vx, Tvy = T * vy;
-    const R n4 = (g[1] - g[3]) * -2 + (g[5] - g[6] - g[7] + g[8]);
-    const R n6 = (g[2] - g[4]) * -2 + (g[5] + g[6] - g[7] - g[8]);
-    const R h4 = n4 * R(1.0 / 12.0), h6 = n6 * R(1.0 / 12.0);
-    const R X = Tvx * R(5.0 / 12.0) + h4, Xd = Tvx * R(1.0 / 6.0) + h4;
-    const R Y = Tvy * R(5.0 / 12.0) + h6, Yd = Tvy * R(1.0 / 6.0) + h6;
-    const R B = TS * R(1.0 / 9.0) - T * R(1.0 / 18.0);
-    const R P1 = B + Xd, P2 = B - Xd;
-    g[1] = B + X;
-    g[3] = B - X;
-    g[2] = B + Y;
-    g[4] = B - Y;
-    g[5] = P1 + Yd;
-    g[8] = P1 - Yd;
-    g[6] = P2 + Yd;
-    g[7] = P2 - Yd;
-    // binary32 keeps the heat of the node to one rounding (see from_moments_conserving)
-    if constexpr (sizeof(R) == 4) g[0] = TS - (((g[1] + g[2]) + (g[3] + g[4])) + ((g[5] + g[6]) + (g[7] + g[8])));
-    else g[0] = B + T * 0.5f;
+    R n4, n6;
+    if constexpr (sizeof(R) == 4) {
+      n4 = (g[1] - g[3]) * -2 + (g[5] - g[6] - g[7] + g[8]);
+      n6 = (g[2] - g[4]) * -2 + (g[5] + g[6] - g[7] - g[8]);
+    } else {
+      heat_fluxes(g, n4, n6);
+    }
+    relax_heat_unit(n4, n6, T, vx, vy, S0, g);
     return;
   } else if (P.heat_unit_rates) {
     // compromised model with s_k = 1 for k >= 1: every non-conserved moment relaxes to its equilibrium,

@@ -62,11 +62,11 @@ struct SplitBuffers {
   int fused_tile = 1;  // 0: 32x16, 1: 32x8, 2: 32x16 two nodes per thread, 3: 32x32 two per thread (maps match)
 };
 
-// ev: null, or split_kernel_count(P) + 1 events recorded before the first and after each kernel.
+// ev: null, or split_kernel_count(P, prec) + 1 events recorded before the first and after each kernel.
 cudaError_t split_step(const SplitBuffers& b, const DevParams& P, int prec, int cur, long long step, cudaStream_t st,
                        cudaEvent_t* ev = nullptr);
-int split_kernel_count(const DevParams& P);
-const char* split_kernel_name(int k);
+int split_kernel_count(const DevParams& P, int prec);
+const char* split_kernel_name(int prec, int k);
 cudaError_t split_init(const SplitBuffers& b, const DevParams& P, int prec, const double* rho, const double* T,
                        const double* ux, const double* uy, cudaStream_t st);
 cudaError_t split_sums(const SplitBuffers& b, const DevParams& P, int prec, int cur, cudaStream_t st);
@@ -132,7 +132,7 @@ template <class S> struct alignas(16) SegInst {
   int tiles_x;               // tiles per row
   int first;                 // the instance's first step (its source term starts from phi itself)
 };
-constexpr size_t kSegParamBytes = 32000;  // within the 32,764 bytes of kernel parameters
+constexpr size_t kSegParamBytes = 32512;  // within the 32,764 bytes of kernel parameters
 template <class S> constexpr int seg_capacity() {
   return (int)((kSegParamBytes - 32) / (sizeof(SegInst<S>) + sizeof(int))) & ~3;
 }

@@ -1,15 +1,22 @@
-// Split form of the coupled step: three node-parallel kernels per time step.
+// Split form of the coupled step: node-parallel kernels over scratch planes.
 //
+// Binary32 arithmetic, three kernels:
 //   k_macro    pull-stream + boundary closures; rho, j, T (moments), p_EOS -> psi and (dp/dT)_rho
 //              (Eq. 56); optional per-block partial sums of rho for the buoyancy reference rho_ave.
 //   k_force    psi stencil -> F = F_int + F_ads + F_b, v = (j + F/2)/rho, sigma term Q.
 //   k_collide  pull again (same closures); isotropic grad T, lap T, grad rho, div v; source phi of
 //              Eq. 28 and S0 of Eq. 46; flow MRT collide with forcing; thermal MRT collide with the
 //              corrections of Eqs. 54-55; store post-collision f*, g* (pull scheme, A/B buffers).
+// Binary64 and double-word arithmetic, two kernels: k_macro also leaves the flow moments and heat fluxes, and
+// k_collide_tile takes the force and the collisions together.
 //
-// Each kernel reads its node's stencil straight from global memory (L1/L2 serve the reuse). With
-// FP64 arithmetic the step is bound by the FP64 pipe, not by HBM, and this split computes every
-// EOS evaluation, force and velocity exactly once per node and step.
+// Each kernel reads its node's stencil straight from global memory (L1/L2 serve the reuse). With FP64
+// arithmetic the step is bound by the FP64 pipe (84 % busy in both kernels), not by HBM, so its time is its
+// count of FP64 instructions: 229 per node and step (k_macro 85, k_collide_tile 144). Three kernels that
+// pulled f and g twice and rebuilt m* from all nine moments took 283. GB300, droplet evaporation 2048^2: 1.82 ms
+// a step against 2.24 ms; 128^2 17.1 us against 20.6 us. Double-word arithmetic: 0.479 against 0.533 ms.
+#include <type_traits>
+
 #include "lbpc_device.cuh"
 #include "lbpc_internal.h"
 
@@ -64,31 +71,49 @@ template <class R> __device__ __forceinline__ R lap(const R c[3][3]) {
          (c[2][2] + c[2][0] + c[0][0] + c[0][2] - ctr * 4) * R(1.0 / 6.0);
 }
 
-template <class S, class R>
-__global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc, Planes<R> pl,
-                                                 DevParams P, long long step, int do_partials,
-                                                 double* __restrict__ partials, long long* __restrict__ status) {
+// STASH (binary64 and double-word steps): the flow moments and the heat fluxes n4, n6 go into the destination
+// buffers (planes 0..5 of fdst, 0..1 of gdst), which nothing else uses until k_collide_tile overwrites the same
+// entries of the same node with f*, g*.
+template <class S, class R, bool STASH>
+__global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc, S* __restrict__ fdst,
+                                                 S* __restrict__ gdst, Planes<R> pl, DevParams P, long long step,
+                                                 int do_partials, double* __restrict__ partials,
+                                                 long long* __restrict__ status) {
   __shared__ double red[BLOCK / 32];
-  const Coefs<R>& C = coefs<R>(P);
-  const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
+  const int t = (int)threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + t;
   double rho_d = 0.0;
   if (i < P.N) {
     const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
     R f[9], g[9];
     pull_closed<S, R>(fsrc, gsrc, P, x, y, f, g);
-    const R rho = density_of(f);
-    const R jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
-    const R jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
-    R Tlo;
+    R rho, jx, jy, Tlo, dpdT, inv_rho, psi2;
     const R T = heat_of(g, Tlo);
-    R p, dpdT, inv_rho;
-    eos(rho, T, P, p, dpdT, &inv_rho);
-    const R psi2 = psi_squared(p, dpdT, Tlo, rho, C);
+    if constexpr (sizeof(R) == 4) {
+      rho = density_of(f);
+      jx = f[1] - f[3] + f[5] - f[6] - f[7] + f[8];
+      jy = f[2] - f[4] + f[5] + f[6] - f[7] - f[8];
+      R p;
+      eos(rho, T, P, p, dpdT, &inv_rho);
+      psi2 = psi_squared(p, dpdT, Tlo, rho, coefs<R>(P));
+    } else {
+      R m[6];
+      rho = flow_moments(f, jx, jy, m);
+      psi2 = eos_psi_squared(rho, T, P, dpdT, inv_rho);
+      if (STASH) {
+#pragma unroll
+        for (int a = 0; a < 6; ++a) fdst[(long long)a * P.N + i] = m[a];
+        R n4, n6;
+        heat_fluxes(g, n4, n6);
+        gdst[i] = n4;
+        gdst[P.N + i] = n6;
+      }
+    }
     const int bad = classify(rho, T, psi2, P);
     if (bad) report(status, step, x, y, bad);
     pl.p[P_RHO][i] = rho;
     pl.p[P_T][i] = T;
-    pl.p[P_PSI][i] = sqrt(fmax(psi2, R(0)));
+    pl.p[P_PSI][i] = psi_of(psi2);
     pl.p[P_JX][i] = jx;
     pl.p[P_JY][i] = jy;
     pl.p[P_DPDT][i] = dpdT;
@@ -97,14 +122,15 @@ __global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc,
   }
   if (do_partials) {
     const double s = block_sum<BLOCK>(rho_d, red);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    if (t == 0) partials[blockIdx.x] = s;
   }
 }
 
 template <class R>
 __global__ void __launch_bounds__(BLOCK) k_force(Planes<R> pl, DevParams P, const double* __restrict__ rho_ave) {
+  const int t = (int)threadIdx.x;
   const Coefs<R>& C = coefs<R>(P);
-  const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + t;
   if (i >= P.N) return;
   const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
   const R* __restrict__ psi = pl.p[P_PSI];
@@ -139,20 +165,14 @@ __global__ void __launch_bounds__(BLOCK) k_force(Planes<R> pl, DevParams P, cons
 // BLOCK nodes, the next BLOCK threads run the source and thermal collision of the same nodes. The
 // roles share no data (both read the scratch planes), so a node's work splits into two independent
 // chains and twice as many warps hide the FP64 latency on small grids.
-//
-// BY_BLOCK = false: each block of 2 * BLOCK threads holds both roles of BLOCK nodes. BY_BLOCK = true:
-// blocks of BLOCK threads, the first half of the grid runs the flow role and the second half the
-// thermal role. Blocks start roughly in index order, so an SM then runs one role's code at a time,
-// which keeps long double-word code (LBPC_DF64) in the instruction caches.
-template <class S, class R, bool BY_BLOCK>
-__global__ void __launch_bounds__(BY_BLOCK ? BLOCK : 2 * BLOCK)
+template <class S, class R>
+__global__ void __launch_bounds__(2 * BLOCK)
     k_collide(PopBuf<S> fsrc, PopBuf<S> gsrc, PopBuf<S> fdst, PopBuf<S> gdst, Planes<R> pl, R* __restrict__ phi_prev,
               DevParams P, int first) {
   const Coefs<R>& C = coefs<R>(P);
-  const unsigned half = gridDim.x >> 1;
-  const bool heat = BY_BLOCK ? blockIdx.x >= half : threadIdx.x >= BLOCK;
-  const long long i = BY_BLOCK ? (long long)(blockIdx.x - (heat ? half : 0u)) * BLOCK + threadIdx.x
-                               : (long long)blockIdx.x * BLOCK + (threadIdx.x - (heat ? BLOCK : 0));
+  const int t = (int)threadIdx.x;
+  const bool heat = t >= BLOCK;
+  const long long i = (long long)blockIdx.x * BLOCK + (t - (heat ? BLOCK : 0));
   if (i >= P.N) return;
   const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
   const R vx = pl.p[P_VX][i], vy = pl.p[P_VY][i];
@@ -210,6 +230,180 @@ __global__ void __launch_bounds__(BY_BLOCK ? BLOCK : 2 * BLOCK)
   pop_store<S, R>(gdst, P.N, i, g, T + S0, C.wg);
 }
 
+// Source offsets of the 3x3 neighbourhood of (x, y): rows below, at and above, columns left, at and right, as
+// element offsets of a plane. interior: no neighbour lies beyond an edge.
+struct Around {
+  unsigned row[3], col[3];
+};
+__device__ __forceinline__ Around around(const DevParams& P, int x, int y, bool interior) {
+  Around n;
+  const unsigned nx = (unsigned)P.nx;
+  n.row[1] = (unsigned)y * nx;
+  n.col[1] = (unsigned)x;
+  if (interior) {
+    n.row[0] = n.row[1] - nx;
+    n.row[2] = n.row[1] + nx;
+    n.col[0] = n.col[1] - 1u;
+    n.col[2] = n.col[1] + 1u;
+  } else {
+    n.row[0] = y == 0 ? (P.yper ? (unsigned)(P.ny - 1) * nx : n.row[1]) : n.row[1] - nx;
+    n.row[2] = y == P.ny - 1 ? (P.yper ? 0u : n.row[1]) : n.row[1] + nx;
+    n.col[0] = x == 0 ? nx - 1u : n.col[1] - 1u;
+    n.col[2] = x == P.nx - 1 ? 0u : n.col[1] + 1u;
+  }
+  return n;
+}
+template <class R> __device__ __forceinline__ void gather(const R* __restrict__ X, const Around& n, R c[3][3]) {
+#pragma unroll
+  for (int j = 0; j < 3; ++j)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) c[j][k] = ldgv(X + (size_t)(n.row[j] + n.col[k]));
+}
+
+// Force and collision of the binary64 and double-word steps in one kernel over tiles of CX x CY nodes. The
+// velocities of the tile and its 1-ring go to shared memory (the force of the ring is repeated), so the force,
+// the velocity and the sigma term never visit device memory and the step is two launches. Then the two roles of
+// k_collide: the first half of the block relaxes f from the moments that k_macro left in fdst, the second half
+// evaluates the source and relaxes g from T, n4, n6 (or pulls g again where the rates are not all 1).
+//
+// The isotropic differences are taken without their common scale: d = (4 axis + diagonal)/12 and
+// lap = (4 axes + diagonals - 20 centre)/6; the 1/12 and 1/6 join a coefficient that multiplies anyway.
+template <class S, int CX, int CY>
+__global__ void __launch_bounds__(2 * CX* CY)
+    k_collide_tile(PopBuf<S> gsrc, PopBuf<S> fdst, PopBuf<S> gdst, Planes<S> pl, S* __restrict__ phi_prev, DevParams P,
+                   int first, int tiles_x, const double* __restrict__ rho_ave) {
+  using R = S;
+  constexpr int CN = CX * CY, RING = 2 * (CX + 2) + 2 * CY;
+  static_assert(RING <= CN, "one ring node per thread of the second half");
+  __shared__ R s_vx[CY + 2][CX + 2], s_vy[CY + 2][CX + 2];
+  const Coefs<R>& C = coefs<R>(P);
+  const int t = (int)threadIdx.x;
+  const bool heat = t >= CN;
+  const int x0 = (int)(blockIdx.x % (unsigned)tiles_x) * CX, y0 = (int)(blockIdx.x / (unsigned)tiles_x) * CY;
+  const bool interior = x0 >= 2 && x0 + CX + 2 <= P.nx && y0 >= 2 && y0 + CY + 2 <= P.ny;
+  // velocity node of this thread, in coordinates of the tile with its ring: the tile's own nodes, then the ring
+  int hx, hy;
+  const int q = heat ? t - CN : t;
+  if (!heat) {
+    hx = 1 + q % CX;
+    hy = 1 + q / CX;
+  } else if (q < 2 * (CX + 2)) {
+    hx = q % (CX + 2);
+    hy = q < CX + 2 ? 0 : CY + 1;
+  } else {
+    hx = (q & 1) ? CX + 1 : 0;
+    hy = 1 + (q - 2 * (CX + 2)) / 2;
+  }
+  R Fx = R(0), Fy = R(0), Q = R(0), vx = R(0), vy = R(0), rho = R(0), jx = R(0), jy = R(0);
+  if (!heat || q < RING) {
+    int x = x0 + hx - 1, y = y0 + hy - 1;
+    if (!interior) {
+      while (x < 0) x += P.nx;
+      while (x >= P.nx) x -= P.nx;
+      if (P.yper) {
+        while (y < 0) y += P.ny;
+        while (y >= P.ny) y -= P.ny;
+      } else {  // a ghost row's velocity is the edge row's
+        y = min(max(y, 0), P.ny - 1);
+      }
+    }
+    const Around n = around(P, x, y, interior);
+    const size_t i = n.row[1] + n.col[1];
+    R c[3][3];
+    gather(pl.p[P_PSI], n, c);
+    rho = ldgv(pl.p[P_RHO] + i);
+    const R inv_rho = ldgv(pl.p[P_IRHO] + i);
+    jx = ldgv(pl.p[P_JX] + i);
+    jy = ldgv(pl.p[P_JY] + i);
+    const R pc = c[1][1];
+    const R a = c[2][2] - c[0][0], b = c[0][2] - c[2][0];
+    const R sx = (c[1][2] - c[1][0]) * 4 + (a + b);
+    const R sy = (c[2][1] - c[0][1]) * 4 + (a - b);
+    const R Gp = pc * C.flow.G12;
+    Fx = Gp * sx;
+    Fy = Gp * sy;
+    if (!P.yper && y == 0 && P.ybc_lo == BC_WALL) Fy += C.G_wall * 0.5f * pc * pc;
+    if (P.buoyancy) {
+      const R dr = rho - (P.buoyancy == 1 ? R(*rho_ave) : C.rho_bc_hi);
+      Fx += dr * C.gx;
+      Fy += dr * C.gy;
+    }
+    vx = (jx + Fx * 0.5f) * inv_rho;
+    vy = (jy + Fy * 0.5f) * inv_rho;
+    s_vx[hy][hx] = vx;
+    s_vy[hy][hx] = vy;
+    if (!heat) Q = C.flow.qG144 * (sx * sx + sy * sy);
+  }
+  __syncthreads();
+  const int tx = q % CX, ty = q / CX;
+  const int x = x0 + tx, y = y0 + ty;
+  if (x >= P.nx || y >= P.ny) return;
+  const Around n = around(P, x, y, interior);
+  const size_t i = n.row[1] + n.col[1];
+  if (!heat) {
+    R m[6], f[9];
+    S* pf = fdst.p + i;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) m[a] = pf[(size_t)a * P.N];
+    relax_flow(m, jx, jy, rho, vx, vy, Fx, Fy, Q, C, f);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) pf[(size_t)a * P.N] = f[a];
+    wall_force_store(fdst.wall, P, x, y, Fx, Fy);
+    return;
+  }
+  hx = tx + 1;
+  hy = ty + 1;
+  R c[3][3];
+  gather(pl.p[P_T], n, c);
+  const R inv_rho = ldgv(pl.p[P_IRHO] + i), dpdT = ldgv(pl.p[P_DPDT] + i);
+  const R T = c[1][1];
+  const R lap6 = (((c[1][2] + c[1][0]) + (c[2][1] + c[0][1])) * 4 + ((c[2][2] + c[2][0]) + (c[0][0] + c[0][2]))) - T * 20;
+  const R gTa = c[2][2] - c[0][0], gTb = c[0][2] - c[2][0];
+  const R gTx = (c[1][2] - c[1][0]) * 4 + (gTa + gTb), gTy = (c[2][1] - c[0][1]) * 4 + (gTa - gTb);  // 12 grad T
+  // 12 div v: the diagonals of d_x vx and d_y vy share their weights
+  const R dv1 = (s_vx[hy][hx + 1] - s_vx[hy][hx - 1]) + (s_vy[hy + 1][hx] - s_vy[hy - 1][hx]);
+  const R dv2 = ((s_vx[hy + 1][hx + 1] + s_vy[hy + 1][hx + 1]) - (s_vx[hy - 1][hx - 1] + s_vy[hy - 1][hx - 1])) +
+                ((s_vx[hy - 1][hx + 1] - s_vy[hy - 1][hx + 1]) - (s_vx[hy + 1][hx - 1] - s_vy[hy + 1][hx - 1]));
+  const R div12 = dv1 * 4 + dv2;
+  vx = s_vx[hy][hx];
+  vy = s_vy[hy][hx];
+  const R inv_rcv12 = inv_rho * C.flow.inv_cV12;  // 1 / (12 rho c_V)
+  const R compress = (T * div12) * (R(1.0 / 12.0) - dpdT * inv_rcv12);
+  R phi, S0, tau_inv = R(0);
+  if (P.model == 2) {  // Gong-Cheng: Eq. 13 source, local tau_g (Sec. IV A)
+    phi = compress;
+    S0 = phi;
+    tau_inv = R(1) / ((P.lambda_mode == 0 ? C.lambda * 36 * inv_rcv12 : C.chi * 3) + R(0.5));
+  } else {
+    // phi: the underlined terms of Eq. 28 with k = (1/s_3 - 1/2) c_s^2
+    if (P.lambda_mode == 0) {
+      phi = lap6 * (C.flow.lambda2 * inv_rcv12 - C.flow.kdiff6) + compress;
+    } else {  // div(lambda grad T)/(rho c_V) = chi (lap T + grad rho . grad T / rho)
+      gather(pl.p[P_RHO], n, c);
+      const R gra = c[2][2] - c[0][0], grb = c[0][2] - c[2][0];
+      const R grx = (c[1][2] - c[1][0]) * 4 + (gra + grb), gry = (c[2][1] - c[0][1]) * 4 + (gra - grb);
+      phi = lap6 * C.flow.chi6 + ((C.flow.chi144 * inv_rho) * (grx * gTx + gry * gTy) + compress);
+    }
+    S0 = phi;
+    if (P.model == 0) {  // S0 = phi + 0.5 dt d_t phi, d_t phi ~ [phi(t) - phi(t - dt)]/dt (Eq. 46)
+      const R pp = first ? phi : phi_prev[i];
+      S0 = phi + (phi - pp) * 0.5f;
+    }
+  }
+  phi_prev[i] = phi;
+  R g[9];
+  S* pg = gdst.p + i;
+  if (P.model == 0 && P.heat_unit_rates) {
+    relax_heat_unit(pg[0], pg[P.N], T, vx, vy, S0, g);
+  } else {
+    pull<S, R>(gsrc, C.wg, P, x, y, g);
+    heat_closure(g, P, x, y);
+    collide_heat(g, T, vx, vy, S0, P, tau_inv);
+  }
+#pragma unroll
+  for (int a = 0; a < 9; ++a) pg[(size_t)a * P.N] = g[a];
+}
+
 // Fixed-order sum of the block partials: each thread accumulates a strided subset in order, then one
 // block reduction. out[k] = sum(partials[k * stride + 0 .. n)) * scale.
 __global__ void __launch_bounds__(BLOCK) k_finish(const double* __restrict__ partials, int n, int stride, int count,
@@ -229,7 +423,7 @@ template <class S>
 __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_in, const double* __restrict__ T_in,
                                                 const double* __restrict__ ux_in, const double* __restrict__ uy_in,
                                                 PopBuf<S> f, PopBuf<S> g, DevParams P) {
-  const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + (int)threadIdx.x;
   if (i >= P.N) return;
   const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
   double fv[9], gv[9];
@@ -270,7 +464,8 @@ template <class S>
 __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P,
                                                 double* __restrict__ partials, int stride) {
   __shared__ double red[BLOCK / 32];
-  const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
+  const int tid = (int)threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + tid;
   double r = 0.0, t = 0.0;
   if (i < P.N) {
     const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
@@ -280,16 +475,16 @@ __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, 
     t = g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + g[6] + g[7] + g[8];
   }
   const double sr = block_sum<BLOCK>(r, red);
-  if (threadIdx.x == 0) partials[blockIdx.x] = sr;
+  if (tid == 0) partials[blockIdx.x] = sr;
   const double st = block_sum<BLOCK>(t, red);
-  if (threadIdx.x == 0) partials[stride + blockIdx.x] = st;
+  if (tid == 0) partials[stride + blockIdx.x] = st;
 }
 
 // Post-boundary populations of the current state as FP64 [9][N] (which = 0: f, 1: g).
 template <class S>
 __global__ void __launch_bounds__(BLOCK) k_export_pops(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P, int which,
                                                        int only, double* __restrict__ out) {
-  const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + (int)threadIdx.x;
   if (i >= P.N) return;
   const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
   double f[9], g[9];
@@ -306,7 +501,7 @@ __global__ void __launch_bounds__(BLOCK) k_export_pops(PopBuf<S> fsrc, PopBuf<S>
 template <class R>
 __global__ void __launch_bounds__(BLOCK) k_export_fields(Planes<R> pl, DevParams P, double* rho, double* ux, double* uy,
                                                          double* T) {
-  const long long i = (long long)blockIdx.x * BLOCK + threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + (int)threadIdx.x;
   if (i >= P.N) return;
   if (rho) rho[i] = (double)pl.p[P_RHO][i];
   if (ux) ux[i] = (double)pl.p[P_VX][i];
@@ -330,26 +525,20 @@ template <class S> static PopBuf<S> fbuf(const SplitBuffers& b, int k) {
 }
 template <class S> static PopBuf<S> gbuf(const SplitBuffers& b, int k) { return PopBuf<S>{(S*)b.g[k], b.ref_g[k]}; }
 
-// Role layout of k_collide per storage type (both compute the same step): roles by block for the
-// long double-word code (measured 15 % faster at 2048^2), roles within a block otherwise.
-template <class S> static constexpr bool collide_by_block() { return is_dw_t<S>::value; }
-
+// The binary32 step as three kernels over scratch planes.
 template <class S, class R>
 static cudaError_t step_impl(const SplitBuffers& b, const DevParams& P, int cur, long long step, cudaStream_t st,
                              cudaEvent_t* ev) {
   const unsigned nb = blocks_for(P.N);
   Planes<R> pl = planes_of<S, R>(b);
   if (ev) cudaEventRecord(ev[0], st);
-  k_macro<S, R><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), pl, P, step, P.buoyancy == 1, b.partials, b.status);
+  k_macro<S, R, false><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), nullptr, nullptr, pl, P, step,
+                                             P.buoyancy == 1, b.partials, b.status);
   if (ev) cudaEventRecord(ev[1], st);
   k_force<R><<<nb, BLOCK, 0, st>>>(pl, P, b.scalars);
   if (ev) cudaEventRecord(ev[2], st);
-  if (collide_by_block<S>())
-    k_collide<S, R, true><<<2 * nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), fbuf<S>(b, cur ^ 1),
-                                                   gbuf<S>(b, cur ^ 1), pl, (R*)b.phi_prev, P, step == 0);
-  else
-    k_collide<S, R, false><<<nb, 2 * BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), fbuf<S>(b, cur ^ 1),
-                                                    gbuf<S>(b, cur ^ 1), pl, (R*)b.phi_prev, P, step == 0);
+  k_collide<S, R><<<nb, 2 * BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), fbuf<S>(b, cur ^ 1), gbuf<S>(b, cur ^ 1),
+                                            pl, (R*)b.phi_prev, P, step == 0);
   if (ev) cudaEventRecord(ev[3], st);
   if (P.buoyancy == 1) {
     k_finish<<<1, BLOCK, 0, st>>>(b.partials, (int)nb, 0, 1, 1.0 / (double)P.N, b.scalars);
@@ -358,19 +547,56 @@ static cudaError_t step_impl(const SplitBuffers& b, const DevParams& P, int cur,
   return cudaGetLastError();
 }
 
+// The binary64 and double-word steps as two kernels.
+template <class S>
+static cudaError_t step_wide(const SplitBuffers& b, const DevParams& P, int cur, long long step, cudaStream_t st,
+                             cudaEvent_t* ev) {
+  const unsigned nb = blocks_for(P.N);
+  Planes<S> pl = planes_of<S, S>(b);
+  const PopBuf<S> fd = fbuf<S>(b, cur ^ 1), gd = gbuf<S>(b, cur ^ 1);
+  if (ev) cudaEventRecord(ev[0], st);
+  k_macro<S, S, true><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), fd.p, gd.p, pl, P, step, P.buoyancy == 1,
+                                            b.partials, b.status);
+  if (ev) cudaEventRecord(ev[1], st);
+  auto collide = [&](auto cx, auto cy) {
+    constexpr int CX = decltype(cx)::value, CY = decltype(cy)::value;
+    const int tiles_x = (P.nx + CX - 1) / CX;
+    const unsigned tiles = (unsigned)((long long)tiles_x * ((P.ny + CY - 1) / CY));
+    k_collide_tile<S, CX, CY><<<tiles, 2 * CX * CY, 0, st>>>(gbuf<S>(b, cur), fd, gd, pl, (S*)b.phi_prev, P, step == 0,
+                                                            tiles_x, b.scalars);
+  };
+  // 16 x 8 tiles; large binary64 grids take 32 x 8, whose ring repeats less of the force (1.33 instead of 1.41 times
+  // the tile): 2048^2 1811 us a step against 1831. Below, more blocks matter more: 128^2 12.0 against 17.1 us,
+  // 350^2 64 against 69 us. In double-word arithmetic 16 x 8 is the faster at every size (2048^2 467, 471 us).
+  if (sizeof(S) == 8 && !is_dw_t<S>::value && P.N >= (1 << 20))
+    collide(std::integral_constant<int, 32>(), std::integral_constant<int, 8>());
+  else
+    collide(std::integral_constant<int, 16>(), std::integral_constant<int, 8>());
+  if (ev) cudaEventRecord(ev[2], st);
+  if (P.buoyancy == 1) {
+    k_finish<<<1, BLOCK, 0, st>>>(b.partials, (int)nb, 0, 1, 1.0 / (double)P.N, b.scalars);
+    if (ev) cudaEventRecord(ev[3], st);
+  }
+  return cudaGetLastError();
+}
+
 cudaError_t split_step(const SplitBuffers& b, const DevParams& P, int prec, int cur, long long step, cudaStream_t st,
                        cudaEvent_t* ev) {
-  if (prec == 0) return step_impl<double, double>(b, P, cur, step, st, ev);
+  if (prec == 0) return step_wide<double>(b, P, cur, step, st, ev);
   if (prec == 1) return step_impl<float, float>(b, P, cur, step, st, ev);
-  if (prec == 3) return step_impl<dw, dw>(b, P, cur, step, st, ev);
+  if (prec == 3) return step_wide<dw>(b, P, cur, step, st, ev);
   return step_impl<__half, float>(b, P, cur, step, st, ev);
 }
 
-int split_kernel_count(const DevParams& P) { return P.buoyancy == 1 ? 4 : 3; }
+static bool is_wide(int prec) { return prec == 0 || prec == 3; }  // 8-byte storage: two kernels
 
-const char* split_kernel_name(int k) {
+int split_kernel_count(const DevParams& P, int prec) { return (is_wide(prec) ? 2 : 3) + (P.buoyancy == 1); }
+
+const char* split_kernel_name(int prec, int k) {
   static const char* names[] = {"k_macro", "k_force", "k_collide", "k_finish"};
-  return (k >= 0 && k < 4) ? names[k] : "";
+  static const char* wide[] = {"k_macro", "k_collide", "k_finish"};
+  if (k < 0 || k >= (is_wide(prec) ? 3 : 4)) return "";
+  return is_wide(prec) ? wide[k] : names[k];
 }
 
 template <class S>
@@ -417,7 +643,8 @@ static cudaError_t fields_impl(const SplitBuffers& b, const DevParams& P, int cu
                                double* ux, double* uy, double* T, cudaStream_t st) {
   const unsigned nb = blocks_for(P.N);
   Planes<R> pl = planes_of<S, R>(b);
-  k_macro<S, R><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), pl, P, step, 0, b.partials, b.status);
+  k_macro<S, R, false><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), nullptr, nullptr, pl, P, step, 0,
+                                             b.partials, b.status);
   k_force<R><<<nb, BLOCK, 0, st>>>(pl, P, b.scalars);
   k_export_fields<R><<<nb, BLOCK, 0, st>>>(pl, P, rho, ux, uy, T);
   return cudaGetLastError();

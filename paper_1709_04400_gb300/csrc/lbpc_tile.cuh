@@ -205,21 +205,29 @@ __device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S
     }
     const R* fk = f[k];
     const R* gk = g[k];
-    rho[k] = density_of(fk);
-    const R jx = fk[1] - fk[3] + fk[5] - fk[6] - fk[7] + fk[8];
-    const R jy = fk[2] - fk[4] + fk[5] + fk[6] - fk[7] - fk[8];
+    R jx, jy;
+    if constexpr (sizeof(R) == 4) {
+      rho[k] = density_of(fk);
+      jx = fk[1] - fk[3] + fk[5] - fk[6] - fk[7] + fk[8];
+      jy = fk[2] - fk[4] + fk[5] + fk[6] - fk[7] - fk[8];
+    } else {  // the flow moments take the place of f until stage 3 (slots 0..5, then jx, jy)
+      R m[6];
+      rho[k] = flow_moments(fk, jx, jy, m);
+#pragma unroll
+      for (int a = 0; a < 6; ++a) f[k][a] = m[a];
+      f[k][6] = jx;
+      f[k][7] = jy;
+    }
     R Tlo;
     T[k] = heat_of(gk, Tlo);
-    R p;
-    eos(rho[k], T[k], P, p, dpdT[k]);
-    const R psi2 = psi_squared(p, dpdT[k], Tlo, rho[k], C);
+    const R psi2 = node_psi_squared(rho[k], T[k], Tlo, P, dpdT[k]);
     if (active[k]) {
       const int bad = classify(rho[k], T[k], psi2, P);
       if (bad) report(status, step_at ? *step_at : step, gx, gy, bad);  // step_at: read only to report
     }
     s_rho[ty + 2][tx + 2] = rho[k];
     s_T[ty + 2][tx + 2] = T[k];
-    s_psi[ty + 2][tx + 2] = sqrt(fmax(psi2, R(0)));
+    s_psi[ty + 2][tx + 2] = psi_of(psi2);
     s_jx[ty + 2][tx + 2] = jx;
     s_jy[ty + 2][tx + 2] = jy;
   }
@@ -249,17 +257,23 @@ __device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S
       const int x = wrap_any(x0 + hx - 2, P.nx), y = row_of(P, y0 + hy - 2);
       pull_closed<S, R, IX>(fsrc, gsrc, P, x, y, fr, gr);
     }
-    const R rr = density_of(fr);
-    R Trlo;
+    R rr, jx, jy;
+    if constexpr (sizeof(R) == 4) {
+      rr = density_of(fr);
+      jx = fr[1] - fr[3] + fr[5] - fr[6] - fr[7] + fr[8];
+      jy = fr[2] - fr[4] + fr[5] + fr[6] - fr[7] - fr[8];
+    } else {
+      R m[6];
+      rr = flow_moments(fr, jx, jy, m);
+    }
+    R Trlo, dr;
     const R Tr = heat_of(gr, Trlo);
-    R pr, dr;
-    eos(rr, Tr, P, pr, dr);
-    const R psi2 = psi_squared(pr, dr, Trlo, rr, C);
+    const R psi2 = node_psi_squared(rr, Tr, Trlo, P, dr);
     s_rho[hy][hx] = rr;
     s_T[hy][hx] = Tr;
-    s_psi[hy][hx] = sqrt(fmax(psi2, R(0)));
-    s_jx[hy][hx] = fr[1] - fr[3] + fr[5] - fr[6] - fr[7] + fr[8];
-    s_jy[hy][hx] = fr[2] - fr[4] + fr[5] + fr[6] - fr[7] - fr[8];
+    s_psi[hy][hx] = psi_of(psi2);
+    s_jx[hy][hx] = jx;
+    s_jy[hy][hx] = jy;
   }
   if (P.buoyancy == 1) {
     double own = 0.0;
@@ -273,9 +287,9 @@ __device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S
   after_stage1();
 
   // ---- stage 2: F and v on tile + 1 ----
+  const R rho_ref = P.buoyancy == 1 ? R(*rho_ave) : (P.buoyancy == 2 ? C.rho_bc_hi : R(0));
   // F at stage-2 position (vx_, vy_) of the domain node (x, y); the stencil rows come from the clamped
   // node's own region rows so a ghost position reproduces the edge node exactly.
-  const R rho_ref = P.buoyancy == 1 ? R(*rho_ave) : (P.buoyancy == 2 ? C.rho_bc_hi : R(0));
   auto force_at = [&](int hx, int hy, int y, R& Fx, R& Fy, R& Q, R& vx, R& vy) {
     // hx, hy: stage-1 region coordinates of the node whose F is computed
     const R c00 = s_psi[hy - 1][hx - 1], c01 = s_psi[hy - 1][hx], c02 = s_psi[hy - 1][hx + 1];
@@ -387,7 +401,10 @@ __device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S
       __stwb(phi_prev + i, phi);
     else
       phi_prev[i] = phi;
-    collide_flow(f[k], rho[k], vx[k], vy[k], Fx[k], Fy[k], Q[k], P);
+    if constexpr (sizeof(R) == 4)
+      collide_flow(f[k], rho[k], vx[k], vy[k], Fx[k], Fy[k], Q[k], P);
+    else
+      relax_flow(f[k], f[k][6], f[k][7], rho[k], vx[k], vy[k], Fx[k], Fy[k], Q[k], C, f[k]);
     collide_heat(g[k], Tk, vx[k], vy[k], S0, P, tau_inv);
     if constexpr (IDX32) {
       pop_store_global<S, R, IX>(fdst, (IX)P.N, i, f[k], rho[k], C.wf);
