@@ -97,10 +97,10 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
       const long long step = I.step;
       const bool interior = tile.x0 >= 3 && tile.x0 + TX + 3 <= P.nx && tile.y0 >= 3 && tile.y0 + TY + 3 <= P.ny;
       if (interior)
-        fused_body<1, S, R, TX, TY, NPT, true>(I.f[cur], I.g[cur], I.f[cur ^ 1], I.g[cur ^ 1], (R*)I.phi_prev, P, step,
+        fused_body<1, S, R, TX, TY, NPT, true>(threadIdx.x, I.f[cur], I.g[cur], I.f[cur ^ 1], I.g[cur ^ 1], (R*)I.phi_prev, P, step,
                                          step == 0, I.scalars, I.partials, I.status, sm, tile.x0, tile.y0, tile.pslot);
       else
-        fused_body<0, S, R, TX, TY, NPT, true>(I.f[cur], I.g[cur], I.f[cur ^ 1], I.g[cur ^ 1], (R*)I.phi_prev, P, step,
+        fused_body<0, S, R, TX, TY, NPT, true>(threadIdx.x, I.f[cur], I.g[cur], I.f[cur ^ 1], I.g[cur ^ 1], (R*)I.phi_prev, P, step,
                                          step == 0, I.scalars, I.partials, I.status, sm, tile.x0, tile.y0, tile.pslot);
     }
     // The CTA's last tile: it issued no copy, so its threads leave without waiting for one another.

@@ -34,10 +34,10 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   const int x0 = (t % I.tiles_x) * TX, y0 = (t / I.tiles_x) * TY;
   const bool interior = x0 >= 3 && x0 + TX + 3 <= P.nx && y0 >= 3 && y0 + TY + 3 <= P.ny;
   if (interior)
-    fused_body<1, S, R, TX, TY, NPT>(I.fs, I.gs, I.fd, I.gd, (R*)I.phi_prev, P, 0, I.first, I.scalars, I.partials,
+    fused_body<1, S, R, TX, TY, NPT>(threadIdx.x, I.fs, I.gs, I.fd, I.gd, (R*)I.phi_prev, P, 0, I.first, I.scalars, I.partials,
                                      I.status, sm, x0, y0, t, TmaTile<S>{nullptr}, I.step);
   else  // edge tiles wrap and clamp their indices: cheaper in 32 bits
-    fused_body<0, S, R, TX, TY, NPT, true>(I.fs, I.gs, I.fd, I.gd, (R*)I.phi_prev, P, 0, I.first, I.scalars,
+    fused_body<0, S, R, TX, TY, NPT, true>(threadIdx.x, I.fs, I.gs, I.fd, I.gd, (R*)I.phi_prev, P, 0, I.first, I.scalars,
                                            I.partials, I.status, sm, x0, y0, t, TmaTile<S>{nullptr}, I.step);
   if (b == (int)gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -116,6 +116,19 @@ template <class R> inline DevParamsOf<R> params_of(const DevParams& P) {
   return q;
 }
 
+// First call of every kernel launched with launch_pdl, by every thread, before it reads or writes device memory:
+// wait until all earlier work of the stream is complete and visible. Returns threadIdx.x (NTH: the block's
+// threads, a power of two), read after the wait: addresses formed from it cannot be loaded from before the wait,
+// not even by read-only loads, which the compiler may otherwise move across it.
+template <int NTH> __device__ __forceinline__ int pdl_wait() {
+  static_assert((NTH & (NTH - 1)) == 0, "power of two");
+  int t;
+  asm volatile("griddepcontrol.wait;\n mov.u32 %0, %%tid.x;" : "=r"(t)::"memory");
+  return t & (NTH - 1);
+}
+// A value that an earlier kernel of the stream wrote, at an address that no thread index enters.
+__device__ __forceinline__ double load_after_wait(const double* p) { return *(const volatile double*)p; }
+
 // ------------------------------------------------------------------------------------------------
 // moment transforms: m = M x and x = M^{-1} m with M^{-1} = M^T diag(1/9,1/36,1/36,1/6,1/12,1/6,1/12,1/4,1/4)
 // ------------------------------------------------------------------------------------------------

@@ -19,11 +19,12 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
   const bool interior = x0 >= 3 && x0 + TX + 3 <= P.nx && y0 >= 3 && y0 + TY + 3 <= P.ny;
   const int pslot = blockIdx.y * gridDim.x + blockIdx.x;
+  const int t = pdl_wait<TX * TY / NPT>();
   if (interior)
-    fused_body<1, S, R, TX, TY, NPT>(fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+    fused_body<1, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
                                      x0, y0, pslot);
   else
-    fused_body<0, S, R, TX, TY, NPT>(fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+    fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
                                      x0, y0, pslot);
 }
 
@@ -41,14 +42,17 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
   const bool interior = x0 >= 3 && x0 + TX + 3 <= P.nx && y0 >= 3 && y0 + TY + 3 <= P.ny;
   const int pslot = blockIdx.y * gridDim.x + blockIdx.x;
+  uint64_t* bar = (uint64_t*)(dyn + B::BYTES - 128);
+  if (interior) {
+    if (threadIdx.x == 0) mbar_init(bar, 1);
+    __syncthreads();
+  }
+  const int t = pdl_wait<TX * TY / NPT>();
   if (!interior) {
-    fused_body<0, S, R, TX, TY, NPT>(fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+    fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
                                      x0, y0, pslot);
     return;
   }
-  uint64_t* bar = (uint64_t*)(dyn + B::BYTES - 128);
-  if (threadIdx.x == 0) mbar_init(bar, 1);
-  __syncthreads();
   if (threadIdx.x == 0) {
     mbar_expect_tx(bar, (unsigned)(18 * B::BX * B::BY * sizeof(S) + (B::HALF ? 2 * B::REFX * B::BY * 4 : 0)));
     for (int a = 0; a < 9; ++a) {
@@ -69,7 +73,7 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
     mbar_wait_bounded(bar, 0);  // let the copies in flight land before the block's shared memory goes away
     return;
   }
-  fused_body<2, S, R, TX, TY, NPT>(fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+  fused_body<2, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
                                    x0, y0, pslot, TmaTile<S>{dyn});
 }
 
@@ -121,6 +125,7 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
     const unsigned long long k = atomicAdd(tickets, 1ull);
     return k < (unsigned long long)ntiles ? (int)k : ntiles;
   };
+  pdl_wait<TX * TY / NPT>();  // every address below depends on a ticket or a staged copy taken after it
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
     const int t0 = take();
@@ -152,11 +157,11 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
         return;
       }
       parity ^= 1u;
-      fused_body<2, S, R, TX, TY, NPT>(fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+      fused_body<2, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
                                        x0, y0, tile, TmaTile<S>{dyn}, nullptr, start_next);
     } else {
       start_next();
-      fused_body<0, S, R, TX, TY, NPT>(fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+      fused_body<0, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
                                        x0, y0, tile);
     }
     __syncthreads();  // the tile body is done with the shared arrays; the next walk state has landed
@@ -209,25 +214,29 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
         if ((long long)grid.x * grid.y > 8LL * resident) {
           unsigned long long* tickets = (unsigned long long*)(b.status + 6);
           if ((e = cudaMemsetAsync(tickets, 0, sizeof *tickets, st)) != cudaSuccess) return e;
-          k_fused_tma_loop<S, R, TX, TY, NPT><<<resident, TX * TY / NPT, B::BYTES, st>>>(
-              fs, gs, fd, gd, (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, tickets,
-              *b.tma[cur]);
+          if ((e = launch_pdl(k_fused_tma_loop<S, R, TX, TY, NPT>, resident, TX * TY / NPT, B::BYTES, st, fs, gs, fd, gd,
+                              (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, tickets,
+                              *b.tma[cur])) != cudaSuccess)
+            return e;
           persistent = true;
         }
       }
       if (!persistent) {
-        const cudaError_t e =
+        cudaError_t e =
             cudaFuncSetAttribute(k_fused_tma<S, R, TX, TY, NPT>, cudaFuncAttributeMaxDynamicSharedMemorySize, B::BYTES);
         if (e != cudaSuccess) return e;
-        k_fused_tma<S, R, TX, TY, NPT><<<grid, TX * TY / NPT, B::BYTES, st>>>(
-            fs, gs, fd, gd, (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, *b.tma[cur]);
+        if ((e = launch_pdl(k_fused_tma<S, R, TX, TY, NPT>, grid, TX * TY / NPT, B::BYTES, st, fs, gs, fd, gd,
+                            (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, *b.tma[cur])) != cudaSuccess)
+          return e;
       }
       staged = true;
     }
   }
-  if (!staged)
-    k_fused<S, R, TX, TY, NPT><<<grid, TX * TY / NPT, 0, st>>>(fs, gs, fd, gd, (R*)b.phi_prev, P, step, step == 0,
-                                                               b.scalars, b.partials, b.status);
+  if (!staged) {
+    const cudaError_t e = launch_pdl(k_fused<S, R, TX, TY, NPT>, grid, TX * TY / NPT, 0, st, fs, gs, fd, gd, (R*)b.phi_prev,
+                                     P, step, step == 0, b.scalars, b.partials, b.status);
+    if (e != cudaSuccess) return e;
+  }
   if (ev) cudaEventRecord(ev[1], st);
   if (P.buoyancy == 1) {
     fused_finish(b, P, (int)(grid.x * grid.y), st);

@@ -19,6 +19,28 @@ struct TraceRange {
   TraceRange& operator=(const TraceRange&) = delete;
 };
 
+// Launch with programmatic stream serialization: the kernel is set up while the one before it on the stream
+// ends. Every kernel launched so calls pdl_wait() first, which waits for the completion of everything before it
+// on the stream. Ordinary launches leave about 2.5 us between dependent kernels on GB300, in steps of 2.05 us
+// (chains of small kernels, 152 CTAs: 4.1 us each; 1.4 us launched this way), as much as the kernels of a small
+// grid take. No kernel lets its successor start early (griddepcontrol.launch_dependents): the waiting blocks then
+// fill whatever slots are free, unevenly over the SMs (binary64 256^2: 54 us a step instead of 40; 43 with
+// ordinary launches).
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 template <class S, int TX, int TY> struct TmaBox {
   static constexpr int XOFF = 16 / (int)sizeof(S) > 4 ? 16 / (int)sizeof(S) : 4;
   static constexpr int EPR = 16 / (int)sizeof(S);                // elements per 16 bytes

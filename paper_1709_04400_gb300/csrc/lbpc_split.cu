@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc,
                                                  int do_partials, double* __restrict__ partials,
                                                  long long* __restrict__ status) {
   __shared__ double red[BLOCK / 32];
-  const int t = (int)threadIdx.x;
+  const int t = pdl_wait<BLOCK>();
   const long long i = (long long)blockIdx.x * BLOCK + t;
   double rho_d = 0.0;
   if (i < P.N) {
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc,
 
 template <class R>
 __global__ void __launch_bounds__(BLOCK) k_force(Planes<R> pl, DevParams P, const double* __restrict__ rho_ave) {
-  const int t = (int)threadIdx.x;
+  const int t = pdl_wait<BLOCK>();
   const Coefs<R>& C = coefs<R>(P);
   const long long i = (long long)blockIdx.x * BLOCK + t;
   if (i >= P.N) return;
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(BLOCK) k_force(Planes<R> pl, DevParams P, cons
   if (!P.yper && y == 0 && P.ybc_lo == BC_WALL) Fy += C.G_wall * 0.5f * pc * pc;
   const R rho = pl.p[P_RHO][i];
   if (P.buoyancy) {  // F_b = (rho - rho_ref) g: rho_ref = rho_ave (Sec. IV B) or the y+ edge's held density
-    const R dr = rho - (P.buoyancy == 1 ? R(*rho_ave) : C.rho_bc_hi);
+    const R dr = rho - (P.buoyancy == 1 ? R(load_after_wait(rho_ave)) : C.rho_bc_hi);
     Fx += dr * C.gx;
     Fy += dr * C.gy;
   }
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(2 * BLOCK)
     k_collide(PopBuf<S> fsrc, PopBuf<S> gsrc, PopBuf<S> fdst, PopBuf<S> gdst, Planes<R> pl, R* __restrict__ phi_prev,
               DevParams P, int first) {
   const Coefs<R>& C = coefs<R>(P);
-  const int t = (int)threadIdx.x;
+  const int t = pdl_wait<2 * BLOCK>();
   const bool heat = t >= BLOCK;
   const long long i = (long long)blockIdx.x * BLOCK + (t - (heat ? BLOCK : 0));
   if (i >= P.N) return;
@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(2 * CX* CY)
   static_assert(RING <= CN, "one ring node per thread of the second half");
   __shared__ R s_vx[CY + 2][CX + 2], s_vy[CY + 2][CX + 2];
   const Coefs<R>& C = coefs<R>(P);
-  const int t = (int)threadIdx.x;
+  const int t = pdl_wait<2 * CN>();
   const bool heat = t >= CN;
   const int x0 = (int)(blockIdx.x % (unsigned)tiles_x) * CX, y0 = (int)(blockIdx.x / (unsigned)tiles_x) * CY;
   const bool interior = x0 >= 2 && x0 + CX + 2 <= P.nx && y0 >= 2 && y0 + CY + 2 <= P.ny;
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(2 * CX* CY)
     Fy = Gp * sy;
     if (!P.yper && y == 0 && P.ybc_lo == BC_WALL) Fy += C.G_wall * 0.5f * pc * pc;
     if (P.buoyancy) {
-      const R dr = rho - (P.buoyancy == 1 ? R(*rho_ave) : C.rho_bc_hi);
+      const R dr = rho - (P.buoyancy == 1 ? R(load_after_wait(rho_ave)) : C.rho_bc_hi);
       Fx += dr * C.gx;
       Fy += dr * C.gy;
     }
@@ -404,17 +404,22 @@ __global__ void __launch_bounds__(2 * CX* CY)
   for (int a = 0; a < 9; ++a) pg[(size_t)a * P.N] = g[a];
 }
 
-// Fixed-order sum of the block partials: each thread accumulates a strided subset in order, then one
-// block reduction. out[k] = sum(partials[k * stride + 0 .. n)) * scale.
-__global__ void __launch_bounds__(BLOCK) k_finish(const double* __restrict__ partials, int n, int stride, int count,
-                                                  double scale, double* __restrict__ out) {
-  __shared__ double red[BLOCK / 32];
-  for (int k = 0; k < count; ++k) {
-    double s = 0.0;
-    for (int j = threadIdx.x; j < n; j += BLOCK) s += partials[(long long)k * stride + j];
-    s = block_sum<BLOCK>(s, red);
-    if (threadIdx.x == 0) out[k] = s * scale;
-  }
+// Fixed-order sums of the block partials, one block per sum: out[k] = sum(partials[k * stride + 0 .. n)) * scale.
+// A thread adds every FINISH-th partial, four at a time so that four loads are in flight (the sum is one block's
+// latency: with 64 threads and one load at a time it took 8 us of a 300 x 200 step's 30).
+constexpr int FINISH = 512;
+__global__ void __launch_bounds__(FINISH) k_finish(const double* __restrict__ partials, int n, int stride, double scale,
+                                                   double* __restrict__ out) {
+  __shared__ double red[FINISH / 32];
+  const int tid = pdl_wait<FINISH>();
+  const double* p = partials + (long long)blockIdx.x * stride;
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (int j = tid; j < n; j += 4 * FINISH)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (j + k * FINISH < n) s[k] += p[j + k * FINISH];
+  const double t = block_sum<FINISH>((s[0] + s[1]) + (s[2] + s[3]), red);
+  if (tid == 0) out[blockIdx.x] = t * scale;
 }
 
 // Equilibrium start: writes post-collision-layout buffers whose pull gives f = M^{-1} m_eq(rho, u),
@@ -423,7 +428,7 @@ template <class S>
 __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_in, const double* __restrict__ T_in,
                                                 const double* __restrict__ ux_in, const double* __restrict__ uy_in,
                                                 PopBuf<S> f, PopBuf<S> g, DevParams P) {
-  const long long i = (long long)blockIdx.x * BLOCK + (int)threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
   const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
   double fv[9], gv[9];
@@ -464,7 +469,7 @@ template <class S>
 __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P,
                                                 double* __restrict__ partials, int stride) {
   __shared__ double red[BLOCK / 32];
-  const int tid = (int)threadIdx.x;
+  const int tid = pdl_wait<BLOCK>();
   const long long i = (long long)blockIdx.x * BLOCK + tid;
   double r = 0.0, t = 0.0;
   if (i < P.N) {
@@ -484,7 +489,7 @@ __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, 
 template <class S>
 __global__ void __launch_bounds__(BLOCK) k_export_pops(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P, int which,
                                                        int only, double* __restrict__ out) {
-  const long long i = (long long)blockIdx.x * BLOCK + (int)threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
   const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
   double f[9], g[9];
@@ -501,7 +506,7 @@ __global__ void __launch_bounds__(BLOCK) k_export_pops(PopBuf<S> fsrc, PopBuf<S>
 template <class R>
 __global__ void __launch_bounds__(BLOCK) k_export_fields(Planes<R> pl, DevParams P, double* rho, double* ux, double* uy,
                                                          double* T) {
-  const long long i = (long long)blockIdx.x * BLOCK + (int)threadIdx.x;
+  const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
   if (rho) rho[i] = (double)pl.p[P_RHO][i];
   if (ux) ux[i] = (double)pl.p[P_VX][i];
@@ -532,16 +537,16 @@ static cudaError_t step_impl(const SplitBuffers& b, const DevParams& P, int cur,
   const unsigned nb = blocks_for(P.N);
   Planes<R> pl = planes_of<S, R>(b);
   if (ev) cudaEventRecord(ev[0], st);
-  k_macro<S, R, false><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), nullptr, nullptr, pl, P, step,
+  launch_pdl(k_macro<S, R, false>, nb, BLOCK, 0, st, fbuf<S>(b, cur), gbuf<S>(b, cur), nullptr, nullptr, pl, P, step,
                                              P.buoyancy == 1, b.partials, b.status);
   if (ev) cudaEventRecord(ev[1], st);
-  k_force<R><<<nb, BLOCK, 0, st>>>(pl, P, b.scalars);
+  launch_pdl(k_force<R>, nb, BLOCK, 0, st, pl, P, b.scalars);
   if (ev) cudaEventRecord(ev[2], st);
-  k_collide<S, R><<<nb, 2 * BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), fbuf<S>(b, cur ^ 1), gbuf<S>(b, cur ^ 1),
+  launch_pdl(k_collide<S, R>, nb, 2 * BLOCK, 0, st, fbuf<S>(b, cur), gbuf<S>(b, cur), fbuf<S>(b, cur ^ 1), gbuf<S>(b, cur ^ 1),
                                             pl, (R*)b.phi_prev, P, step == 0);
   if (ev) cudaEventRecord(ev[3], st);
   if (P.buoyancy == 1) {
-    k_finish<<<1, BLOCK, 0, st>>>(b.partials, (int)nb, 0, 1, 1.0 / (double)P.N, b.scalars);
+    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars);
     if (ev) cudaEventRecord(ev[4], st);
   }
   return cudaGetLastError();
@@ -555,14 +560,14 @@ static cudaError_t step_wide(const SplitBuffers& b, const DevParams& P, int cur,
   Planes<S> pl = planes_of<S, S>(b);
   const PopBuf<S> fd = fbuf<S>(b, cur ^ 1), gd = gbuf<S>(b, cur ^ 1);
   if (ev) cudaEventRecord(ev[0], st);
-  k_macro<S, S, true><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), fd.p, gd.p, pl, P, step, P.buoyancy == 1,
+  launch_pdl(k_macro<S, S, true>, nb, BLOCK, 0, st, fbuf<S>(b, cur), gbuf<S>(b, cur), fd.p, gd.p, pl, P, step, P.buoyancy == 1,
                                             b.partials, b.status);
   if (ev) cudaEventRecord(ev[1], st);
   auto collide = [&](auto cx, auto cy) {
     constexpr int CX = decltype(cx)::value, CY = decltype(cy)::value;
     const int tiles_x = (P.nx + CX - 1) / CX;
     const unsigned tiles = (unsigned)((long long)tiles_x * ((P.ny + CY - 1) / CY));
-    k_collide_tile<S, CX, CY><<<tiles, 2 * CX * CY, 0, st>>>(gbuf<S>(b, cur), fd, gd, pl, (S*)b.phi_prev, P, step == 0,
+    launch_pdl(k_collide_tile<S, CX, CY>, tiles, 2 * CX * CY, 0, st, gbuf<S>(b, cur), fd, gd, pl, (S*)b.phi_prev, P, step == 0,
                                                             tiles_x, b.scalars);
   };
   // 16 x 8 tiles; large binary64 grids take 32 x 8, whose ring repeats less of the force (1.33 instead of 1.41 times
@@ -574,7 +579,7 @@ static cudaError_t step_wide(const SplitBuffers& b, const DevParams& P, int cur,
     collide(std::integral_constant<int, 16>(), std::integral_constant<int, 8>());
   if (ev) cudaEventRecord(ev[2], st);
   if (P.buoyancy == 1) {
-    k_finish<<<1, BLOCK, 0, st>>>(b.partials, (int)nb, 0, 1, 1.0 / (double)P.N, b.scalars);
+    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars);
     if (ev) cudaEventRecord(ev[3], st);
   }
   return cudaGetLastError();
@@ -608,10 +613,10 @@ static cudaError_t init_impl(const SplitBuffers& b, const DevParams& P, const do
       const cudaError_t e = cudaMemsetAsync(b.wall[k], 0, wall_doubles(P.nx) * sizeof(double), st);
       if (e != cudaSuccess) return e;
     }
-  k_init<S><<<nb, BLOCK, 0, st>>>(rho, T, ux, uy, fbuf<S>(b, 0), gbuf<S>(b, 0), P);
+  launch_pdl(k_init<S>, nb, BLOCK, 0, st, rho, T, ux, uy, fbuf<S>(b, 0), gbuf<S>(b, 0), P);
   // rho_ave of the initial (post-boundary) state
-  k_sums<S><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, 0), gbuf<S>(b, 0), P, b.partials, (int)nb);
-  k_finish<<<1, BLOCK, 0, st>>>(b.partials, (int)nb, (int)nb, 1, 1.0 / (double)P.N, b.scalars);
+  launch_pdl(k_sums<S>, nb, BLOCK, 0, st, fbuf<S>(b, 0), gbuf<S>(b, 0), P, b.partials, (int)nb);
+  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, (int)nb, 1.0 / (double)P.N, b.scalars);
   return cudaGetLastError();
 }
 
@@ -626,8 +631,8 @@ cudaError_t split_init(const SplitBuffers& b, const DevParams& P, int prec, cons
 template <class S>
 static cudaError_t sums_impl(const SplitBuffers& b, const DevParams& P, int cur, cudaStream_t st) {
   const unsigned nb = blocks_for(P.N);
-  k_sums<S><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), P, b.partials, (int)nb);
-  k_finish<<<1, BLOCK, 0, st>>>(b.partials, (int)nb, (int)nb, 2, 1.0, b.scalars + 1);
+  launch_pdl(k_sums<S>, nb, BLOCK, 0, st, fbuf<S>(b, cur), gbuf<S>(b, cur), P, b.partials, (int)nb);
+  launch_pdl(k_finish, 2, FINISH, 0, st, b.partials, (int)nb, (int)nb, 1.0, b.scalars + 1);
   return cudaGetLastError();
 }
 
@@ -643,10 +648,10 @@ static cudaError_t fields_impl(const SplitBuffers& b, const DevParams& P, int cu
                                double* ux, double* uy, double* T, cudaStream_t st) {
   const unsigned nb = blocks_for(P.N);
   Planes<R> pl = planes_of<S, R>(b);
-  k_macro<S, R, false><<<nb, BLOCK, 0, st>>>(fbuf<S>(b, cur), gbuf<S>(b, cur), nullptr, nullptr, pl, P, step, 0,
+  launch_pdl(k_macro<S, R, false>, nb, BLOCK, 0, st, fbuf<S>(b, cur), gbuf<S>(b, cur), nullptr, nullptr, pl, P, step, 0,
                                              b.partials, b.status);
-  k_force<R><<<nb, BLOCK, 0, st>>>(pl, P, b.scalars);
-  k_export_fields<R><<<nb, BLOCK, 0, st>>>(pl, P, rho, ux, uy, T);
+  launch_pdl(k_force<R>, nb, BLOCK, 0, st, pl, P, b.scalars);
+  launch_pdl(k_export_fields<R>, nb, BLOCK, 0, st, pl, P, rho, ux, uy, T);
   return cudaGetLastError();
 }
 
@@ -662,18 +667,18 @@ cudaError_t split_export_pops(const SplitBuffers& b, const DevParams& P, int pre
                               double* out, cudaStream_t st) {
   const unsigned nb = blocks_for(P.N);
   if (prec == 0)
-    k_export_pops<double><<<nb, BLOCK, 0, st>>>(fbuf<double>(b, cur), gbuf<double>(b, cur), P, which, only, out);
+    launch_pdl(k_export_pops<double>, nb, BLOCK, 0, st, fbuf<double>(b, cur), gbuf<double>(b, cur), P, which, only, out);
   else if (prec == 1)
-    k_export_pops<float><<<nb, BLOCK, 0, st>>>(fbuf<float>(b, cur), gbuf<float>(b, cur), P, which, only, out);
+    launch_pdl(k_export_pops<float>, nb, BLOCK, 0, st, fbuf<float>(b, cur), gbuf<float>(b, cur), P, which, only, out);
   else if (prec == 3)
-    k_export_pops<dw><<<nb, BLOCK, 0, st>>>(fbuf<dw>(b, cur), gbuf<dw>(b, cur), P, which, only, out);
+    launch_pdl(k_export_pops<dw>, nb, BLOCK, 0, st, fbuf<dw>(b, cur), gbuf<dw>(b, cur), P, which, only, out);
   else
-    k_export_pops<__half><<<nb, BLOCK, 0, st>>>(fbuf<__half>(b, cur), gbuf<__half>(b, cur), P, which, only, out);
+    launch_pdl(k_export_pops<__half>, nb, BLOCK, 0, st, fbuf<__half>(b, cur), gbuf<__half>(b, cur), P, which, only, out);
   return cudaGetLastError();
 }
 
 void fused_finish(const SplitBuffers& b, const DevParams& P, int n, cudaStream_t st) {
-  k_finish<<<1, BLOCK, 0, st>>>(b.partials, n, 0, 1, 1.0 / (double)P.N, b.scalars);
+  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, n, 0, 1.0 / (double)P.N, b.scalars);
 }
 
 int split_nplanes() { return NPLANES; }

@@ -139,6 +139,7 @@ template <class S, int NTH, int NPT> __host__ __device__ constexpr int fused_min
 // issued as global ones explicitly. This is for buffers whose pointers come from a descriptor in shared
 // memory (the batch's work-list kernel): the compiler cannot infer their space, and each wider index costs
 // registers there. Where the pointers and sizes are kernel parameters, 64-bit indices are faster.
+// t: the thread's index in the block (pdl_wait's in kernels launched with launch_pdl).
 // after_stage1: called by every thread once the tile has finished reading its staged populations (after
 // the block barrier that closes stage 1); the persistent TMA kernel starts the next tile's copy there.
 struct NoStageHook {
@@ -147,7 +148,7 @@ struct NoStageHook {
 
 template <int MODE, class S, class R, int TX, int TY, int NPT = 1, bool IDX32 = false, class PT = DevParams,
           class AfterStage1 = NoStageHook>
-__device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S>& gsrc, const PopBuf<S>& fdst,
+__device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const PopBuf<S>& gsrc, const PopBuf<S>& fdst,
                                            const PopBuf<S>& gdst, R* __restrict__ phi_prev,
                                            const PT& P, long long step, int first,
                                            const double* __restrict__ rho_ave, double* __restrict__ partials,
@@ -173,7 +174,16 @@ __device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S
   double* s_red = sm.red;
 
   const Coefs<R>& C = coefs<R>(P);
-  const int t = threadIdx.x;
+
+  // The buoyancy's reference density. With the parameters in PT's compact form (the batch) it is read here, before
+  // the pulls, whose latency hides it (in stage 2 the batched step is 8 % slower); with DevParams in stage 2 (here
+  // the single-instance step of a 1023 x 1025 grid is 3 % slower).
+  constexpr bool kEarlyRef = !std::is_same<PT, DevParams>::value;
+  auto read_ref = [&]() {
+    return P.buoyancy == 1 ? R(load_after_wait(rho_ave)) : (P.buoyancy == 2 ? C.rho_bc_hi : R(0));
+  };
+  R rho_ref = R(0);
+  if constexpr (kEarlyRef) rho_ref = read_ref();
 
   // ---- stage 1a: own nodes (kept in registers) ----
   R f[NPT][9], g[NPT][9];
@@ -287,7 +297,7 @@ __device__ __forceinline__ void fused_body(const PopBuf<S>& fsrc, const PopBuf<S
   after_stage1();
 
   // ---- stage 2: F and v on tile + 1 ----
-  const R rho_ref = P.buoyancy == 1 ? R(*rho_ave) : (P.buoyancy == 2 ? C.rho_bc_hi : R(0));
+  if constexpr (!kEarlyRef) rho_ref = read_ref();
   // F at stage-2 position (vx_, vy_) of the domain node (x, y); the stencil rows come from the clamped
   // node's own region rows so a ghost position reproduces the edge node exactly.
   auto force_at = [&](int hx, int hy, int y, R& Fx, R& Fy, R& Q, R& vx, R& vy) {
