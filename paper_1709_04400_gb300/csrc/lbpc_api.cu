@@ -724,15 +724,31 @@ LBPC_API lbpc_status lbpc_sums(lbpc_ctx* c, double* mass, double* heat) {
   return LBPC_OK;
 }
 
+// The address under which the reduction kernel can write the caller's two doubles itself (memory of the context's
+// device, or pinned host memory mapped for it), or null where a copy is needed. A copy of 16 bytes costs a monitored
+// step its two ordinary stream dependencies besides (binary64 256^2, step and sums: 63 us with it, 53 without).
+static double* device_writable(lbpc_ctx* c, double* out) {
+  cudaPointerAttributes at{};
+  if (((uintptr_t)out & 7) != 0 || cudaPointerGetAttributes(&at, out) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (at.type == cudaMemoryTypeDevice && at.device == c->device) return out;
+  if (at.type == cudaMemoryTypeHost) return (double*)at.devicePointer;
+  return nullptr;
+}
+
 LBPC_API lbpc_status lbpc_sums_async(lbpc_ctx* c, double* out, int on_device) {
   lbpc::TraceRange trace_("lbpc_sums_async");
   if (!c || !out) return LBPC_EINVAL;
   if (!c->initialised) return LBPC_ESTATE;
   DeviceGuard g(c->device);
-  CU(c, lbpc::split_sums(c->buf, c->dp, c->p.prec, c->cur, c->stream), "lbpc_sums_async kernels");
-  CU(c, cudaMemcpyAsync(out, c->buf.scalars + 1, 2 * sizeof(double),
-                        on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream),
-     "lbpc_sums_async copy");
+  double* direct = device_writable(c, out);
+  CU(c, lbpc::split_sums(c->buf, c->dp, c->p.prec, c->cur, c->stream, direct), "lbpc_sums_async kernels");
+  if (!direct)
+    CU(c, cudaMemcpyAsync(out, c->buf.scalars + 1, 2 * sizeof(double),
+                          on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream),
+       "lbpc_sums_async copy");
   return LBPC_OK;
 }
 

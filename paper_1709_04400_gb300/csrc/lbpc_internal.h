@@ -91,7 +91,9 @@ int split_kernel_count(const DevParams& P, int prec);
 const char* split_kernel_name(int prec, int k);
 cudaError_t split_init(const SplitBuffers& b, const DevParams& P, int prec, const double* rho, const double* T,
                        const double* ux, const double* uy, cudaStream_t st);
-cudaError_t split_sums(const SplitBuffers& b, const DevParams& P, int prec, int cur, cudaStream_t st);
+// Domain sums into scalars[1], scalars[2] and, unless null, out[0], out[1] (memory the device can write).
+cudaError_t split_sums(const SplitBuffers& b, const DevParams& P, int prec, int cur, cudaStream_t st,
+                       double* out = nullptr);
 cudaError_t split_fields(const SplitBuffers& b, const DevParams& P, int prec, int cur, long long step, double* rho,
                          double* ux, double* uy, double* T, cudaStream_t st);
 // which = 0: f, 1: g; only < 0: all 9 planes [9][N], else plane `only` into out[N].

@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(2 * CX* CY)
 // latency: with 64 threads and one load at a time it took 8 us of a 300 x 200 step's 30).
 constexpr int FINISH = 512;
 __global__ void __launch_bounds__(FINISH) k_finish(const double* __restrict__ partials, int n, int stride, double scale,
-                                                   double* __restrict__ out) {
+                                                   double* __restrict__ out, double* out2) {
   __shared__ double red[FINISH / 32];
   const int tid = pdl_wait<FINISH>();
   const double* p = partials + (long long)blockIdx.x * stride;
@@ -419,7 +419,10 @@ __global__ void __launch_bounds__(FINISH) k_finish(const double* __restrict__ pa
     for (int k = 0; k < 4; ++k)
       if (j + k * FINISH < n) s[k] += p[j + k * FINISH];
   const double t = block_sum<FINISH>((s[0] + s[1]) + (s[2] + s[3]), red);
-  if (tid == 0) out[blockIdx.x] = t * scale;
+  if (tid == 0) {
+    out[blockIdx.x] = t * scale;
+    if (out2) out2[blockIdx.x] = t * scale;  // the caller's copy, in device or pinned host memory
+  }
 }
 
 // Equilibrium start: writes post-collision-layout buffers whose pull gives f = M^{-1} m_eq(rho, u),
@@ -464,20 +467,24 @@ __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_i
   pop_store<S, double>(g, P.N, i, gv, T_in[i], P.cd.wg);
 }
 
-// Sums of rho and T over the current (post-boundary) state into per-block partials.
-template <class S>
+// Sums of rho and T over the current (post-boundary) state into per-block partials. Bound by the FP64 pipe
+// (16 additions per node, and a conversion per population of a narrower storage), so a thread takes K nodes
+// before the block's reduction, whose 30 instructions per warp K = 1 pays for every 32 nodes.
+template <class S, int K>
 __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P,
                                                 double* __restrict__ partials, int stride) {
   __shared__ double red[BLOCK / 32];
   const int tid = pdl_wait<BLOCK>();
-  const long long i = (long long)blockIdx.x * BLOCK + tid;
   double r = 0.0, t = 0.0;
-  if (i < P.N) {
+#pragma unroll 2
+  for (int k = 0; k < K; ++k) {
+    const long long i = ((long long)blockIdx.x * K + k) * BLOCK + tid;
+    if (i >= P.N) break;
     const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
     double f[9], g[9];
     pull_closed<S, double>(fsrc, gsrc, P, x, y, f, g);
-    r = f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
-    t = g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + g[6] + g[7] + g[8];
+    r += f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
+    t += g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + g[6] + g[7] + g[8];
   }
   const double sr = block_sum<BLOCK>(r, red);
   if (tid == 0) partials[blockIdx.x] = sr;
@@ -546,7 +553,7 @@ static cudaError_t step_impl(const SplitBuffers& b, const DevParams& P, int cur,
                                             pl, (R*)b.phi_prev, P, step == 0);
   if (ev) cudaEventRecord(ev[3], st);
   if (P.buoyancy == 1) {
-    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars);
+    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars, nullptr);
     if (ev) cudaEventRecord(ev[4], st);
   }
   return cudaGetLastError();
@@ -579,7 +586,7 @@ static cudaError_t step_wide(const SplitBuffers& b, const DevParams& P, int cur,
     collide(std::integral_constant<int, 16>(), std::integral_constant<int, 8>());
   if (ev) cudaEventRecord(ev[2], st);
   if (P.buoyancy == 1) {
-    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars);
+    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars, nullptr);
     if (ev) cudaEventRecord(ev[3], st);
   }
   return cudaGetLastError();
@@ -604,6 +611,19 @@ const char* split_kernel_name(int prec, int k) {
   return is_wide(prec) ? wide[k] : names[k];
 }
 
+// Enqueue k_sums; returns its number of blocks. Four nodes per thread on large grids (2048^2 with k_finish: binary64
+// 264 us, 303 with one node; binary32 399, 436), one where latency counts (256^2: 13.1 us, 15.4 with four).
+template <class S> static int launch_sums(const SplitBuffers& b, const DevParams& P, int k, cudaStream_t st) {
+  const int stride = (int)blocks_for(P.N);
+  if (P.N < (1 << 20)) {
+    launch_pdl(k_sums<S, 1>, stride, BLOCK, 0, st, fbuf<S>(b, k), gbuf<S>(b, k), P, b.partials, stride);
+    return stride;
+  }
+  const int nb = (stride + 3) / 4;
+  launch_pdl(k_sums<S, 4>, nb, BLOCK, 0, st, fbuf<S>(b, k), gbuf<S>(b, k), P, b.partials, stride);
+  return nb;
+}
+
 template <class S>
 static cudaError_t init_impl(const SplitBuffers& b, const DevParams& P, const double* rho, const double* T,
                              const double* ux, const double* uy, cudaStream_t st) {
@@ -615,8 +635,8 @@ static cudaError_t init_impl(const SplitBuffers& b, const DevParams& P, const do
     }
   launch_pdl(k_init<S>, nb, BLOCK, 0, st, rho, T, ux, uy, fbuf<S>(b, 0), gbuf<S>(b, 0), P);
   // rho_ave of the initial (post-boundary) state
-  launch_pdl(k_sums<S>, nb, BLOCK, 0, st, fbuf<S>(b, 0), gbuf<S>(b, 0), P, b.partials, (int)nb);
-  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, (int)nb, 1.0 / (double)P.N, b.scalars);
+  const int ns = launch_sums<S>(b, P, 0, st);
+  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, ns, 0, 1.0 / (double)P.N, b.scalars, nullptr);
   return cudaGetLastError();
 }
 
@@ -629,18 +649,17 @@ cudaError_t split_init(const SplitBuffers& b, const DevParams& P, int prec, cons
 }
 
 template <class S>
-static cudaError_t sums_impl(const SplitBuffers& b, const DevParams& P, int cur, cudaStream_t st) {
-  const unsigned nb = blocks_for(P.N);
-  launch_pdl(k_sums<S>, nb, BLOCK, 0, st, fbuf<S>(b, cur), gbuf<S>(b, cur), P, b.partials, (int)nb);
-  launch_pdl(k_finish, 2, FINISH, 0, st, b.partials, (int)nb, (int)nb, 1.0, b.scalars + 1);
+static cudaError_t sums_impl(const SplitBuffers& b, const DevParams& P, int cur, double* out, cudaStream_t st) {
+  const int nb = launch_sums<S>(b, P, cur, st);
+  launch_pdl(k_finish, 2, FINISH, 0, st, b.partials, nb, (int)blocks_for(P.N), 1.0, b.scalars + 1, out);
   return cudaGetLastError();
 }
 
-cudaError_t split_sums(const SplitBuffers& b, const DevParams& P, int prec, int cur, cudaStream_t st) {
-  if (prec == 0) return sums_impl<double>(b, P, cur, st);
-  if (prec == 1) return sums_impl<float>(b, P, cur, st);
-  if (prec == 3) return sums_impl<dw>(b, P, cur, st);
-  return sums_impl<__half>(b, P, cur, st);
+cudaError_t split_sums(const SplitBuffers& b, const DevParams& P, int prec, int cur, cudaStream_t st, double* out) {
+  if (prec == 0) return sums_impl<double>(b, P, cur, out, st);
+  if (prec == 1) return sums_impl<float>(b, P, cur, out, st);
+  if (prec == 3) return sums_impl<dw>(b, P, cur, out, st);
+  return sums_impl<__half>(b, P, cur, out, st);
 }
 
 template <class S, class R>
@@ -678,7 +697,7 @@ cudaError_t split_export_pops(const SplitBuffers& b, const DevParams& P, int pre
 }
 
 void fused_finish(const SplitBuffers& b, const DevParams& P, int n, cudaStream_t st) {
-  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, n, 0, 1.0 / (double)P.N, b.scalars);
+  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, n, 0, 1.0 / (double)P.N, b.scalars, nullptr);
 }
 
 int split_nplanes() { return NPLANES; }
