@@ -179,6 +179,22 @@ template <class R> __device__ __forceinline__ void from_moments_conserving(const
   if constexpr (sizeof(R) == 4) x[0] = m[0] - (((x[1] + x[2]) + (x[3] + x[4])) + ((x[5] + x[6]) + (x[7] + x[8])));
 }
 
+// Reciprocal and roots. Binary32 takes the hardware's approximations without the compiler's handling of
+// subnormal and huge arguments (a test, a select and two products each, about 4 % of the fused step's
+// instructions): the same bits for normal arguments, and a state with others is outside the equation of state's range.
+template <class R> __device__ __forceinline__ R inverse_of(R x) { return R(1) / x; }
+template <> __device__ __forceinline__ float inverse_of<float>(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+template <class R> __device__ __forceinline__ R inverse_root_of(R x) { return rsqrt(x); }
+template <> __device__ __forceinline__ float inverse_root_of<float>(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
 // ------------------------------------------------------------------------------------------------
 // Peng-Robinson EOS (Eq. 56) and (dp/dT)_rho
 // ------------------------------------------------------------------------------------------------
@@ -187,7 +203,7 @@ template <class R, class PT> __device__ __forceinline__ void eos(R rho, R T, con
   // theta(T) = [1 + kappa (1 - sqrt(T/T_c))]^2 and d theta/dT = -kappa [..] / sqrt(T T_c); one rsqrt
   // gives both sqrt(T/T_c) = t rsqrt(t) and 1/sqrt(T T_c) = rsqrt(t) / T_c with t = T/T_c.
   const R t = T * C.inv_Tc;
-  const R rs = rsqrt(t);
+  const R rs = inverse_root_of(t);
   const R sq = t * rs;
   const R th1 = R(1) + C.kappa * (R(1) - sq);
   const R theta = th1 * th1;
@@ -199,11 +215,11 @@ template <class R, class PT> __device__ __forceinline__ void eos(R rho, R T, con
   const R d12 = d1 * d2;
   R r12;
   if (inv_rho) {
-    const R r = R(1) / (rho * d12);
+    const R r = inverse_of(rho * d12);
     *inv_rho = d12 * r;
     r12 = rho * r;
   } else {
-    r12 = R(1) / d12;
+    r12 = inverse_of(d12);
   }
   const R inv1 = d2 * r12, inv2 = d1 * r12;
   const R r2 = rho * rho;
@@ -215,7 +231,6 @@ template <class R, class PT> __device__ __forceinline__ void eos(R rho, R T, con
 // the arithmetic pipe): psi^2, (dp/dT)_rho and 1/rho from one reciprocal and one reciprocal square root.
 // With u = rho R / (1 - b rho), A = a rho^2 / (1 + 2 b rho - b^2 rho^2) and h = 1 + kappa (1 - sqrt(T/T_c)):
 // p = u T - A h^2 and dp/dT = u + A h kappa / sqrt(T T_c).
-template <class R> __device__ __forceinline__ R inverse_of(R x) { return R(1) / x; }
 template <> __device__ __forceinline__ dw inverse_of<dw>(dw x) {  // binary32 reciprocal, corrected once
   x = dw_norm(x);
   const float r = __frcp_rn(x.hi);
@@ -250,6 +265,11 @@ __device__ __forceinline__ void roots_of(dw x, dw& inv_root, dw& root) {
 }
 // psi = sqrt(max(psi^2, 0)), a NaN counting as 0; the tests of the binary64 form run on the integer pipe.
 template <class R> __device__ __forceinline__ R psi_of(R psi2) { return sqrt(fmax(psi2, R(0))); }
+template <> __device__ __forceinline__ float psi_of<float>(float psi2) {
+  float y;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(::fmaxf(psi2, 0.0f)));
+  return y;
+}
 template <> __device__ __forceinline__ double psi_of<double>(double psi2) {
   const long long b = __double_as_longlong(psi2);
   double inv_root, root;
@@ -822,6 +842,19 @@ template <class R, class PT> __device__ __forceinline__ int classify(R rho, R T,
   if (!(T > R(0))) return ST_T_LE0;
   if (!(psi2 >= R(0))) return ST_PSI2_NEG;
   return 0;
+}
+
+// Report a node that is not physical. Binary32 first tests everything at once (a NaN fails every comparison) and
+// classifies only what fails.
+template <class R, class PT>
+__device__ __forceinline__ void check_node(R rho, R T, R psi2, const PT& P, long long* status, const long long* step_at,
+                                           long long step, int x, int y) {
+  if constexpr (sizeof(R) == 4) {
+    const R top = R(3.402823466e38);
+    if (rho > R(0) && coefs<R>(P).b * rho < R(1) && T > R(0) && T <= top && psi2 >= R(0) && psi2 <= top) return;
+  }
+  const int bad = classify(rho, T, psi2, P);
+  if (bad) report(status, step_at ? *step_at : step, x, y, bad);  // step_at: read only to report
 }
 
 }  // namespace lbpc

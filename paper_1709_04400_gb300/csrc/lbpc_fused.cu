@@ -55,13 +55,11 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   }
   if (threadIdx.x == 0) {
     mbar_expect_tx(bar, (unsigned)(18 * B::BX * B::BY * sizeof(S) + (B::HALF ? 2 * B::REFX * B::BY * 4 : 0)));
-    for (int a = 0; a < 9; ++a) {
-      tma_load_3d(dyn + a * B::PLANE, &maps.f, x0 - B::XOFF, y0 - 3, a, bar);
-      tma_load_3d(dyn + (9 + a) * B::PLANE, &maps.g, x0 - B::XOFF, y0 - 3, a, bar);
-    }
+    tma_load_3d(dyn, &maps.f, x0 - B::XOFF, y0 - 3, 0, bar);
+    tma_load_3d(dyn + B::SET, &maps.g, x0 - B::XOFF, y0 - 3, 0, bar);
     if (B::HALF) {
-      tma_load_2d(dyn + 18 * B::PLANE, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
-      tma_load_2d(dyn + 18 * B::PLANE + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
+      tma_load_2d(dyn + 2 * B::SET, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
+      tma_load_2d(dyn + 2 * B::SET + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
     }
   }
   // Every thread polls the barrier. Measured against one polling thread with the others parked at a block
@@ -82,8 +80,11 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
 // re-read meet in L2), and each starts its next interior tile's copy as soon as the current tile has
 // finished reading its staged populations (after stage 1). The copy then runs under stages 2 and 3
 // instead of in front of the next tile. An edge tile reads nothing staged, so the next copy starts
-// before it. One mbarrier serves every copy; the waits alternate its phase parity. tickets is zeroed
-// before the launch.
+// before it. One mbarrier serves every copy; the waits alternate its phase parity.
+//
+// Bound by HBM in FP32 (4096^2: 413 us, 91 % of the measured copy bandwidth at 152 B per node) and by issue in
+// FP16. What the walk itself costs counts: with each ticket awaited where the next copy starts, one tensor copy
+// per population plane, and tile origins divided out by every thread, 4096^2 took 469 us (FP16 528, now 470).
 template <class S, int TX, int TY>
 __device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar, const TmaMaps& maps, int x0, int y0) {
   using B = TmaBox<S, TX, TY>;
@@ -91,13 +92,11 @@ __device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar
   // reads before the copy engine's writes
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   mbar_expect_tx(bar, (unsigned)(18 * B::BX * B::BY * sizeof(S) + (B::HALF ? 2 * B::REFX * B::BY * 4 : 0)));
-  for (int a = 0; a < 9; ++a) {
-    tma_load_3d(dyn + a * B::PLANE, &maps.f, x0 - B::XOFF, y0 - 3, a, bar);
-    tma_load_3d(dyn + (9 + a) * B::PLANE, &maps.g, x0 - B::XOFF, y0 - 3, a, bar);
-  }
+  tma_load_3d(dyn, &maps.f, x0 - B::XOFF, y0 - 3, 0, bar);
+  tma_load_3d(dyn + B::SET, &maps.g, x0 - B::XOFF, y0 - 3, 0, bar);
   if (B::HALF) {
-    tma_load_2d(dyn + 18 * B::PLANE, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
-    tma_load_2d(dyn + 18 * B::PLANE + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
+    tma_load_2d(dyn + 2 * B::SET, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
+    tma_load_2d(dyn + 2 * B::SET + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
   }
 }
 
@@ -109,63 +108,71 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
                      unsigned long long* __restrict__ tickets, const __grid_constant__ TmaMaps maps) {
   using B = TmaBox<S, TX, TY>;
   __shared__ FusedSmem<R, TX, TY> sm;
-  // walk state, double-buffered by iteration parity: this tile and the next one (being staged); thread 0
-  // fills the other slot during the tile, so one block barrier per tile orders both
-  __shared__ int s_tile[2], s_next[2];
+  // walk state, double-buffered by iteration parity: this tile and the next one (being staged), each with its
+  // origin (x < 0: no tile left); thread 0 fills the other slot during the tile, so one block barrier per tile
+  // orders both
+  struct Tile {
+    int x, y, index;
+  };
+  __shared__ Tile s_tile[2], s_next[2];
   extern __shared__ __align__(128) unsigned char dyn[];
   uint64_t* bar = (uint64_t*)(dyn + B::BYTES - 128);
   const int ntx = (P.nx + TX - 1) / TX, ntiles = ntx * ((P.ny + TY - 1) / TY);
-  // tile origin, and whether the tile, its 2-ring and their pull sources stay inside the domain
-  auto origin = [&](int tile, int& x0, int& y0) {
-    x0 = (tile % ntx) * TX;
-    y0 = (tile / ntx) * TY;
-    return x0 >= 3 && x0 + TX + 3 <= P.nx && y0 >= 3 && y0 + TY + 3 <= P.ny;
+  auto tile_at = [&](unsigned long long k) {  // thread 0: the k-th tile in order
+    const int i = (int)k;
+    return k < (unsigned long long)ntiles ? Tile{(i % ntx) * TX, (i / ntx) * TY, i} : Tile{-1, 0, 0};
   };
-  auto take = [&]() {  // thread 0: the next tile in order, or ntiles when none is left
-    const unsigned long long k = atomicAdd(tickets, 1ull);
-    return k < (unsigned long long)ntiles ? (int)k : ntiles;
-  };
+  // whether a tile, its 2-ring and their pull sources stay inside the domain
+  auto inside = [&](const Tile& t) { return t.x >= 3 && t.x + TX + 3 <= P.nx && t.y >= 3 && t.y + TY + 3 <= P.ny; };
   pdl_wait<TX * TY / NPT>();  // every address below depends on a ticket or a staged copy taken after it
+  // the first tile of a CTA is its own number's, the later ones are tickets
+  auto take = [&]() { return gridDim.x + atomicAdd(tickets, 1ull); };
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
-    const int t0 = take();
-    int x0, y0;
-    if (t0 < ntiles && origin(t0, x0, y0)) tma_issue_tile<S, TX, TY>(dyn, bar, maps, x0, y0);
+    const Tile t0 = tile_at(blockIdx.x);
+    if (inside(t0)) tma_issue_tile<S, TX, TY>(dyn, bar, maps, t0.x, t0.y);
     s_tile[0] = t0;
-    s_next[0] = t0 < ntiles ? take() : ntiles;
+    s_next[0] = tile_at(take());
   }
   __syncthreads();
   unsigned parity = 0;  // of the mbarrier phase awaited next
   for (int it = 0;; it ^= 1) {
-    const int tile = s_tile[it];
-    if (tile >= ntiles) break;
-    // thread 0 starts the copy of the next tile, if interior, and records it and the tile after it as
-    // the next iteration's walk state
-    auto start_next = [&]() {
+    const Tile tile = s_tile[it];
+    if (tile.x < 0) break;
+    // Thread 0 takes the ticket of the tile after the next one here and turns it into a tile at the end of this
+    // one: the counter's answer takes most of a microsecond, and waiting for it where the next copy starts held
+    // the whole block at its next barrier.
+    unsigned long long ticket = 0;
+    if (threadIdx.x == 0) ticket = take();
+    auto start_next = [&]() {  // thread 0 starts the copy of the next tile, if interior
       if (threadIdx.x != 0) return;
-      const int next = s_next[it];
-      int nx0, ny0;
-      if (next < ntiles && origin(next, nx0, ny0)) tma_issue_tile<S, TX, TY>(dyn, bar, maps, nx0, ny0);
-      s_tile[it ^ 1] = next;
-      s_next[it ^ 1] = next < ntiles ? take() : ntiles;
+      const Tile next = s_next[it];
+      if (inside(next)) tma_issue_tile<S, TX, TY>(dyn, bar, maps, next.x, next.y);
     };
-    int x0, y0;
-    if (origin(tile, x0, y0)) {
+    if (inside(tile)) {
       if (!mbar_wait_bounded(bar, parity)) {
-        if (threadIdx.x == 0) report(status, step, x0, y0, ST_TIMEOUT);
+        if (threadIdx.x == 0) report(status, step, tile.x, tile.y, ST_TIMEOUT);
         mbar_wait_bounded(bar, parity);  // let the copy in flight land before the block's shared memory goes away
-        return;
+        break;
       }
       parity ^= 1u;
       fused_body<2, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
-                                       x0, y0, tile, TmaTile<S>{dyn}, nullptr, start_next);
+                                       tile.x, tile.y, tile.index, TmaTile<S>{dyn}, nullptr, start_next);
     } else {
       start_next();
       fused_body<0, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
-                                       x0, y0, tile);
+                                       tile.x, tile.y, tile.index);
+    }
+    if (threadIdx.x == 0) {
+      s_tile[it ^ 1] = s_next[it];
+      s_next[it ^ 1] = tile_at(ticket);
     }
     __syncthreads();  // the tile body is done with the shared arrays; the next walk state has landed
   }
+  // The last CTA to end puts the counter back to zero for the next launch (a CTA has its last ticket's answer
+  // when it comes here); the count of ended CTAs wraps to zero by itself.
+  if (threadIdx.x == 0 && atomicInc((unsigned*)(tickets + 1), gridDim.x - 1) == gridDim.x - 1)
+    atomicExch(tickets, 0ull);
 }
 
 // Resident CTAs of the persistent kernel on the current device (SMs x CTAs per SM), queried once per
@@ -209,11 +216,11 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
         if (e != cudaSuccess) return e;
         int resident = 0;  // CTAs of the persistent kernel that fit on the device at once
         if ((e = loop_residency<S, R, TX, TY, NPT>(B::BYTES, &resident)) != cudaSuccess) return e;
-        // persistent CTAs pay off where each walks many tiles (measured: +5 % to +12 % in FP32 from
-        // 2048^2, 27 or more per CTA; 1-8 % slower at 1024^2, 7 per CTA); smaller grids take one CTA per tile
-        if ((long long)grid.x * grid.y > 8LL * resident) {
+        // Persistent CTAs pay off where each walks many tiles, more of them in FP16, whose tiles are shorter of
+        // memory time to hide. FP32, one CTA per tile against persistent: 768^2 (3.8 tiles per CTA) 21.6, 23.0 us;
+        // 1024^2 (6.7) 38.3, 36.6; 2048^2 131, 113. FP16: 1024^2 45.1, 48.8; 1536^2 (15) 85.5, 85.6; 2048^2 138, 135.
+        if ((long long)grid.x * grid.y > (is_half_t<S>::value ? 12LL : 5LL) * resident) {
           unsigned long long* tickets = (unsigned long long*)(b.status + 6);
-          if ((e = cudaMemsetAsync(tickets, 0, sizeof *tickets, st)) != cudaSuccess) return e;
           if ((e = launch_pdl(k_fused_tma_loop<S, R, TX, TY, NPT>, resident, TX * TY / NPT, B::BYTES, st, fs, gs, fd, gd,
                               (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, tickets,
                               *b.tma[cur])) != cudaSuccess)
@@ -272,7 +279,7 @@ static bool encode_t(TmaMaps* m, void* f, void* g, float* rf, float* rg, const D
                                                 : (sizeof(S) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64);
   const cuuint64_t dims[3] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny, 9};
   const cuuint64_t strides[2] = {(cuuint64_t)P.nx * sizeof(S), (cuuint64_t)P.N * sizeof(S)};
-  const cuuint32_t box[3] = {(cuuint32_t)B::BX, (cuuint32_t)B::BY, 1};
+  const cuuint32_t box[3] = {(cuuint32_t)B::BX, (cuuint32_t)B::BY, 9};
   const cuuint32_t es[3] = {1, 1, 1};
   auto enc3 = [&](CUtensorMap* t, void* base) {
     return fn(t, dt, 3, base, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,

@@ -46,11 +46,12 @@ template <class S, int TX, int TY> struct TmaBox {
   static constexpr int EPR = 16 / (int)sizeof(S);                // elements per 16 bytes
   static constexpr int BX = ((TX + XOFF + 3 + EPR - 1) / EPR) * EPR;
   static constexpr int BY = TY + 6;
-  static constexpr int PLANE = ((BX * BY * (int)sizeof(S) + 127) / 128) * 128;  // bytes, 128-aligned
+  static constexpr int PLANE = BX * BY * (int)sizeof(S);                        // bytes
+  static constexpr int SET = ((9 * PLANE + 127) / 128) * 128;                   // f or g: one copy of nine planes
   static constexpr int REFX = ((TX + XOFF + 3 + 3) / 4) * 4;                    // float reference planes
   static constexpr int RPLANE = ((REFX * BY * 4 + 127) / 128) * 128;
   static constexpr bool HALF = is_half_t<S>::value;
-  static constexpr int BYTES = 18 * PLANE + (HALF ? 2 * RPLANE : 0) + 128;       // + the mbarrier
+  static constexpr int BYTES = 2 * SET + (HALF ? 2 * RPLANE : 0) + 128;       // + the mbarrier
 };
 
 struct alignas(64) TmaMaps {
@@ -79,7 +80,7 @@ struct SplitBuffers {
   void* planes[16];  // scratch planes of the split kernels, arithmetic type
   double* partials;  // per-block (split) or per-tile (fused) partial sums: max(2 * nblocks, fused_max_tiles)
   double* scalars;   // [0] rho_ave, [1] mass, [2] heat
-  long long* status; // [0] flag, [1] step, [2] x, [3] y, [4] code; [6] tile tickets of the persistent fused step
+  long long* status; // [0] flag, [1] step, [2] x, [3] y, [4] code; [6], [7] tile tickets and ended CTAs of the persistent fused step, zero between launches
   const TmaMaps* tma[2] = {nullptr, nullptr};  // tensor maps of buffer A / B for the TMA-staged fused step
   int fused_tile = 1;  // 0: 32x16, 1: 32x8, 2: 32x16 two nodes per thread, 3: 32x32 two per thread (maps match)
 };

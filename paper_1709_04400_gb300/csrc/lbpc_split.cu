@@ -109,8 +109,7 @@ __global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc,
         gdst[P.N + i] = n6;
       }
     }
-    const int bad = classify(rho, T, psi2, P);
-    if (bad) report(status, step, x, y, bad);
+    check_node(rho, T, psi2, P, status, nullptr, step, x, y);
     pl.p[P_RHO][i] = rho;
     pl.p[P_T][i] = T;
     pl.p[P_PSI][i] = psi_of(psi2);

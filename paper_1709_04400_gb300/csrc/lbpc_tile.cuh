@@ -103,8 +103,8 @@ template <class S> struct TmaTile {
 template <class S, class R, int TX, int TY>
 __device__ __forceinline__ void pull_staged(const TmaTile<S>& t, int set, const R* w, int hx, int hy, R v[9]) {
   using B = TmaBox<S, TX, TY>;
-  const S* pop = (const S*)(t.base + (size_t)set * 9 * B::PLANE);
-  const float* ref = (const float*)(t.base + 18 * B::PLANE + (size_t)set * B::RPLANE);
+  const S* pop = (const S*)(t.base + (size_t)set * B::SET);
+  const float* ref = (const float*)(t.base + 2 * B::SET + (size_t)set * B::RPLANE);
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     const int row = hy + 1 - EY(a), col = hx + B::XOFF - 2 - EX(a);
@@ -196,7 +196,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     const int n = t + k * NTH;
     const int tx = n % TX, ty = n / TX;
     const int gx = x0 + tx, gy = y0 + ty;
-    active[k] = gx < P.nx && gy < P.ny;
+    active[k] = INTERIOR || (gx < P.nx && gy < P.ny);
     if constexpr (IDX32)
       pp[k] = (active[k] && P.model == 0 && !first) ? __ldg(phi_prev + ((IX)gy * P.nx + gx)) : R(0);
     else
@@ -231,10 +231,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     R Tlo;
     T[k] = heat_of(gk, Tlo);
     const R psi2 = node_psi_squared(rho[k], T[k], Tlo, P, dpdT[k]);
-    if (active[k]) {
-      const int bad = classify(rho[k], T[k], psi2, P);
-      if (bad) report(status, step_at ? *step_at : step, gx, gy, bad);  // step_at: read only to report
-    }
+    if (active[k]) check_node(rho[k], T[k], psi2, P, status, step_at, step, gx, gy);
     s_rho[ty + 2][tx + 2] = rho[k];
     s_T[ty + 2][tx + 2] = T[k];
     s_psi[ty + 2][tx + 2] = psi_of(psi2);
@@ -319,7 +316,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
       Fy += d * C.gy;
     }
     Q = C.qG2 * (sx * sx + sy * sy);
-    const R ir = R(1) / rr;
+    const R ir = inverse_of(rr);
     vx = (s_jx[hy][hx] + Fx * 0.5f) * ir;
     vy = (s_jy[hy][hx] + Fy * 0.5f) * ir;
   };
@@ -384,7 +381,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
                    (s_vy[uy + 1][ux] - s_vy[uy - 1][ux]) * R(1.0 / 3.0) +
                    (s_vy[uy + 1][ux + 1] + s_vy[uy + 1][ux - 1] - s_vy[uy - 1][ux - 1] - s_vy[uy - 1][ux + 1]) * R(1.0 / 12.0);
     const R rcv = rho[k] * C.cV;
-    const R inv_rcv = R(1) / rcv;
+    const R inv_rcv = inverse_of(rcv);
     R div_lam_gradT;
     if (P.lambda_mode == 0) {
       div_lam_gradT = C.lambda * lapT;
@@ -401,7 +398,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     if (P.model == 2) {  // Gong-Cheng: Eq. 13 source, local tau_g (Sec. IV A)
       phi = compress;
       S0 = phi;
-      tau_inv = R(1) / ((P.lambda_mode == 0 ? C.lambda * 3 * inv_rcv : C.chi * 3) + R(0.5));
+      tau_inv = inverse_of((P.lambda_mode == 0 ? C.lambda * 3 * inv_rcv : C.chi * 3) + R(0.5));
     } else {
       phi = div_lam_gradT * inv_rcv - C.kdiff * lapT + compress;
       S0 = phi;
