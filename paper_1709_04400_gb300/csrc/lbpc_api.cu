@@ -61,14 +61,16 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 struct Layout {
   size_t f[2], g[2], ref_f[2], ref_g[2], wall[2], phi, planes, partials, scalars, status, total;
   size_t store, real;
-  long long N;
+  int pitch;
+  long long N;  // pitch * ny
   int nblocks;
 };
 
 Layout layout_of(const lbpc_params* p) {
   Layout L{};
-  L.N = (long long)p->nx * p->ny;
   L.store = (p->prec == LBPC_FP64 || p->prec == LBPC_DF64) ? 8 : (p->prec == LBPC_FP32 ? 4 : 2);
+  L.pitch = lbpc::row_pitch(p->nx, p->ny, L.store);
+  L.N = (long long)L.pitch * p->ny;
   L.real = (p->prec == LBPC_FP64 || p->prec == LBPC_DF64) ? 8 : 4;
   L.nblocks = (int)((L.N + lbpc::split_block() - 1) / lbpc::split_block());
   size_t off = 0;
@@ -195,11 +197,12 @@ template <class R> void fill_coefs(lbpc::Coefs<R>& c, const lbpc_params* p) {
   }
 }
 
-DevParams make_dev_params(const lbpc_params* p) {
+DevParams make_dev_params(const lbpc_params* p, int pitch) {
   DevParams d{};
   d.nx = p->nx;
   d.ny = p->ny;
-  d.N = (long long)p->nx * p->ny;
+  d.pitch = pitch;
+  d.N = (long long)pitch * p->ny;
   d.yper = p->flow_bc[2] == LBPC_PERIODIC;
   d.ybc_lo = p->flow_bc[2];
   d.ybc_hi = p->flow_bc[3];
@@ -253,7 +256,7 @@ template <class F> double bisect(F fn, double lo, double hi) {
 }  // namespace
 
 namespace lbpc {
-DevParams make_dev_params_public(const lbpc_params* p) { return make_dev_params(p); }
+DevParams make_dev_params_public(const lbpc_params* p, int pitch) { return make_dev_params(p, pitch); }
 }  // namespace lbpc
 
 // ================================================================================================
@@ -374,7 +377,7 @@ LBPC_API lbpc_status lbpc_create(const lbpc_params* p, void* ws, size_t bytes, v
   if (!c) return LBPC_ENOMEM;
   memset(c, 0, sizeof(lbpc_ctx));
   c->p = *p;
-  c->dp = make_dev_params(p);
+  c->dp = make_dev_params(p, L.pitch);
   if (cudaGetDevice(&c->device) != cudaSuccess) {
     free(c);
     return LBPC_ECUDA;
@@ -417,22 +420,23 @@ LBPC_API lbpc_status lbpc_init(lbpc_ctx* c, const double* rho, const double* T, 
   if (c->err != LBPC_OK) return LBPC_ESTATE;
   if (!rho || !T) return fail(c, LBPC_EINVAL, "lbpc_init: rho and T are required");
   DeviceGuard g(c->device);
-  const size_t nb = (size_t)c->dp.N * sizeof(double);
+  const long long N = (long long)c->p.nx * c->p.ny;
+  const size_t nb = (size_t)N * sizeof(double);
   const double *d_rho = rho, *d_T = T, *d_ux = ux, *d_uy = uy;
   if (!on_device) {  // stage in the B half (the init kernel writes the A half)
     double* s = (double*)c->buf.f[1];
     CU(c, cudaMemcpyAsync(s, rho, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D rho");
-    CU(c, cudaMemcpyAsync(s + c->dp.N, T, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D T");
+    CU(c, cudaMemcpyAsync(s + N, T, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D T");
     d_rho = s;
-    d_T = s + c->dp.N;
+    d_T = s + N;
     d_ux = d_uy = nullptr;
     if (ux) {
-      CU(c, cudaMemcpyAsync(s + 2 * c->dp.N, ux, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D ux");
-      d_ux = s + 2 * c->dp.N;
+      CU(c, cudaMemcpyAsync(s + 2 * N, ux, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D ux");
+      d_ux = s + 2 * N;
     }
     if (uy) {
-      CU(c, cudaMemcpyAsync(s + 3 * c->dp.N, uy, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D uy");
-      d_uy = s + 3 * c->dp.N;
+      CU(c, cudaMemcpyAsync(s + 3 * N, uy, nb, cudaMemcpyHostToDevice, c->stream), "lbpc_init H2D uy");
+      d_uy = s + 3 * N;
     }
   }
   CU(c, cudaMemsetAsync(c->buf.status, 0, 8 * sizeof(long long), c->stream), "lbpc_init status reset");
@@ -459,11 +463,11 @@ static cudaError_t launch_step(lbpc_ctx* c, cudaEvent_t* ev) {
 }
 
 static int step_kernel_count(const lbpc_ctx* c) {
-  return use_fused(c) ? (c->dp.buoyancy == 1 ? 2 : 1) : lbpc::split_kernel_count(c->dp, c->p.prec);
+  return use_fused(c) ? 1 : lbpc::split_kernel_count(c->dp, c->p.prec);
 }
 
 static const char* step_kernel_name(const lbpc_ctx* c, int k) {
-  if (use_fused(c)) return k == 0 ? "k_fused" : (k == 1 ? "k_finish" : "");
+  if (use_fused(c)) return k == 0 ? "k_fused" : "";
   return lbpc::split_kernel_name(c->p.prec, k);
 }
 
@@ -564,7 +568,7 @@ LBPC_API lbpc_status lbpc_fields(lbpc_ctx* c, double* rho, double* ux, double* u
   if (!c) return LBPC_EINVAL;
   if (!c->initialised) return LBPC_ESTATE;
   DeviceGuard g(c->device);
-  const long long N = c->dp.N;
+  const long long N = (long long)c->p.nx * c->p.ny;
   const size_t nb = (size_t)N * sizeof(double);
   if (on_device) {
     CU(c, lbpc::split_fields(c->buf, c->dp, c->p.prec, c->cur, c->step, rho, ux, uy, T, c->stream), "lbpc_fields kernels");
@@ -603,10 +607,20 @@ static_assert(sizeof(lbpc_params) == 16 * 4 + 39 * 8, "lbpc_params has no paddin
 
 void ckpt_sizes(const lbpc_ctx* c, size_t& pop, size_t& ref, size_t& phi, size_t& wall) {
   const Layout L = layout_of(&c->p);
-  pop = 9 * (size_t)L.N * L.store;
-  ref = c->p.prec == LBPC_FP16DEV ? (size_t)L.N * sizeof(float) : 0;
-  phi = (size_t)L.N * L.real;
+  const size_t nodes = (size_t)c->p.nx * c->p.ny;
+  pop = 9 * nodes * L.store;
+  ref = c->p.prec == LBPC_FP16DEV ? nodes * sizeof(float) : 0;
+  phi = nodes * L.real;
   wall = (size_t)lbpc::wall_doubles(c->p.nx) * sizeof(double);
+}
+
+// Copy rows rows of nx elements between a plane set of the context (rows pitch elements apart) and a buffer without
+// padding.
+cudaError_t copy_rows(const lbpc_ctx* c, void* dst, bool dst_padded, const void* src, size_t elem, size_t rows,
+                      cudaMemcpyKind kind) {
+  const size_t row = (size_t)c->p.nx * elem, pitch = (size_t)c->dp.pitch * elem;
+  if (row == pitch) return cudaMemcpyAsync(dst, src, row * rows, kind, c->stream);
+  return cudaMemcpy2DAsync(dst, dst_padded ? pitch : row, src, dst_padded ? row : pitch, row, rows, kind, c->stream);
 }
 }  // namespace
 
@@ -647,17 +661,19 @@ LBPC_API lbpc_status lbpc_save(lbpc_ctx* c, void* buf, size_t bytes, int on_devi
                         c->stream),
      "lbpc_save header");
   size_t off = kCkptHeader;
-  CU(c, cudaMemcpyAsync(dst + off, c->buf.f[c->cur], pop, d2x, c->stream), "lbpc_save f");
+  const Layout L = layout_of(&c->p);
+  const size_t ny = (size_t)c->p.ny;
+  CU(c, copy_rows(c, dst + off, false, c->buf.f[c->cur], L.store, 9 * ny, d2x), "lbpc_save f");
   off += pop;
-  CU(c, cudaMemcpyAsync(dst + off, c->buf.g[c->cur], pop, d2x, c->stream), "lbpc_save g");
+  CU(c, copy_rows(c, dst + off, false, c->buf.g[c->cur], L.store, 9 * ny, d2x), "lbpc_save g");
   off += pop;
   if (ref) {
-    CU(c, cudaMemcpyAsync(dst + off, c->buf.ref_f[c->cur], ref, d2x, c->stream), "lbpc_save ref_f");
+    CU(c, copy_rows(c, dst + off, false, c->buf.ref_f[c->cur], sizeof(float), ny, d2x), "lbpc_save ref_f");
     off += ref;
-    CU(c, cudaMemcpyAsync(dst + off, c->buf.ref_g[c->cur], ref, d2x, c->stream), "lbpc_save ref_g");
+    CU(c, copy_rows(c, dst + off, false, c->buf.ref_g[c->cur], sizeof(float), ny, d2x), "lbpc_save ref_g");
     off += ref;
   }
-  CU(c, cudaMemcpyAsync(dst + off, c->buf.phi_prev, phi, d2x, c->stream), "lbpc_save phi_prev");
+  CU(c, copy_rows(c, dst + off, false, c->buf.phi_prev, L.real, ny, d2x), "lbpc_save phi_prev");
   off += phi;
   CU(c, cudaMemcpyAsync(dst + off, c->buf.wall[c->cur], wall, d2x, c->stream), "lbpc_save wall");
   CU(c, cudaStreamSynchronize(c->stream), "lbpc_save sync");
@@ -687,17 +703,19 @@ LBPC_API lbpc_status lbpc_load(lbpc_ctx* c, const void* buf, size_t bytes, int o
     return fail(c, LBPC_EINVAL, "lbpc_load: section sizes do not match");
   const cudaMemcpyKind x2d = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
   size_t off = kCkptHeader;
-  CU(c, cudaMemcpyAsync(c->buf.f[0], src + off, pop, x2d, c->stream), "lbpc_load f");
+  const Layout L = layout_of(&c->p);
+  const size_t ny = (size_t)c->p.ny;
+  CU(c, copy_rows(c, c->buf.f[0], true, src + off, L.store, 9 * ny, x2d), "lbpc_load f");
   off += pop;
-  CU(c, cudaMemcpyAsync(c->buf.g[0], src + off, pop, x2d, c->stream), "lbpc_load g");
+  CU(c, copy_rows(c, c->buf.g[0], true, src + off, L.store, 9 * ny, x2d), "lbpc_load g");
   off += pop;
   if (ref) {
-    CU(c, cudaMemcpyAsync(c->buf.ref_f[0], src + off, ref, x2d, c->stream), "lbpc_load ref_f");
+    CU(c, copy_rows(c, c->buf.ref_f[0], true, src + off, sizeof(float), ny, x2d), "lbpc_load ref_f");
     off += ref;
-    CU(c, cudaMemcpyAsync(c->buf.ref_g[0], src + off, ref, x2d, c->stream), "lbpc_load ref_g");
+    CU(c, copy_rows(c, c->buf.ref_g[0], true, src + off, sizeof(float), ny, x2d), "lbpc_load ref_g");
     off += ref;
   }
-  CU(c, cudaMemcpyAsync(c->buf.phi_prev, src + off, phi, x2d, c->stream), "lbpc_load phi_prev");
+  CU(c, copy_rows(c, c->buf.phi_prev, true, src + off, L.real, ny, x2d), "lbpc_load phi_prev");
   off += phi;
   CU(c, cudaMemcpyAsync(c->buf.wall[0], src + off, wall, x2d, c->stream), "lbpc_load wall");
   CU(c, cudaMemcpyAsync(c->buf.scalars, &h.rho_ave, sizeof(double), cudaMemcpyHostToDevice, c->stream),
@@ -757,9 +775,10 @@ LBPC_API lbpc_status lbpc_populations(lbpc_ctx* c, double* f, double* g, int on_
   if (!c) return LBPC_EINVAL;
   if (!c->initialised) return LBPC_ESTATE;
   DeviceGuard dg(c->device);
-  const size_t nb = 9 * (size_t)c->dp.N * sizeof(double);
+  const size_t N = (size_t)c->p.nx * c->p.ny;
+  const size_t nb = 9 * N * sizeof(double);
   double* outs[2] = {f, g};
-  const size_t plane = (size_t)c->dp.N * sizeof(double);
+  const size_t plane = N * sizeof(double);
   for (int which = 0; which < 2; ++which) {
     if (!outs[which]) continue;
     if (on_device) {
@@ -775,7 +794,7 @@ LBPC_API lbpc_status lbpc_populations(lbpc_ctx* c, double* f, double* g, int on_
       for (int a = 0; a < 9; ++a) {
         CU(c, lbpc::split_export_pops(c->buf, c->dp, c->p.prec, c->cur, which, a, dst, c->stream),
            "lbpc_populations kernel");
-        CU(c, cudaMemcpyAsync(outs[which] + (size_t)a * c->dp.N, dst, plane, cudaMemcpyDeviceToHost, c->stream),
+        CU(c, cudaMemcpyAsync(outs[which] + (size_t)a * N, dst, plane, cudaMemcpyDeviceToHost, c->stream),
            "lbpc_populations D2H");
         CU(c, cudaStreamSynchronize(c->stream), "lbpc_populations sync");
       }

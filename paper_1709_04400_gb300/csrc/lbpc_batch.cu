@@ -22,7 +22,7 @@
 #define LBPC_API extern "C" __attribute__((visibility("default")))
 
 namespace lbpc {
-DevParams make_dev_params_public(const lbpc_params* p);
+DevParams make_dev_params_public(const lbpc_params* p, int pitch);
 }
 
 namespace {
@@ -86,7 +86,7 @@ struct HostInst {
   bool used = false;
   lbpc_params p{};
   lbpc::DevParams dp{};
-  long long N = 0;
+  long long N = 0;  // nodes
   size_t off = 0, bytes = 0;  // arena block of the instance
   size_t f[2], g[2], rf[2], rg[2], wall[2], phi, partials, scalars;
   size_t npartials = 0;
@@ -99,8 +99,8 @@ size_t real_bytes(int prec) { return prec == LBPC_FP64 ? 8 : 4; }
 
 // Lay out one instance inside a block starting at 0; returns the block size.
 size_t layout_instance(const lbpc_params* p, HostInst* h) {
-  const long long N = (long long)p->nx * p->ny;
   const size_t sb = store_bytes(p->prec), rb = real_bytes(p->prec);
+  const long long N = (long long)lbpc::row_pitch(p->nx, p->ny, sb) * p->ny;
   const size_t pop = a256(9 * (size_t)N * sb);
   size_t off = 0;
   // f0 g0 f1 g1 contiguous so the dead half can stage FP64 transfers
@@ -288,7 +288,7 @@ lbpc::SplitBuffers split_view(lbpc_batch* b, const HostInst& h, char* scratch) {
   s.scalars = (double*)(base + h.scalars);
   s.status = (long long*)(b->base + b->status_off) + 8 * (&h - b->inst.data());
   if (scratch) {
-    const size_t plane = a256((size_t)h.N * real_bytes(b->prec));
+    const size_t plane = a256((size_t)h.dp.N * real_bytes(b->prec));
     for (int k = 0; k < lbpc::split_nplanes(); ++k) s.planes[k] = scratch + k * plane;
   }
   return s;
@@ -498,7 +498,7 @@ LBPC_API lbpc_status lbpc_batch_add(lbpc_batch* b, const lbpc_params* p, const d
   }
   HostInst h;
   h.p = *p;
-  h.dp = lbpc::make_dev_params_public(p);
+  h.dp = lbpc::make_dev_params_public(p, lbpc::row_pitch(p->nx, p->ny, store_bytes(p->prec)));
   h.N = (long long)p->nx * p->ny;
   h.bytes = layout_instance(p, &h);
   if (!b->arena.alloc(h.bytes, &h.off)) {
@@ -602,7 +602,7 @@ LBPC_API lbpc_status lbpc_batch_fields(lbpc_batch* b, int32_t id, double* rho, d
   if (!b || id < 0 || id >= (int)b->inst.size() || !b->inst[id].used) return LBPC_EINVAL;
   DevGuard g(b->device);
   HostInst& h = b->inst[id];
-  const size_t plane = a256((size_t)h.N * real_bytes(b->prec));
+  const size_t plane = a256((size_t)h.dp.N * real_bytes(b->prec));
   const size_t sbytes = plane * lbpc::split_nplanes();
   size_t soff;
   if (!b->arena.alloc(sbytes, &soff)) return bfail(b, LBPC_ENOMEM, "lbpc_batch_fields: no room for %zu scratch bytes", sbytes);

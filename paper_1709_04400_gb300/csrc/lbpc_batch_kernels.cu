@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(128) k_batch_advance(BatchInst<S>* __restrict_
     double acc = 0.0;
     for (int j = threadIdx.x; j < I.ntiles; j += 128) acc += I.partials[j];
     acc = block_sum<128>(acc, red);
-    if (threadIdx.x == 0) I.scalars[0] = acc / (double)I.P.N;
+    if (threadIdx.x == 0) I.scalars[0] = acc / node_count(I.P);
   }
   if (threadIdx.x == 0) {
     I.cur ^= 1;

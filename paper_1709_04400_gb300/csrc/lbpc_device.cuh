@@ -70,7 +70,7 @@ template <class R> struct Coefs {
 // it uses with 16-byte asynchronous copies.
 struct alignas(16) DevParams {
   int nx, ny;
-  long long N;       // nx * ny
+  long long N;       // pitch * ny: elements of a plane, the stride between planes
   int yper;          // y periodic
   int ybc_lo, ybc_hi;
   int tbc[4];
@@ -79,6 +79,7 @@ struct alignas(16) DevParams {
   int lambda_mode;   // 0 const, 1 rho cV chi
   int buoyancy;
   int heat_unit_rates;  // s_g[1..8] all 1: the thermal relaxation sets every non-conserved moment to m_eq
+  int pitch;         // elements of a stored row: nx, or nx rounded up to whole 16-byte pieces (row_pitch)
   alignas(16) Coefs<double> cd;
   alignas(16) Coefs<float> cf;
   alignas(16) Coefs<dw> cw;  // double-word arithmetic (LBPC_DF64)
@@ -103,10 +104,11 @@ template <class R> struct alignas(16) DevParamsOf {
   int lambda_mode;
   int buoyancy;
   int heat_unit_rates;
+  int pitch;
   alignas(16) Coefs<R> c;
 };
 static_assert(offsetof(DevParamsOf<float>, c) == offsetof(DevParams, cd) &&
-                  offsetof(DevParamsOf<float>, heat_unit_rates) == offsetof(DevParams, heat_unit_rates),
+                  offsetof(DevParamsOf<float>, pitch) == offsetof(DevParams, pitch),
               "DevParamsOf repeats the header of DevParams");
 template <class R> __host__ __device__ __forceinline__ const Coefs<R>& coefs(const DevParamsOf<R>& P) { return P.c; }
 template <class R> inline DevParamsOf<R> params_of(const DevParams& P) {
@@ -374,6 +376,9 @@ template <class S> struct PopBuf {
   double* wall;  // flow buffers: wall-row forces (null where unused; aggregate init leaves it null)
 };
 
+// nodes of a domain
+template <class PT> __host__ __device__ __forceinline__ double node_count(const PT& P) { return (double)P.nx * (double)P.ny; }
+
 // Index of a wall row's entries in PopBuf::wall: edge 0 = y-, 1 = y+; component 0 = Fx, 1 = Fy.
 __host__ __device__ __forceinline__ long long wall_slot(int nx, int edge, int comp, int x) {
   return (long long)(2 * edge + comp) * nx + x;
@@ -457,7 +462,7 @@ __device__ __forceinline__ void pull_from(const PopBuf<S>& src, const R* w, cons
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     const int r = s.row[EY(a) + 1];
-    v[a] = r >= 0 ? pop_load<S, R, IX>(src, (IX)P.N, a, (IX)r * P.nx + s.col[EX(a) + 1], w) : R(0);
+    v[a] = r >= 0 ? pop_load<S, R, IX>(src, (IX)P.N, a, (IX)r * P.pitch + s.col[EX(a) + 1], w) : R(0);
   }
 }
 

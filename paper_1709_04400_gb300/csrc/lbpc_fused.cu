@@ -13,7 +13,7 @@ namespace lbpc {
 template <class S, class R, int TX, int TY, int NPT>
 __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NPT, NPT>()) k_fused(PopBuf<S> fsrc, PopBuf<S> gsrc, PopBuf<S> fdst, PopBuf<S> gdst,
                                                    R* __restrict__ phi_prev, DevParams P, long long step, int first,
-                                                   const double* __restrict__ rho_ave, double* __restrict__ partials,
+                                                   const MeanOf mean, double* __restrict__ partials,
                                                    long long* __restrict__ status) {
   __shared__ FusedSmem<R, TX, TY> sm;
   const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
@@ -21,11 +21,11 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   const int pslot = blockIdx.y * gridDim.x + blockIdx.x;
   const int t = pdl_wait<TX * TY / NPT>();
   if (interior)
-    fused_body<1, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
-                                     x0, y0, pslot);
+    fused_body<1, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, mean.out, partials, status, sm,
+                                     x0, y0, pslot, TmaTile<S>{nullptr}, nullptr, NoStageHook{}, &mean);
   else
-    fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
-                                     x0, y0, pslot);
+    fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, mean.out, partials, status, sm,
+                                     x0, y0, pslot, TmaTile<S>{nullptr}, nullptr, NoStageHook{}, &mean);
 }
 
 // Same step with the interior tiles' populations staged in shared memory by TMA (dynamic shared
@@ -202,10 +202,13 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
   dim3 grid((P.nx + TX - 1) / TX, (P.ny + TY - 1) / TY);
   const PopBuf<S> fs{(S*)b.f[cur], b.ref_f[cur], b.wall[cur]}, gs{(S*)b.g[cur], b.ref_g[cur]};
   const PopBuf<S> fd{(S*)b.f[cur ^ 1], b.ref_f[cur ^ 1], b.wall[cur ^ 1]}, gd{(S*)b.g[cur ^ 1], b.ref_g[cur ^ 1]};
+  const MeanOf mean{b.scalars, (unsigned*)(b.status + 5), grid.x * grid.y, 1.0 / node_count(P)};
   if (ev) cudaEventRecord(ev[0], st);
   bool staged = false;
   if constexpr (sizeof(S) <= 4) {  // the TMA-staged kernel exists for FP32 and FP16 storage
-    if (b.tma[cur]) {
+    // FP32 grids of less than one tile per resident CTA pull straight from L2: nothing is left to overlap the staging
+    // with (256^2 5.5 us against 6.2, 150 x 300 9.1 against 9.4; 300 x 400 7.9 against 7.7). FP16 is staged at every size.
+    if (b.tma[cur] && (is_half_t<S>::value || P.N >= 100000)) {
       using B = TmaBox<S, TX, TY>;
       // The dynamic shared-memory limit is held per device context, so it is set before every launch:
       // the call is cheap, thread-safe, and right after a device reset or on a second device.
@@ -236,19 +239,17 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
                             (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, *b.tma[cur])) != cudaSuccess)
           return e;
       }
+      // the mean as a kernel of its own: its code in the staged kernels costs every step of theirs 2 to 5 %
+      if (P.buoyancy == 1) fused_finish(b, P, (int)(grid.x * grid.y), st);
       staged = true;
     }
   }
   if (!staged) {
     const cudaError_t e = launch_pdl(k_fused<S, R, TX, TY, NPT>, grid, TX * TY / NPT, 0, st, fs, gs, fd, gd, (R*)b.phi_prev,
-                                     P, step, step == 0, b.scalars, b.partials, b.status);
+                                     P, step, step == 0, mean, b.partials, b.status);
     if (e != cudaSuccess) return e;
   }
   if (ev) cudaEventRecord(ev[1], st);
-  if (P.buoyancy == 1) {
-    fused_finish(b, P, (int)(grid.x * grid.y), st);
-    if (ev) cudaEventRecord(ev[2], st);
-  }
   return cudaGetLastError();
 }
 
@@ -274,11 +275,11 @@ static bool encode_t(TmaMaps* m, void* f, void* g, float* rf, float* rg, const D
   using B = TmaBox<S, TX, TY>;
   auto fn = encode_fn();
   if (!fn) return false;
-  if (((size_t)P.nx * sizeof(S)) % 16 != 0) return false;  // row stride must be a multiple of 16 bytes
+  if (((size_t)P.pitch * sizeof(S)) % 16 != 0) return false;  // row stride must be a multiple of 16 bytes
   const CUtensorMapDataType dt = sizeof(S) == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
                                                 : (sizeof(S) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64);
   const cuuint64_t dims[3] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny, 9};
-  const cuuint64_t strides[2] = {(cuuint64_t)P.nx * sizeof(S), (cuuint64_t)P.N * sizeof(S)};
+  const cuuint64_t strides[2] = {(cuuint64_t)P.pitch * sizeof(S), (cuuint64_t)P.N * sizeof(S)};
   const cuuint32_t box[3] = {(cuuint32_t)B::BX, (cuuint32_t)B::BY, 9};
   const cuuint32_t es[3] = {1, 1, 1};
   auto enc3 = [&](CUtensorMap* t, void* base) {
@@ -288,7 +289,7 @@ static bool encode_t(TmaMaps* m, void* f, void* g, float* rf, float* rg, const D
   if (!enc3(&m->f, f) || !enc3(&m->g, g)) return false;
   if (B::HALF) {
     const cuuint64_t d2[2] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny};
-    const cuuint64_t s2[1] = {(cuuint64_t)P.nx * 4};
+    const cuuint64_t s2[1] = {(cuuint64_t)P.pitch * 4};
     const cuuint32_t b2[2] = {(cuuint32_t)B::REFX, (cuuint32_t)B::BY};
     auto enc2 = [&](CUtensorMap* t, void* base) {
       return fn(t, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, d2, s2, b2, es, CU_TENSOR_MAP_INTERLEAVE_NONE,

@@ -69,6 +69,17 @@ inline size_t fused_max_tiles(int nx, int ny) { return (size_t)((nx + 31) / 32) 
 // FP32 and FP16).
 constexpr int kDefaultFusedTile = 4;
 
+// Elements of a stored row of populations, phi and scratch planes. 4- and 2-byte rows are padded to whole 16-byte
+// pieces, which the tensor copies of the fused step need (a 1023 x 1025 FP32 step 43 us without them, 37 with). Rows
+// shorter than a tile with its rings, which no tensor copy serves, and a padding that would take a batch
+// instance's 32-bit population indices past their range are left alone. Data that enters or leaves the library
+// has no padding.
+inline int row_pitch(int nx, int ny, size_t store) {
+  if (store >= 8 || nx < 64) return nx;
+  const int per = (int)(16 / store), pitch = (nx + per - 1) / per * per;
+  return 9LL * pitch * ny > 2147483647LL && 9LL * nx * ny <= 2147483647LL ? nx : pitch;
+}
+
 // Device buffers of a context, carved from the caller's workspace.
 struct SplitBuffers {
   void* f[2];        // populations f, post-collision layout, A/B (storage type)
@@ -80,7 +91,7 @@ struct SplitBuffers {
   void* planes[16];  // scratch planes of the split kernels, arithmetic type
   double* partials;  // per-block (split) or per-tile (fused) partial sums: max(2 * nblocks, fused_max_tiles)
   double* scalars;   // [0] rho_ave, [1] mass, [2] heat
-  long long* status; // [0] flag, [1] step, [2] x, [3] y, [4] code; [6], [7] tile tickets and ended CTAs of the persistent fused step, zero between launches
+  long long* status; // [0] flag, [1] step, [2] x, [3] y, [4] code; [5] partial sums of rho written by the fused step, [6], [7] tile tickets and ended CTAs of the persistent fused step, zero between launches
   const TmaMaps* tma[2] = {nullptr, nullptr};  // tensor maps of buffer A / B for the TMA-staged fused step
   int fused_tile = 1;  // 0: 32x16, 1: 32x8, 2: 32x16 two nodes per thread, 3: 32x32 two per thread (maps match)
 };
@@ -97,7 +108,7 @@ cudaError_t split_sums(const SplitBuffers& b, const DevParams& P, int prec, int 
                        double* out = nullptr);
 cudaError_t split_fields(const SplitBuffers& b, const DevParams& P, int prec, int cur, long long step, double* rho,
                          double* ux, double* uy, double* T, cudaStream_t st);
-// which = 0: f, 1: g; only < 0: all 9 planes [9][N], else plane `only` into out[N].
+// which = 0: f, 1: g; only < 0: all 9 planes [9][ny][nx], else plane `only` into out[ny][nx].
 cudaError_t split_export_pops(const SplitBuffers& b, const DevParams& P, int prec, int cur, int which, int only,
                               double* out, cudaStream_t st);
 int split_nplanes();
@@ -190,7 +201,8 @@ cudaError_t fused_step(const SplitBuffers& b, const DevParams& P, int prec, int 
 // Encode the tensor maps of one buffer (populations f, g and, for FP16, the reference planes) for the
 // TMA-staged fused step; false when the layout does not allow TMA (row stride not 16-byte aligned).
 bool fused_tma_encode(TmaMaps* m, int prec, int tile, void* f, void* g, float* rf, float* rg, const DevParams& P);
-// rho_ave <- sum of n per-tile partials / N (fixed order), on st.
+
+// rho_ave <- sum of n per-tile partials / nodes (fixed order), on st.
 void fused_finish(const SplitBuffers& b, const DevParams& P, int n, cudaStream_t st);
 
 }  // namespace lbpc

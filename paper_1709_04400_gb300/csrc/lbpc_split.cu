@@ -31,7 +31,7 @@ template <class R> struct Planes {
   R* p[NPLANES];
 };
 
-__device__ __forceinline__ long long node_index(const DevParams& P, int x, int y) { return (long long)y * P.nx + x; }
+__device__ __forceinline__ long long node_index(const DevParams& P, int x, int y) { return (long long)y * P.pitch + x; }
 
 // Neighbour row for a stencil: wraps when y is periodic, else clamps to the edge row (ghost rows
 // copy the edge row). out_lo/out_hi report a ghost beyond the lower / upper edge.
@@ -50,7 +50,7 @@ template <class R> __device__ __forceinline__ void gather9(const R* __restrict__
 #pragma unroll
   for (int dy = -1; dy <= 1; ++dy) {
     bool lo, hi;
-    const long long row = (long long)nb_row(P, y, dy, lo, hi) * P.nx;
+    const long long row = (long long)nb_row(P, y, dy, lo, hi) * P.pitch;
     c[dy + 1][0] = ldgv(X + row + xm);
     c[dy + 1][1] = ldgv(X + row + x);
     c[dy + 1][2] = ldgv(X + row + xp);
@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc,
   const int t = pdl_wait<BLOCK>();
   const long long i = (long long)blockIdx.x * BLOCK + t;
   double rho_d = 0.0;
-  if (i < P.N) {
-    const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
+  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  if (i < P.N && x < P.nx) {
     R f[9], g[9];
     pull_closed<S, R>(fsrc, gsrc, P, x, y, f, g);
     R rho, jx, jy, Tlo, dpdT, inv_rho, psi2;
@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(BLOCK) k_force(Planes<R> pl, DevParams P, cons
   const Coefs<R>& C = coefs<R>(P);
   const long long i = (long long)blockIdx.x * BLOCK + t;
   if (i >= P.N) return;
-  const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
+  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  if (x >= P.nx) return;
   const R* __restrict__ psi = pl.p[P_PSI];
   R c[3][3];
   gather9(psi, P, x, y, c);
@@ -173,7 +174,8 @@ __global__ void __launch_bounds__(2 * BLOCK)
   const bool heat = t >= BLOCK;
   const long long i = (long long)blockIdx.x * BLOCK + (t - (heat ? BLOCK : 0));
   if (i >= P.N) return;
-  const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
+  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  if (x >= P.nx) return;
   const R vx = pl.p[P_VX][i], vy = pl.p[P_VY][i];
   if (!heat) {
     R f[9];
@@ -236,7 +238,7 @@ struct Around {
 };
 __device__ __forceinline__ Around around(const DevParams& P, int x, int y, bool interior) {
   Around n;
-  const unsigned nx = (unsigned)P.nx;
+  const unsigned nx = (unsigned)P.pitch;
   n.row[1] = (unsigned)y * nx;
   n.col[1] = (unsigned)x;
   if (interior) {
@@ -247,7 +249,7 @@ __device__ __forceinline__ Around around(const DevParams& P, int x, int y, bool 
   } else {
     n.row[0] = y == 0 ? (P.yper ? (unsigned)(P.ny - 1) * nx : n.row[1]) : n.row[1] - nx;
     n.row[2] = y == P.ny - 1 ? (P.yper ? 0u : n.row[1]) : n.row[1] + nx;
-    n.col[0] = x == 0 ? nx - 1u : n.col[1] - 1u;
+    n.col[0] = x == 0 ? (unsigned)P.nx - 1u : n.col[1] - 1u;
     n.col[2] = x == P.nx - 1 ? 0u : n.col[1] + 1u;
   }
   return n;
@@ -432,7 +434,8 @@ __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_i
                                                 PopBuf<S> f, PopBuf<S> g, DevParams P) {
   const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
-  const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
+  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  if (x >= P.nx) return;
   double fv[9], gv[9];
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
@@ -462,8 +465,8 @@ __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_i
     gv[a] = ge[a];
   }
   // FP16 storage: deviations from the rest equilibrium of this slot's own node
-  pop_store<S, double>(f, P.N, i, fv, rho_in[i], P.cd.wf);
-  pop_store<S, double>(g, P.N, i, gv, T_in[i], P.cd.wg);
+  pop_store<S, double>(f, P.N, i, fv, rho_in[(long long)y * P.nx + x], P.cd.wf);
+  pop_store<S, double>(g, P.N, i, gv, T_in[(long long)y * P.nx + x], P.cd.wg);
 }
 
 // Sums of rho and T over the current (post-boundary) state into per-block partials. Bound by the FP64 pipe
@@ -479,7 +482,8 @@ __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, 
   for (int k = 0; k < K; ++k) {
     const long long i = ((long long)blockIdx.x * K + k) * BLOCK + tid;
     if (i >= P.N) break;
-    const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
+    const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+    if (x >= P.nx) continue;
     double f[9], g[9];
     pull_closed<S, double>(fsrc, gsrc, P, x, y, f, g);
     r += f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
@@ -491,21 +495,23 @@ __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, 
   if (tid == 0) partials[stride + blockIdx.x] = st;
 }
 
-// Post-boundary populations of the current state as FP64 [9][N] (which = 0: f, 1: g).
+// Post-boundary populations of the current state as FP64 [9][ny][nx] (which = 0: f, 1: g).
 template <class S>
 __global__ void __launch_bounds__(BLOCK) k_export_pops(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P, int which,
                                                        int only, double* __restrict__ out) {
   const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
-  const int y = (int)(i / P.nx), x = (int)(i - (long long)y * P.nx);
+  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  if (x >= P.nx) return;
   double f[9], g[9];
   pull_closed<S, double>(fsrc, gsrc, P, x, y, f, g);
-  if (only >= 0) {  // one population plane into out[N]
-    out[i] = which ? g[only] : f[only];
+  const long long o = (long long)y * P.nx + x;  // outputs have no padding
+  if (only >= 0) {  // one population plane into out[ny][nx]
+    out[o] = which ? g[only] : f[only];
     return;
   }
 #pragma unroll
-  for (int a = 0; a < 9; ++a) out[(long long)a * P.N + i] = which ? g[a] : f[a];
+  for (int a = 0; a < 9; ++a) out[(long long)a * P.nx * P.ny + o] = which ? g[a] : f[a];
 }
 
 // Copy planes rho, vx, vy, T to FP64 outputs (any may be null).
@@ -514,10 +520,13 @@ __global__ void __launch_bounds__(BLOCK) k_export_fields(Planes<R> pl, DevParams
                                                          double* T) {
   const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
-  if (rho) rho[i] = (double)pl.p[P_RHO][i];
-  if (ux) ux[i] = (double)pl.p[P_VX][i];
-  if (uy) uy[i] = (double)pl.p[P_VY][i];
-  if (T) T[i] = (double)pl.p[P_T][i];
+  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  if (x >= P.nx) return;
+  const long long o = (long long)y * P.nx + x;  // outputs have no padding
+  if (rho) rho[o] = (double)pl.p[P_RHO][i];
+  if (ux) ux[o] = (double)pl.p[P_VX][i];
+  if (uy) uy[o] = (double)pl.p[P_VY][i];
+  if (T) T[o] = (double)pl.p[P_T][i];
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -552,7 +561,7 @@ static cudaError_t step_impl(const SplitBuffers& b, const DevParams& P, int cur,
                                             pl, (R*)b.phi_prev, P, step == 0);
   if (ev) cudaEventRecord(ev[3], st);
   if (P.buoyancy == 1) {
-    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars, nullptr);
+    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / node_count(P), b.scalars, nullptr);
     if (ev) cudaEventRecord(ev[4], st);
   }
   return cudaGetLastError();
@@ -585,7 +594,7 @@ static cudaError_t step_wide(const SplitBuffers& b, const DevParams& P, int cur,
     collide(std::integral_constant<int, 16>(), std::integral_constant<int, 8>());
   if (ev) cudaEventRecord(ev[2], st);
   if (P.buoyancy == 1) {
-    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / (double)P.N, b.scalars, nullptr);
+    launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, (int)nb, 0, 1.0 / node_count(P), b.scalars, nullptr);
     if (ev) cudaEventRecord(ev[3], st);
   }
   return cudaGetLastError();
@@ -635,7 +644,7 @@ static cudaError_t init_impl(const SplitBuffers& b, const DevParams& P, const do
   launch_pdl(k_init<S>, nb, BLOCK, 0, st, rho, T, ux, uy, fbuf<S>(b, 0), gbuf<S>(b, 0), P);
   // rho_ave of the initial (post-boundary) state
   const int ns = launch_sums<S>(b, P, 0, st);
-  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, ns, 0, 1.0 / (double)P.N, b.scalars, nullptr);
+  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, ns, 0, 1.0 / node_count(P), b.scalars, nullptr);
   return cudaGetLastError();
 }
 
@@ -696,7 +705,7 @@ cudaError_t split_export_pops(const SplitBuffers& b, const DevParams& P, int pre
 }
 
 void fused_finish(const SplitBuffers& b, const DevParams& P, int n, cudaStream_t st) {
-  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, n, 0, 1.0 / (double)P.N, b.scalars, nullptr);
+  launch_pdl(k_finish, 1, FINISH, 0, st, b.partials, n, 0, 1.0 / node_count(P), b.scalars, nullptr);
 }
 
 int split_nplanes() { return NPLANES; }

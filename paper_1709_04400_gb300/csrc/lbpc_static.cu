@@ -37,7 +37,7 @@ cudaError_t scratch_on_current_device(double** out) {
 }  // namespace
 
 namespace lbpc {
-DevParams make_dev_params_public(const lbpc_params* p);
+DevParams make_dev_params_public(const lbpc_params* p, int pitch);
 }
 
 LBPC_API lbpc_status lbpc_step_static(const lbpc_params* p, const void* f_in, const void* g_in, void* f_out,
@@ -57,7 +57,7 @@ LBPC_API lbpc_status lbpc_step_static(const lbpc_params* p, const void* f_in, co
   if (scratch_on_current_device(&s) != cudaSuccess) return LBPC_ECUDA;
   cudaStream_t st = (cudaStream_t)stream;
 
-  const lbpc::DevParams dp = lbpc::make_dev_params_public(p);
+  const lbpc::DevParams dp = lbpc::make_dev_params_public(p, p->nx);  // the caller's buffers have no padding
   lbpc::SplitBuffers b{};
   b.f[0] = (void*)f_in;
   b.g[0] = (void*)g_in;

@@ -33,9 +33,9 @@ __device__ __forceinline__ int wrap_any(int x, int n) {
 
 // Post-stream populations of an interior node (no wrap, no closure): src[a][i - e_a].
 template <class S, class R, class IX = long long>
-__device__ __forceinline__ void pull_interior(const PopBuf<S>& src, const R* w, IX N, int nx, IX i, R v[9]) {
+__device__ __forceinline__ void pull_interior(const PopBuf<S>& src, const R* w, IX N, int pitch, IX i, R v[9]) {
 #pragma unroll
-  for (int a = 0; a < 9; ++a) v[a] = pop_load<S, R, IX>(src, N, a, i - (IX)EY(a) * nx - EX(a), w);
+  for (int a = 0; a < 9; ++a) v[a] = pop_load<S, R, IX>(src, N, a, i - (IX)EY(a) * pitch - EX(a), w);
 }
 
 // Domain row for region row offset: wraps when y is periodic, else clamps to the edge row.
@@ -121,7 +121,36 @@ template <class R, int TX, int TY> struct FusedSmem {
   R rho[TY + 4][TX + 4], T[TY + 4][TX + 4], psi[TY + 4][TX + 4], jx[TY + 4][TX + 4], jy[TY + 4][TX + 4];
   R vx[TY + 2][TX + 2], vy[TY + 2][TX + 2];
   double red[TX * TY / 32];
+  R ref;          // the domain mean of the step before
+  int last;       // this block's partial sum is the step's last
 };
+
+// The domain mean of rho by the last block of a step to write its partial sum (n of them), instead of a kernel of its
+// own after the step (2.3 us of a 150 x 300 step's 9.4). Every block has read the mean of the step before by then: it
+// does so before the block barrier that its partial sum passes.
+struct MeanOf {
+  double* out;         // rho_ave
+  unsigned* arrived;   // partial sums written; wraps to zero
+  unsigned n;
+  double scale;        // 1 / nodes
+};
+template <int NTH>
+__device__ __forceinline__ void finish_mean(int t, const MeanOf& m, double* partials, int& s_last, double* s_red) {
+  if (t == 0) {
+    __threadfence();
+    s_last = atomicInc(m.arrived, m.n - 1) == m.n - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double s[4] = {0.0, 0.0, 0.0, 0.0};
+  for (unsigned j = t; j < m.n; j += 4 * NTH)
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      if (j + k * NTH < m.n) s[k] += __ldcg(partials + j + k * NTH);
+  const double sum = block_sum<NTH>((s[0] + s[1]) + (s[2] + s[3]), s_red);
+  if (t == 0) *m.out = sum * m.scale;
+}
 
 // Resident CTAs per SM requested of the compiler for the tile kernels with 4- and 2-byte storage:
 // 1024 threads per SM with one node per thread (64 registers), 512 with two (128 registers, which
@@ -142,6 +171,7 @@ template <class S, int NTH, int NPT> __host__ __device__ constexpr int fused_min
 // t: the thread's index in the block (pdl_wait's in kernels launched with launch_pdl).
 // after_stage1: called by every thread once the tile has finished reading its staged populations (after
 // the block barrier that closes stage 1); the persistent TMA kernel starts the next tile's copy there.
+// mean: null, or where the step's domain mean of rho goes: the block whose partial sum is the last one takes it.
 struct NoStageHook {
   __device__ __forceinline__ void operator()() const {}
 };
@@ -155,7 +185,8 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
                                            long long* __restrict__ status, FusedSmem<R, TX, TY>& sm, int x0, int y0,
                                            int pslot, const TmaTile<S> staged = TmaTile<S>{nullptr},
                                            const long long* step_at = nullptr,
-                                           AfterStage1 after_stage1 = AfterStage1{}) {
+                                           AfterStage1 after_stage1 = AfterStage1{},
+                                           const MeanOf* mean = nullptr) {
   constexpr bool INTERIOR = MODE != 0;
   using IX = typename std::conditional<IDX32, int, long long>::type;
   constexpr int RX = TX + 4, RY = TY + 4;  // stage-1 region (tile + 2)
@@ -175,15 +206,17 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
 
   const Coefs<R>& C = coefs<R>(P);
 
-  // The buoyancy's reference density. With the parameters in PT's compact form (the batch) it is read here, before
-  // the pulls, whose latency hides it (in stage 2 the batched step is 8 % slower); with DevParams in stage 2 (here
-  // the single-instance step of a 1023 x 1025 grid is 3 % slower).
+  // The buoyancy's reference density. Where the block may itself write the next step's mean (`mean`), thread 0 reads
+  // this step's before the first block barrier; with the batch's parameters (PT) every thread reads it here, where the
+  // pulls hide its latency (in stage 2 the batched step is 8 % slower); otherwise in stage 2, which leaves the
+  // registers of stage 1 alone (the persistent 4096^2 step takes 436 us with the read here, 414 without).
   constexpr bool kEarlyRef = !std::is_same<PT, DevParams>::value;
   auto read_ref = [&]() {
     return P.buoyancy == 1 ? R(load_after_wait(rho_ave)) : (P.buoyancy == 2 ? C.rho_bc_hi : R(0));
   };
   R rho_ref = R(0);
   if constexpr (kEarlyRef) rho_ref = read_ref();
+  if (mean && P.buoyancy == 1 && t == 0) sm.ref = R(load_after_wait(rho_ave));
 
   // ---- stage 1a: own nodes (kept in registers) ----
   R f[NPT][9], g[NPT][9];
@@ -198,18 +231,18 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     const int gx = x0 + tx, gy = y0 + ty;
     active[k] = INTERIOR || (gx < P.nx && gy < P.ny);
     if constexpr (IDX32)
-      pp[k] = (active[k] && P.model == 0 && !first) ? __ldg(phi_prev + ((IX)gy * P.nx + gx)) : R(0);
+      pp[k] = (active[k] && P.model == 0 && !first) ? __ldg(phi_prev + ((IX)gy * P.pitch + gx)) : R(0);
     else
-      pp[k] = (active[k] && P.model == 0 && !first) ? phi_prev[(long long)gy * P.nx + gx] : R(0);
+      pp[k] = (active[k] && P.model == 0 && !first) ? phi_prev[(long long)gy * P.pitch + gx] : R(0);
     const int mx = wrap_any(gx, P.nx);
     my[k] = row_of(P, gy);
     if (MODE == 2) {
       pull_staged<S, R, TX, TY>(staged, 0, C.wf, tx + 2, ty + 2, f[k]);
       pull_staged<S, R, TX, TY>(staged, 1, C.wg, tx + 2, ty + 2, g[k]);
     } else if (INTERIOR) {
-      const IX io = (IX)gy * P.nx + gx;
-      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.nx, io, f[k]);
-      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, P.nx, io, g[k]);
+      const IX io = (IX)gy * P.pitch + gx;
+      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.pitch, io, f[k]);
+      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, P.pitch, io, g[k]);
     } else {
       pull_closed<S, R, IX>(fsrc, gsrc, P, mx, my[k], f[k], g[k]);
     }
@@ -257,9 +290,9 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
       pull_staged<S, R, TX, TY>(staged, 0, C.wf, hx, hy, fr);
       pull_staged<S, R, TX, TY>(staged, 1, C.wg, hx, hy, gr);
     } else if (INTERIOR) {
-      const IX io = (IX)(y0 + hy - 2) * P.nx + (x0 + hx - 2);
-      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.nx, io, fr);
-      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, P.nx, io, gr);
+      const IX io = (IX)(y0 + hy - 2) * P.pitch + (x0 + hx - 2);
+      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.pitch, io, fr);
+      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, P.pitch, io, gr);
     } else {
       const int x = wrap_any(x0 + hx - 2, P.nx), y = row_of(P, y0 + hy - 2);
       pull_closed<S, R, IX>(fsrc, gsrc, P, x, y, fr, gr);
@@ -288,13 +321,17 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     for (int k = 0; k < NPT; ++k) own += active[k] ? (double)rho[k] : 0.0;
     const double sr = block_sum<NTH>(own, s_red);
     if (t == 0) partials[pslot] = sr;
+    if (mean) finish_mean<NTH>(t, *mean, partials, sm.last, s_red);
   } else {
     __syncthreads();
   }
   after_stage1();
 
   // ---- stage 2: F and v on tile + 1 ----
-  if constexpr (!kEarlyRef) rho_ref = read_ref();
+  if (mean)
+    rho_ref = P.buoyancy == 1 ? sm.ref : (P.buoyancy == 2 ? C.rho_bc_hi : R(0));
+  else if constexpr (!kEarlyRef)
+    rho_ref = read_ref();
   // F at stage-2 position (vx_, vy_) of the domain node (x, y); the stencil rows come from the clamped
   // node's own region rows so a ghost position reproduces the edge node exactly.
   auto force_at = [&](int hx, int hy, int y, R& Fx, R& Fy, R& Q, R& vx, R& vy) {
@@ -392,7 +429,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
                     (s_rho[hy + 1][hx + 1] + s_rho[hy + 1][hx - 1] - s_rho[hy - 1][hx - 1] - s_rho[hy - 1][hx + 1]) * R(1.0 / 12.0);
       div_lam_gradT = rcv * C.chi * lapT + C.cV_chi * (grx * gTx + gry * gTy);
     }
-    const IX i = (IX)gy * P.nx + gx;
+    const IX i = (IX)gy * P.pitch + gx;
     const R compress = Tk * (R(1) - dpdT[k] * inv_rcv) * divv;
     R phi, S0, tau_inv = R(0);
     if (P.model == 2) {  // Gong-Cheng: Eq. 13 source, local tau_g (Sec. IV A)
