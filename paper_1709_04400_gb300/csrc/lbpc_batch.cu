@@ -12,6 +12,7 @@
 #include <algorithm>
 #include <map>
 #include <memory>
+#include <type_traits>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -88,7 +89,8 @@ struct HostInst {
   lbpc::DevParams dp{};
   long long N = 0;  // nodes
   size_t off = 0, bytes = 0;  // arena block of the instance
-  size_t f[2], g[2], rf[2], rg[2], wall[2], phi, partials, scalars;
+  size_t f[2], g[2], rf[2], rg[2], wall[2], phi, partials, scalars, maps;
+  bool staged = false;        // the device holds tensor maps of both buffers
   size_t npartials = 0;
   long long step = 0;
   int cur = 0;
@@ -120,6 +122,7 @@ size_t layout_instance(const lbpc_params* p, HostInst* h) {
   h->npartials = std::max(lbpc::fused_max_tiles(p->nx, p->ny), 2 * (size_t)((N + lbpc::split_block() - 1) / lbpc::split_block()));
   h->partials = off; off += a256(h->npartials * sizeof(double));
   h->scalars = off; off += a256(8 * sizeof(double));
+  h->maps = off; off += sb <= 4 ? 2 * sizeof(lbpc::TmaMaps) : 0;
   return off;
 }
 
@@ -294,6 +297,12 @@ lbpc::SplitBuffers split_view(lbpc_batch* b, const HostInst& h, char* scratch) {
   return s;
 }
 
+// Ticket words of launch k of a step (they follow the meta block).
+size_t ticket_bytes(int max_inst) { return ((size_t)max_inst / lbpc::kSegSmall + 1) * 2 * sizeof(unsigned long long); }
+unsigned long long* tickets(lbpc_batch* b, int k) {
+  return (unsigned long long*)(b->base + b->meta_off + a256(sizeof(lbpc::BatchMeta))) + 2 * k;
+}
+
 // One step as per-tile launches (ctas == 0): the active instances in launches of up to seg_capacity, each
 // instance reading the buffer of parity h.cur ^ rel, then the per-instance advance. Whether the step is
 // an instance's first comes from the host's count (h.step + rel), so lbpc_batch_step takes the first
@@ -313,17 +322,19 @@ template <class S> cudaError_t seg_step(lbpc_batch* b, int rel) {
       memset(Ls.get(), 0, sizeof(lbpc::SegLaunch<S, SMALL>));
       Ls->n = L->n;
       Ls->tiles = L->tiles;
+      Ls->staged = L->staged;
       for (int j = 0; j < L->n; ++j) {
         Ls->first_tile[j] = L->first_tile[j];
         Ls->in[j] = L->in[j];
       }
-      e = lbpc::batch_seg_launch(b->prec, b->variant, true, Ls.get(), launches > 0, b->stream);
+      e = lbpc::batch_seg_launch(b->prec, b->variant, true, Ls.get(), tickets(b, launches), launches > 0, b->stream);
     } else {
-      e = lbpc::batch_seg_launch(b->prec, b->variant, false, L.get(), launches > 0, b->stream);
+      e = lbpc::batch_seg_launch(b->prec, b->variant, false, L.get(), tickets(b, launches), launches > 0, b->stream);
     }
     ++launches;
     L->n = 0;
     L->tiles = 0;
+    L->staged = 0;
     return e;
   };
   for (int k = 0; k < (int)b->inst.size(); ++k) {
@@ -347,10 +358,14 @@ template <class S> cudaError_t seg_step(lbpc_batch* b, int rel) {
     r.scalars = (double*)(base + h.scalars);
     r.partials = (double*)(base + h.partials);
     r.status = (long long*)(b->base + b->status_off) + 8 * k;
+    if constexpr (!std::is_same<S, double>::value)
+      r.maps = h.staged ? (const lbpc::TmaMaps*)(base + h.maps) + c : nullptr;
     r.step = (const long long*)(b->base + b->insts_off + (size_t)k * b->inst_struct + offsetof(lbpc::BatchInst<S>, step));
     r.tiles_x = (h.dp.nx + tx - 1) / tx;
     r.first = h.step + rel == 0;
     L->tiles += r.tiles_x * ((h.dp.ny + ty - 1) / ty);
+    if (h.staged && tx == 32 && ty == 8)  // interior tiles: 3 nodes from every edge
+      L->staged += std::max(0, (h.dp.nx - 35) / 32) * std::max(0, (h.dp.ny - 11) / 8);
   }
   const cudaError_t e = flush();
   if (e != cudaSuccess) return e;
@@ -446,7 +461,7 @@ LBPC_API lbpc_status lbpc_batch_create(int32_t prec, int32_t max_instances, void
   b->bytes = bytes;
   b->inst_struct = inst_struct_bytes(prec);
   b->arena.reset(bytes);
-  const size_t fixed[3] = {sizeof(lbpc::BatchMeta), b->inst_struct * (size_t)max_instances,
+  const size_t fixed[3] = {a256(sizeof(lbpc::BatchMeta)) + ticket_bytes(max_instances), b->inst_struct * (size_t)max_instances,
                            8 * sizeof(long long) * (size_t)max_instances};
   size_t offs[3];
   for (int k = 0; k < 3; ++k)
@@ -459,7 +474,8 @@ LBPC_API lbpc_status lbpc_batch_create(int32_t prec, int32_t max_instances, void
   b->status_off = offs[2];
   {
     DevGuard g(b->device);
-    if (cudaMemsetAsync(b->base + b->status_off, 0, fixed[2], b->stream) != cudaSuccess ||
+    if (cudaMemsetAsync(b->base + b->meta_off, 0, fixed[0], b->stream) != cudaSuccess ||
+        cudaMemsetAsync(b->base + b->status_off, 0, fixed[2], b->stream) != cudaSuccess ||
         cudaMemsetAsync(b->base + b->insts_off, 0, fixed[1], b->stream) != cudaSuccess) {
       delete b;
       return LBPC_ECUDA;
@@ -523,6 +539,16 @@ LBPC_API lbpc_status lbpc_batch_add(lbpc_batch* b, const lbpc_params* p, const d
   BCU(b, lbpc::split_init(s, hi.dp, b->prec, d_rho, d_T, nullptr, nullptr, b->stream), "lbpc_batch_add init");
   hi.cur = 0;
   hi.step = 0;
+  hi.staged = false;
+  if (store_bytes(b->prec) <= 4) {
+    lbpc::TmaMaps maps[2] = {};
+    hi.staged = true;
+    for (int k = 0; k < 2; ++k)
+      hi.staged &= lbpc::fused_tma_encode(&maps[k], b->prec, 1, s.f[k], s.g[k], s.ref_f[k], s.ref_g[k], hi.dp);
+    // pageable source: the copy is staged before the call returns
+    BCU(b, cudaMemcpyAsync(b->base + hi.off + hi.maps, maps, sizeof maps, cudaMemcpyHostToDevice, b->stream),
+        "lbpc_batch_add tensor maps");
+  }
   b->dirty = true;
   lbpc_status r = rebuild(b);
   if (r != LBPC_OK) return r;

@@ -23,6 +23,9 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   if (interior)
     fused_body<1, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, mean.out, partials, status, sm,
                                      x0, y0, pslot, TmaTile<S>{nullptr}, nullptr, NoStageHook{}, &mean);
+  else if (rows_inside<TY>(P, y0))
+    fused_body<4, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, mean.out, partials, status, sm,
+                                     x0, y0, pslot, TmaTile<S>{nullptr}, nullptr, NoStageHook{}, &mean);
   else
     fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, mean.out, partials, status, sm,
                                      x0, y0, pslot, TmaTile<S>{nullptr}, nullptr, NoStageHook{}, &mean);
@@ -49,8 +52,12 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
   }
   const int t = pdl_wait<TX * TY / NPT>();
   if (!interior) {
-    fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
-                                     x0, y0, pslot);
+    if (rows_inside<TY>(P, y0))
+      fused_body<4, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+                                       x0, y0, pslot);
+    else
+      fused_body<0, S, R, TX, TY, NPT>(t, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+                                       x0, y0, pslot);
     return;
   }
   if (threadIdx.x == 0) {
@@ -85,21 +92,6 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
 // Bound by HBM in FP32 (4096^2: 413 us, 91 % of the measured copy bandwidth at 152 B per node) and by issue in
 // FP16. What the walk itself costs counts: with each ticket awaited where the next copy starts, one tensor copy
 // per population plane, and tile origins divided out by every thread, 4096^2 took 469 us (FP16 528, now 470).
-template <class S, int TX, int TY>
-__device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar, const TmaMaps& maps, int x0, int y0) {
-  using B = TmaBox<S, TX, TY>;
-  // the box was last read through the generic proxy (stage 1, before a block barrier); order those
-  // reads before the copy engine's writes
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  mbar_expect_tx(bar, (unsigned)(18 * B::BX * B::BY * sizeof(S) + (B::HALF ? 2 * B::REFX * B::BY * 4 : 0)));
-  tma_load_3d(dyn, &maps.f, x0 - B::XOFF, y0 - 3, 0, bar);
-  tma_load_3d(dyn + B::SET, &maps.g, x0 - B::XOFF, y0 - 3, 0, bar);
-  if (B::HALF) {
-    tma_load_2d(dyn + 2 * B::SET, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
-    tma_load_2d(dyn + 2 * B::SET + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
-  }
-}
-
 template <class S, class R, int TX, int TY, int NPT>
 __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NPT, NPT>())
     k_fused_tma_loop(PopBuf<S> fsrc, PopBuf<S> gsrc, PopBuf<S> fdst, PopBuf<S> gdst, R* __restrict__ phi_prev,
@@ -160,8 +152,12 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
                                        tile.x, tile.y, tile.index, TmaTile<S>{dyn}, nullptr, start_next);
     } else {
       start_next();
-      fused_body<0, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
-                                       tile.x, tile.y, tile.index);
+      if (is_half_t<S>::value && rows_inside<TY>(P, tile.y))  // in FP32 a third body costs every tile 4 %
+        fused_body<4, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+                                         tile.x, tile.y, tile.index);
+      else
+        fused_body<0, S, R, TX, TY, NPT>(threadIdx.x, fsrc, gsrc, fdst, gdst, phi_prev, P, step, first, rho_ave, partials, status, sm,
+                                         tile.x, tile.y, tile.index);
     }
     if (threadIdx.x == 0) {
       s_tile[it ^ 1] = s_next[it];

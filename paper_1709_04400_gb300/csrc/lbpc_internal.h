@@ -157,7 +157,11 @@ cudaError_t batch_step_launch(int prec, int variant, int ctas, const BatchMeta* 
 // such launches over the active instances (up to seg_capacity each), then the per-instance advance.
 template <class S> struct ArithOf { using type = float; };  // arithmetic of a storage type in a batch
 template <> struct ArithOf<double> { using type = double; };
-template <class S> struct alignas(16) SegInst {
+template <class S> struct SegMaps {
+  const TmaMaps* maps;       // tensor maps of the source buffers (device memory), or null
+};
+template <> struct SegMaps<double> {};  // binary64 batches are not staged
+template <class S> struct alignas(16) SegInst : SegMaps<S> {
   DevParamsOf<typename ArithOf<S>::type> P;  // header and the one coefficient set the kernel reads
   PopBuf<S> fs, gs, fd, gd;  // this launch's source and destination populations
   void* phi_prev;            // arithmetic type
@@ -168,7 +172,7 @@ template <class S> struct alignas(16) SegInst {
   int tiles_x;               // tiles per row
   int first;                 // the instance's first step (its source term starts from phi itself)
 };
-constexpr size_t kSegParamBytes = 32512;  // within the 32,764 bytes of kernel parameters
+constexpr size_t kSegParamBytes = 32720;  // within the 32,764 bytes of kernel parameters
 template <class S> constexpr int seg_capacity() {
   return (int)((kSegParamBytes - 32) / (sizeof(SegInst<S>) + sizeof(int))) & ~3;
 }
@@ -177,8 +181,9 @@ template <class S> constexpr int seg_capacity() {
 constexpr int kSegSmall = 16;
 template <class S, int CAP> struct SegLaunch {
   int n;      // instances of this launch
-  int tiles;  // its CTAs
-  int pad_[2];
+  int tiles;  // its tiles
+  int staged; // those of them that tensor copies can stage
+  int pad_;
   int first_tile[CAP];  // each instance's first CTA, ascending: kept together so that the search of a
                         // CTA's instance reads a few cache lines
   SegInst<S> in[CAP];
@@ -186,10 +191,12 @@ template <class S, int CAP> struct SegLaunch {
 static_assert(sizeof(SegLaunch<double, seg_capacity<double>()>) <= kSegParamBytes &&
                   sizeof(SegLaunch<float, seg_capacity<float>()>) <= kSegParamBytes,
               "per-tile launch parameters");
+// tickets: two zeroed words of this launch's own in device memory, left zero.
 // Enqueue one per-tile launch over the instances of L, a host SegLaunch<S, CAP> of the batch's storage
 // type with CAP = kSegSmall (small) or seg_capacity<S>(). pdl: the launch may begin while the previous
 // kernel on st drains (its instances are others).
-cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, bool pdl, cudaStream_t st);
+cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, bool pdl,
+                             cudaStream_t st);
 // Enqueue the per-instance advance of a step (rho_ave, buffer parity, step count).
 cudaError_t batch_advance_launch(int prec, void* d_insts, int ninst, cudaStream_t st);
 // Largest resident CTAs per SM of the step kernel for (prec, variant).

@@ -38,6 +38,28 @@ __device__ __forceinline__ void pull_interior(const PopBuf<S>& src, const R* w, 
   for (int a = 0; a < 9; ++a) v[a] = pop_load<S, R, IX>(src, N, a, i - (IX)EY(a) * pitch - EX(a), w);
 }
 
+// Populations of a node whose source rows all lie inside the domain, in a tile that touches an x edge: the columns
+// wrap, and of the closures only a held column's applies.
+template <class S, class R, class IX, class PT>
+__device__ __forceinline__ void pull_columns(const PopBuf<S>& fsrc, const PopBuf<S>& gsrc, const PT& P, int x, int y, R f[9],
+                                             R g[9]) {
+  const Coefs<R>& C = coefs<R>(P);
+  const IX row = (IX)y * P.pitch;
+  const IX at[3] = {row + (x == P.nx - 1 ? 0 : x + 1), row + x, row + (x == 0 ? P.nx - 1 : x - 1)};  // e_x = -1, 0, 1
+#pragma unroll
+  for (int a = 0; a < 9; ++a) {
+    const IX i = at[EX(a) + 1] - (IX)EY(a) * P.pitch;
+    f[a] = pop_load<S, R, IX>(fsrc, (IX)P.N, a, i, C.wf);
+    g[a] = pop_load<S, R, IX>(gsrc, (IX)P.N, a, i, C.wg);
+  }
+  if ((x == 0 && P.tbc[0]) || (x == P.nx - 1 && P.tbc[1])) heat_closure(g, P, x, y);
+}
+
+// Whether a tile's rows, with its ring and their pull sources, lie inside the domain.
+template <int TY, class PT> __device__ __forceinline__ bool rows_inside(const PT& P, int y0) {
+  return y0 >= 3 && y0 + TY + 3 <= P.ny;
+}
+
 // Domain row for region row offset: wraps when y is periodic, else clamps to the edge row.
 template <class PT> __device__ __forceinline__ int row_of(const PT& P, int y) {
   if (P.yper) return wrap_any(y, P.ny);
@@ -93,6 +115,22 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
           smem_u32(dst)),
       "l"(tm), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
+}
+
+// Start the copy of a tile's populations (and FP16 reference planes) into its box, by one thread.
+template <class S, int TX, int TY>
+__device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar, const TmaMaps& maps, int x0, int y0) {
+  using B = TmaBox<S, TX, TY>;
+  // the box was last read through the generic proxy (stage 1, before a block barrier); order those
+  // reads before the copy engine's writes
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  mbar_expect_tx(bar, (unsigned)(18 * B::BX * B::BY * sizeof(S) + (B::HALF ? 2 * B::REFX * B::BY * 4 : 0)));
+  tma_load_3d(dyn, &maps.f, x0 - B::XOFF, y0 - 3, 0, bar);
+  tma_load_3d(dyn + B::SET, &maps.g, x0 - B::XOFF, y0 - 3, 0, bar);
+  if (B::HALF) {
+    tma_load_2d(dyn + 2 * B::SET, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
+    tma_load_2d(dyn + 2 * B::SET + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
+  }
 }
 
 // Shared-memory view of a staged tile.
@@ -161,6 +199,7 @@ template <class S, int NTH, int NPT> __host__ __device__ constexpr int fused_min
 
 // INTERIOR: the tile, its 2-ring and their pull sources lie inside the domain away from every edge,
 // so no index wraps, no boundary closure applies and no ghost row exists (a per-CTA, uniform choice).
+// MODE: 0 general, 1 interior, 2 interior from a staged box, 4 a tile at an x edge whose rows are all inside.
 // NPT nodes per thread: a CTA of TX * TY / NPT threads; thread t owns tile nodes t + k * (TX * TY / NPT),
 // k < NPT, and keeps their populations in registers from stage 1 to stage 3. With NPT = 2 the ring
 // stages keep more of the (fewer) threads busy and every thread carries two independent chains.
@@ -187,7 +226,8 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
                                            const long long* step_at = nullptr,
                                            AfterStage1 after_stage1 = AfterStage1{},
                                            const MeanOf* mean = nullptr) {
-  constexpr bool INTERIOR = MODE != 0;
+  constexpr bool INTERIOR = MODE == 1 || MODE == 2;
+  constexpr bool ROWS = MODE != 0;  // the rows of the tile, its ring and their sources lie inside
   using IX = typename std::conditional<IDX32, int, long long>::type;
   constexpr int RX = TX + 4, RY = TY + 4;  // stage-1 region (tile + 2)
   constexpr int VX = TX + 2, VY = TY + 2;  // stage-2 region (tile + 1)
@@ -229,16 +269,18 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     const int n = t + k * NTH;
     const int tx = n % TX, ty = n / TX;
     const int gx = x0 + tx, gy = y0 + ty;
-    active[k] = INTERIOR || (gx < P.nx && gy < P.ny);
+    active[k] = INTERIOR || (gx < P.nx && (ROWS || gy < P.ny));
     if constexpr (IDX32)
       pp[k] = (active[k] && P.model == 0 && !first) ? __ldg(phi_prev + ((IX)gy * P.pitch + gx)) : R(0);
     else
       pp[k] = (active[k] && P.model == 0 && !first) ? phi_prev[(long long)gy * P.pitch + gx] : R(0);
     const int mx = wrap_any(gx, P.nx);
-    my[k] = row_of(P, gy);
+    my[k] = ROWS ? gy : row_of(P, gy);
     if (MODE == 2) {
       pull_staged<S, R, TX, TY>(staged, 0, C.wf, tx + 2, ty + 2, f[k]);
       pull_staged<S, R, TX, TY>(staged, 1, C.wg, tx + 2, ty + 2, g[k]);
+    } else if (MODE == 4) {
+      pull_columns<S, R, IX>(fsrc, gsrc, P, mx, gy, f[k], g[k]);
     } else if (INTERIOR) {
       const IX io = (IX)gy * P.pitch + gx;
       pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.pitch, io, f[k]);
@@ -289,6 +331,8 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     if (MODE == 2) {
       pull_staged<S, R, TX, TY>(staged, 0, C.wf, hx, hy, fr);
       pull_staged<S, R, TX, TY>(staged, 1, C.wg, hx, hy, gr);
+    } else if (MODE == 4) {
+      pull_columns<S, R, IX>(fsrc, gsrc, P, wrap_any(x0 + hx - 2, P.nx), y0 + hy - 2, fr, gr);
     } else if (INTERIOR) {
       const IX io = (IX)(y0 + hy - 2) * P.pitch + (x0 + hx - 2);
       pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.pitch, io, fr);
@@ -345,7 +389,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     Fx = -C.G * pc * sx;
     Fy = -C.G * pc * sy;
     // F_ads = -G_w psi(x) sum_a w_a psi(x) s(x+e_a) e_a, on the y- wall only (a y+ wall is a neutral lid)
-    if (!INTERIOR && !P.yper && y == 0 && P.ybc_lo == BC_WALL) Fy += C.G_wall * 0.5f * pc * pc;
+    if (!ROWS && !P.yper && y == 0 && P.ybc_lo == BC_WALL) Fy += C.G_wall * 0.5f * pc * pc;
     const R rr = s_rho[hy][hx];
     if (P.buoyancy) {
       const R d = rr - rho_ref;
@@ -359,7 +403,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
   };
   // region row (stage-1 coordinates) holding the clamped domain row of stage-1 row hy
   auto clamp_hy = [&](int hy) {
-    if (INTERIOR || P.yper) return hy;
+    if (ROWS || P.yper) return hy;
     const int y = y0 + hy - 2;
     if (y < 0) return hy - y;                 // row of y = 0
     if (y >= P.ny) return hy - (y - (P.ny - 1));  // row of y = ny - 1
@@ -388,7 +432,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
       hx = (q % 2) ? TX + 1 : 0;
     }
     const int y1 = clamp_hy(hy + 1);
-    const int ydom = row_of(P, y0 + hy - 1);
+    const int ydom = ROWS ? y0 + hy - 1 : row_of(P, y0 + hy - 1);
     R a, b, c, vxr, vyr;
     force_at(hx + 1, y1, ydom, a, b, c, vxr, vyr);
     s_vx[hy][hx] = vxr;
@@ -457,7 +501,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
       pop_store<S, R>(fdst, P.N, i, f[k], rho[k], C.wf);
       pop_store<S, R>(gdst, P.N, i, g[k], Tk + S0, C.wg);
     }
-    if (!INTERIOR) wall_force_store(fdst.wall, P, gx, gy, Fx[k], Fy[k]);
+    if (!ROWS) wall_force_store(fdst.wall, P, gx, gy, Fx[k], Fy[k]);
   }
 }
 
