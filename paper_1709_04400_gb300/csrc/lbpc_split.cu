@@ -33,6 +33,15 @@ template <class R> struct Planes {
 
 __device__ __forceinline__ long long node_index(const DevParams& P, int x, int y) { return (long long)y * P.pitch + x; }
 
+// Node i of the padded rows (i < 2^32, so the division is a 32-bit one).
+struct Node {
+  int x, y;
+};
+__device__ __forceinline__ Node node_at(const DevParams& P, long long i) {
+  const unsigned y = (unsigned)i / (unsigned)P.pitch;
+  return Node{(int)((unsigned)i - y * (unsigned)P.pitch), (int)y};
+}
+
 // Neighbour row for a stencil: wraps when y is periodic, else clamps to the edge row (ghost rows
 // copy the edge row). out_lo/out_hi report a ghost beyond the lower / upper edge.
 __device__ __forceinline__ int nb_row(const DevParams& P, int y, int dy, bool& ghost_lo, bool& ghost_hi) {
@@ -83,10 +92,20 @@ __global__ void __launch_bounds__(BLOCK) k_macro(PopBuf<S> fsrc, PopBuf<S> gsrc,
   const int t = pdl_wait<BLOCK>();
   const long long i = (long long)blockIdx.x * BLOCK + t;
   double rho_d = 0.0;
-  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  const auto [x, y] = node_at(P, i);
   if (i < P.N && x < P.nx) {
     R f[9], g[9];
-    pull_closed<S, R>(fsrc, gsrc, P, x, y, f, g);
+    if (sizeof(R) == 8 && x > 0 && x < P.nx - 1 && y > 0 && y < P.ny - 1) {
+      const S *pf = fsrc.p + i, *pg = gsrc.p + i;  // no wrap, no closure
+#pragma unroll
+      for (int a = 0; a < 9; ++a) {
+        const long long o = (long long)a * P.N - (long long)EY(a) * P.pitch - EX(a);
+        f[a] = R(ldgv(pf + o));
+        g[a] = R(ldgv(pg + o));
+      }
+    } else {
+      pull_closed<S, R>(fsrc, gsrc, P, x, y, f, g);
+    }
     R rho, jx, jy, Tlo, dpdT, inv_rho, psi2;
     const R T = heat_of(g, Tlo);
     if constexpr (sizeof(R) == 4) {
@@ -131,7 +150,7 @@ __global__ void __launch_bounds__(BLOCK) k_force(Planes<R> pl, DevParams P, cons
   const Coefs<R>& C = coefs<R>(P);
   const long long i = (long long)blockIdx.x * BLOCK + t;
   if (i >= P.N) return;
-  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  const auto [x, y] = node_at(P, i);
   if (x >= P.nx) return;
   const R* __restrict__ psi = pl.p[P_PSI];
   R c[3][3];
@@ -174,7 +193,7 @@ __global__ void __launch_bounds__(2 * BLOCK)
   const bool heat = t >= BLOCK;
   const long long i = (long long)blockIdx.x * BLOCK + (t - (heat ? BLOCK : 0));
   if (i >= P.N) return;
-  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  const auto [x, y] = node_at(P, i);
   if (x >= P.nx) return;
   const R vx = pl.p[P_VX][i], vy = pl.p[P_VY][i];
   if (!heat) {
@@ -296,6 +315,31 @@ __global__ void __launch_bounds__(2 * CX* CY)
     hy = 1 + (q - 2 * (CX + 2)) / 2;
   }
   R Fx = R(0), Fy = R(0), Q = R(0), vx = R(0), vy = R(0), rho = R(0), jx = R(0), jy = R(0);
+  // What the node's own role reads besides, asked for before the force so that its latency is hidden: the heat role's
+  // values (double-word 2048^2 442 -> 430 us), and in binary64 the flow role's moments too; their 12 double-word
+  // registers cost more there than they hide (459 us).
+  constexpr bool kFlowFirst = !is_dw_t<S>::value;
+  const int tx = q % CX, ty = q / CX;
+  const bool active = x0 + tx < P.nx && y0 + ty < P.ny;
+  const bool unit = P.model == 0 && P.heat_unit_rates;
+  R m[6], n4 = R(0), n6 = R(0), pp = R(0), dpdT = R(0), inv_rho_own = R(0);
+  auto pre_flow = [&]() {
+    const S* pf = fdst.p + (size_t)(unsigned)(y0 + ty) * (unsigned)P.pitch + (unsigned)(x0 + tx);
+#pragma unroll
+    for (int a = 0; a < 6; ++a) m[a] = pf[(size_t)a * P.N];
+  };
+  auto pre_heat = [&]() {
+    const size_t i = (size_t)(unsigned)(y0 + ty) * (unsigned)P.pitch + (unsigned)(x0 + tx);
+    inv_rho_own = ldgv(pl.p[P_IRHO] + i);
+    dpdT = ldgv(pl.p[P_DPDT] + i);
+    if (P.model == 0 && !first) pp = phi_prev[i];
+    if (unit) {
+      n4 = gdst.p[i];
+      n6 = gdst.p[P.N + i];
+    }
+  };
+  if (kFlowFirst && !heat && active) pre_flow();
+  if (heat && active) pre_heat();
   if (!heat || q < RING) {
     int x = x0 + hx - 1, y = y0 + hy - 1;
     if (!interior) {
@@ -336,16 +380,14 @@ __global__ void __launch_bounds__(2 * CX* CY)
     if (!heat) Q = C.flow.qG144 * (sx * sx + sy * sy);
   }
   __syncthreads();
-  const int tx = q % CX, ty = q / CX;
+  if (!active) return;
   const int x = x0 + tx, y = y0 + ty;
-  if (x >= P.nx || y >= P.ny) return;
+  if (!kFlowFirst && !heat) pre_flow();
   const Around n = around(P, x, y, interior);
   const size_t i = n.row[1] + n.col[1];
   if (!heat) {
-    R m[6], f[9];
+    R f[9];
     S* pf = fdst.p + i;
-#pragma unroll
-    for (int a = 0; a < 6; ++a) m[a] = pf[(size_t)a * P.N];
     relax_flow(m, jx, jy, rho, vx, vy, Fx, Fy, Q, C, f);
 #pragma unroll
     for (int a = 0; a < 9; ++a) pf[(size_t)a * P.N] = f[a];
@@ -356,7 +398,7 @@ __global__ void __launch_bounds__(2 * CX* CY)
   hy = ty + 1;
   R c[3][3];
   gather(pl.p[P_T], n, c);
-  const R inv_rho = ldgv(pl.p[P_IRHO] + i), dpdT = ldgv(pl.p[P_DPDT] + i);
+  const R inv_rho = inv_rho_own;
   const R T = c[1][1];
   const R lap6 = (((c[1][2] + c[1][0]) + (c[2][1] + c[0][1])) * 4 + ((c[2][2] + c[2][0]) + (c[0][0] + c[0][2]))) - T * 20;
   const R gTa = c[2][2] - c[0][0], gTb = c[0][2] - c[2][0];
@@ -387,15 +429,14 @@ __global__ void __launch_bounds__(2 * CX* CY)
     }
     S0 = phi;
     if (P.model == 0) {  // S0 = phi + 0.5 dt d_t phi, d_t phi ~ [phi(t) - phi(t - dt)]/dt (Eq. 46)
-      const R pp = first ? phi : phi_prev[i];
-      S0 = phi + (phi - pp) * 0.5f;
+      S0 = phi + (phi - (first ? phi : pp)) * 0.5f;
     }
   }
   phi_prev[i] = phi;
   R g[9];
   S* pg = gdst.p + i;
-  if (P.model == 0 && P.heat_unit_rates) {
-    relax_heat_unit(pg[0], pg[P.N], T, vx, vy, S0, g);
+  if (unit) {
+    relax_heat_unit(n4, n6, T, vx, vy, S0, g);
   } else {
     pull<S, R>(gsrc, C.wg, P, x, y, g);
     heat_closure(g, P, x, y);
@@ -434,7 +475,7 @@ __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_i
                                                 PopBuf<S> f, PopBuf<S> g, DevParams P) {
   const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
-  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  const auto [x, y] = node_at(P, i);
   if (x >= P.nx) return;
   double fv[9], gv[9];
 #pragma unroll
@@ -482,7 +523,7 @@ __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, 
   for (int k = 0; k < K; ++k) {
     const long long i = ((long long)blockIdx.x * K + k) * BLOCK + tid;
     if (i >= P.N) break;
-    const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+    const auto [x, y] = node_at(P, i);
     if (x >= P.nx) continue;
     double f[9], g[9];
     pull_closed<S, double>(fsrc, gsrc, P, x, y, f, g);
@@ -501,7 +542,7 @@ __global__ void __launch_bounds__(BLOCK) k_export_pops(PopBuf<S> fsrc, PopBuf<S>
                                                        int only, double* __restrict__ out) {
   const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
-  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  const auto [x, y] = node_at(P, i);
   if (x >= P.nx) return;
   double f[9], g[9];
   pull_closed<S, double>(fsrc, gsrc, P, x, y, f, g);
@@ -520,7 +561,7 @@ __global__ void __launch_bounds__(BLOCK) k_export_fields(Planes<R> pl, DevParams
                                                          double* T) {
   const long long i = (long long)blockIdx.x * BLOCK + pdl_wait<BLOCK>();
   if (i >= P.N) return;
-  const int y = (int)(i / P.pitch), x = (int)(i - (long long)y * P.pitch);
+  const auto [x, y] = node_at(P, i);
   if (x >= P.nx) return;
   const long long o = (long long)y * P.nx + x;  // outputs have no padding
   if (rho) rho[o] = (double)pl.p[P_RHO][i];
