@@ -318,18 +318,20 @@ template <class S> cudaError_t seg_step(lbpc_batch* b, int rel) {
   auto flush = [&]() -> cudaError_t {
     if (L->n == 0) return cudaSuccess;
     cudaError_t e;
+    L->waits = launches == 0;
     if (L->n <= SMALL) {  // the same records in the kernel with smaller parameters
       memset(Ls.get(), 0, sizeof(lbpc::SegLaunch<S, SMALL>));
       Ls->n = L->n;
       Ls->tiles = L->tiles;
       Ls->staged = L->staged;
+      Ls->waits = launches == 0;
       for (int j = 0; j < L->n; ++j) {
         Ls->first_tile[j] = L->first_tile[j];
         Ls->in[j] = L->in[j];
       }
-      e = lbpc::batch_seg_launch(b->prec, b->variant, true, Ls.get(), tickets(b, launches), launches > 0, b->stream);
+      e = lbpc::batch_seg_launch(b->prec, b->variant, true, Ls.get(), tickets(b, launches), b->stream);
     } else {
-      e = lbpc::batch_seg_launch(b->prec, b->variant, false, L.get(), tickets(b, launches), launches > 0, b->stream);
+      e = lbpc::batch_seg_launch(b->prec, b->variant, false, L.get(), tickets(b, launches), b->stream);
     }
     ++launches;
     L->n = 0;

@@ -122,17 +122,18 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
 // One block per instance slot: rho_ave from the tile partials (fixed order), then flip the buffers
 // and count the step.
 template <class S>
-__global__ void __launch_bounds__(128) k_batch_advance(BatchInst<S>* __restrict__ insts) {
+__global__ void __launch_bounds__(128) k_batch_advance(BatchInst<S>* insts) {
   __shared__ double red[4];
+  const int t = pdl_wait<128>();
   BatchInst<S>& I = insts[blockIdx.x];
   if (!I.active) return;
   if (I.P.buoyancy == 1) {  // rho_ave for the next step
     double acc = 0.0;
-    for (int j = threadIdx.x; j < I.ntiles; j += 128) acc += I.partials[j];
+    for (int j = t; j < I.ntiles; j += 128) acc += __ldcg(I.partials + j);
     acc = block_sum<128>(acc, red);
-    if (threadIdx.x == 0) I.scalars[0] = acc / node_count(I.P);
+    if (t == 0) I.scalars[0] = acc / node_count(I.P);
   }
-  if (threadIdx.x == 0) {
+  if (t == 0) {
     I.cur ^= 1;
     I.step += 1;
   }
@@ -144,7 +145,7 @@ static cudaError_t batch_launch_t(int ctas, const BatchMeta* d_meta, void* d_ins
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   k_batch_step<S, R, TX, TY, NPT><<<sms * ctas, TX * TY / NPT, 0, st>>>(d_meta, (const BatchInst<S>*)d_insts);
-  if (ninst > 0) k_batch_advance<S><<<ninst, 128, 0, st>>>((BatchInst<S>*)d_insts);
+  if (ninst > 0) launch_pdl(k_batch_advance<S>, ninst, 128, 0, st, (BatchInst<S>*)d_insts);
   return cudaGetLastError();
 }
 
@@ -163,9 +164,9 @@ static cudaError_t batch_launch_p(int variant, int ctas, const BatchMeta* d_meta
 
 cudaError_t batch_advance_launch(int prec, void* d_insts, int ninst, cudaStream_t st) {
   if (ninst <= 0) return cudaSuccess;
-  if (prec == 0) k_batch_advance<double><<<ninst, 128, 0, st>>>((BatchInst<double>*)d_insts);
-  else if (prec == 1) k_batch_advance<float><<<ninst, 128, 0, st>>>((BatchInst<float>*)d_insts);
-  else k_batch_advance<__half><<<ninst, 128, 0, st>>>((BatchInst<__half>*)d_insts);
+  if (prec == 0) launch_pdl(k_batch_advance<double>, ninst, 128, 0, st, (BatchInst<double>*)d_insts);
+  else if (prec == 1) launch_pdl(k_batch_advance<float>, ninst, 128, 0, st, (BatchInst<float>*)d_insts);
+  else launch_pdl(k_batch_advance<__half>, ninst, 128, 0, st, (BatchInst<__half>*)d_insts);
   return cudaGetLastError();
 }
 

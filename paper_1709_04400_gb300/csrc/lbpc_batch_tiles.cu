@@ -13,8 +13,9 @@ namespace lbpc {
 // The launches of one step cover disjoint instances, so each lets the next one start while its own
 // last CTAs run (programmatic dependent launch). The last CTA of a launch waits, before it exits, for
 // the launch before it to complete: a launch then completes only after every earlier launch of the step
-// has, and the advance kernel that follows in stream order sees the whole step. The earlier launch's
-// CTAs have all started when this one starts, so the wait always ends.
+// has, and the advance kernel, which waits for the last one, sees the whole step. The first launch of a
+// step (waits) in turn waits for the advance kernel before it reads anything. The earlier launch's
+// CTAs have all started when this one starts, so the waits always end.
 template <class S, class R, int TX, int TY, int NPT, int CAP>
 __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NPT, NPT>())
     k_batch_tiles(const __grid_constant__ SegLaunch<S, CAP> L) {
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
     k_batch_walk(const __grid_constant__ SegLaunch<S, CAP> L, unsigned long long* __restrict__ tickets) {
   using B = TmaBox<S, TX, TY>;
   constexpr int NTH = TX * TY;
+  if (L.waits) pdl_wait<NTH>();  // every address below depends on shared memory written after it
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ FusedSmem<R, TX, TY> sm;
   struct Tile {
@@ -136,7 +138,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
 }
 
 template <class S, class R, int CAP>
-static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, bool pdl, cudaStream_t st, bool* done) {
+static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, cudaStream_t st, bool* done) {
   using B = TmaBox<S, 32, 8>;
   const SegLaunch<S, CAP>& L = *(const SegLaunch<S, CAP>*)Lh;
   auto* kernel = k_batch_walk<S, R, 32, 8, CAP>;
@@ -163,12 +165,12 @@ static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, bo
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, L, tickets);
 }
 
 template <class S, class R, int TX, int TY, int NPT, int CAP>
-static cudaError_t seg_launch_t(const void* Lh, bool pdl, cudaStream_t st) {
+static cudaError_t seg_launch_t(const void* Lh, cudaStream_t st) {
   const SegLaunch<S, CAP>& L = *(const SegLaunch<S, CAP>*)Lh;
   if (L.n <= 0 || L.tiles <= 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
@@ -179,44 +181,44 @@ static cudaError_t seg_launch_t(const void* Lh, bool pdl, cudaStream_t st) {
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  // a step's first launch is an ordinary one: a wait in the kernel costs every tile of it 1 %
+  cfg.numAttrs = L.waits ? 0 : 1;
   return cudaLaunchKernelEx(&cfg, k_batch_tiles<S, R, TX, TY, NPT, CAP>, L);
 }
 
 template <class S, class R, int CAP>
-static cudaError_t seg_launch_c(int variant, const void* L, bool pdl, cudaStream_t st) {
+static cudaError_t seg_launch_c(int variant, const void* L, cudaStream_t st) {
   switch (variant) {
-    case 1: return seg_launch_t<S, R, 32, 16, 1, CAP>(L, pdl, st);
-    case 2: return seg_launch_t<S, R, 64, 8, 1, CAP>(L, pdl, st);
-    case 3: return seg_launch_t<S, R, 32, 16, 2, CAP>(L, pdl, st);
-    case 4: return seg_launch_t<S, R, 64, 16, 2, CAP>(L, pdl, st);
-    case 5: return seg_launch_t<S, R, 32, 32, 2, CAP>(L, pdl, st);
-    default: return seg_launch_t<S, R, 32, 8, 1, CAP>(L, pdl, st);
+    case 1: return seg_launch_t<S, R, 32, 16, 1, CAP>(L, st);
+    case 2: return seg_launch_t<S, R, 64, 8, 1, CAP>(L, st);
+    case 3: return seg_launch_t<S, R, 32, 16, 2, CAP>(L, st);
+    case 4: return seg_launch_t<S, R, 64, 16, 2, CAP>(L, st);
+    case 5: return seg_launch_t<S, R, 32, 32, 2, CAP>(L, st);
+    default: return seg_launch_t<S, R, 32, 8, 1, CAP>(L, st);
   }
 }
 
 template <class S, class R>
-static cudaError_t seg_launch_p(int variant, bool small, const void* L, bool pdl, cudaStream_t st) {
-  return small ? seg_launch_c<S, R, kSegSmall>(variant, L, pdl, st)
-               : seg_launch_c<S, R, seg_capacity<S>()>(variant, L, pdl, st);
+static cudaError_t seg_launch_p(int variant, bool small, const void* L, cudaStream_t st) {
+  return small ? seg_launch_c<S, R, kSegSmall>(variant, L, st)
+               : seg_launch_c<S, R, seg_capacity<S>()>(variant, L, st);
 }
 
-cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, bool pdl,
-                             cudaStream_t st) {
+cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, cudaStream_t st) {
   if (variant == 0 && (prec == 1 || prec == 2)) {
     bool done = false;
     cudaError_t e;
     if (prec == 1)
-      e = small ? walk_launch_c<float, float, kSegSmall>(L, tickets, pdl, st, &done)
-                : walk_launch_c<float, float, seg_capacity<float>()>(L, tickets, pdl, st, &done);
+      e = small ? walk_launch_c<float, float, kSegSmall>(L, tickets, st, &done)
+                : walk_launch_c<float, float, seg_capacity<float>()>(L, tickets, st, &done);
     else
-      e = small ? walk_launch_c<__half, float, kSegSmall>(L, tickets, pdl, st, &done)
-                : walk_launch_c<__half, float, seg_capacity<__half>()>(L, tickets, pdl, st, &done);
+      e = small ? walk_launch_c<__half, float, kSegSmall>(L, tickets, st, &done)
+                : walk_launch_c<__half, float, seg_capacity<__half>()>(L, tickets, st, &done);
     if (e != cudaSuccess || done) return e;
   }
-  if (prec == 0) return seg_launch_p<double, double>(variant, small, L, pdl, st);
-  if (prec == 1) return seg_launch_p<float, float>(variant, small, L, pdl, st);
-  return seg_launch_p<__half, float>(variant, small, L, pdl, st);
+  if (prec == 0) return seg_launch_p<double, double>(variant, small, L, st);
+  if (prec == 1) return seg_launch_p<float, float>(variant, small, L, st);
+  return seg_launch_p<__half, float>(variant, small, L, st);
 }
 
 }  // namespace lbpc

@@ -183,7 +183,7 @@ template <class S, int CAP> struct SegLaunch {
   int n;      // instances of this launch
   int tiles;  // its tiles
   int staged; // those of them that tensor copies can stage
-  int pad_;
+  int waits;  // the first launch of its step: waits for the step before it
   int first_tile[CAP];  // each instance's first CTA, ascending: kept together so that the search of a
                         // CTA's instance reads a few cache lines
   SegInst<S> in[CAP];
@@ -191,12 +191,11 @@ template <class S, int CAP> struct SegLaunch {
 static_assert(sizeof(SegLaunch<double, seg_capacity<double>()>) <= kSegParamBytes &&
                   sizeof(SegLaunch<float, seg_capacity<float>()>) <= kSegParamBytes,
               "per-tile launch parameters");
-// tickets: two zeroed words of this launch's own in device memory, left zero.
 // Enqueue one per-tile launch over the instances of L, a host SegLaunch<S, CAP> of the batch's storage
-// type with CAP = kSegSmall (small) or seg_capacity<S>(). pdl: the launch may begin while the previous
-// kernel on st drains (its instances are others).
-cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, bool pdl,
-                             cudaStream_t st);
+// type with CAP = kSegSmall (small) or seg_capacity<S>(). Unless L waits, the launch may begin while the previous
+// kernel on st drains (its instances are others). tickets: two zeroed words of this launch's own in device memory,
+// left zero.
+cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, cudaStream_t st);
 // Enqueue the per-instance advance of a step (rho_ave, buffer parity, step count).
 cudaError_t batch_advance_launch(int prec, void* d_insts, int ninst, cudaStream_t st);
 // Largest resident CTAs per SM of the step kernel for (prec, variant).
