@@ -222,21 +222,22 @@ def fused_bytes_per_node(prec_bytes):
     return prec_bytes * (18 + 18 + 2)
 
 
-# Algorithmic traffic of the split collide kernel per node: pull 9 f + 9 g, write 9 f* + 9 g*,
-# read/write phi_prev, read the centre of 9 scratch planes (rho, T, 1/rho, vx, vy, Fx, Fy, Q, dp/dT);
-# the neighbour reads of T, vx, vy (and rho) are served by L1/L2 and not counted.
+# Algorithmic traffic of the split collide kernel per node. 8-byte storage (force and collision in one kernel): read
+# the six flow moments, the two heat fluxes and the centre of 7 scratch planes (rho, T, psi, jx, jy, 1/rho,
+# dp/dT), write 9 f* + 9 g*, read/write phi_prev. Otherwise: pull 9 f + 9 g, write 9 f* + 9 g*, read/write phi_prev,
+# read the centre of 9 scratch planes (rho, T, 1/rho, vx, vy, Fx, Fy, Q, dp/dT). The neighbour reads are served
+# by L1/L2 and not counted.
 def collide_bytes_per_node(prec_bytes):
-    return prec_bytes * (18 + 18 + 2 + 9)
+    return prec_bytes * ((8 + 7 + 18 + 2) if prec_bytes == 8 else (18 + 18 + 2 + 9))
 
 
 # Algorithmic FP64 operations of the split collide kernel per node (each add, subtract, multiply and
 # divide counted once; an FMA counts as its multiply and its add), counted term by term from the
-# kernel: flow collision 136 (moments 34, equilibria and forcing 29, relaxation of 6 moments 30,
-# back-transform 41, momentum update 2); heat role 93 with unit thermal rates (gradients 41, source 14,
-# thermal collision in closed form 38); general thermal rates take the full MRT collision, 78 more;
-# lambda = rho c_V chi adds 20 for grad rho.
+# binary64 kernel: force, velocity and sigma term 23 (the repeats on a tile's ring are not counted); flow collision
+# from its moments 82; heat role 62 with unit thermal rates (lap T 10, div v 12, source 12, thermal collision in
+# closed form 28); general thermal rates take the full MRT collision, 88 more; lambda = rho c_V chi adds 25.
 def collide_flops(lambda_mode, unit_heat_rates):
-    return 229 + (20 if lambda_mode == "rho_cv_chi" else 0) + (0 if unit_heat_rates else 78)
+    return 167 + (25 if lambda_mode == "rho_cv_chi" else 0) + (0 if unit_heat_rates else 88)
 
 
 # arithmetic type of each storage precision ("df64": double-word, pairs of binary32 with a 48-bit

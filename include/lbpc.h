@@ -174,8 +174,8 @@ lbpc_status lbpc_step_timed(lbpc_ctx* c, float* kernel_ms, int32_t max_kernels, 
 const char* lbpc_kernel_name(const lbpc_ctx* c, int32_t k);
 
 /* Kernel organisation of lbpc_step. LBPC_PATH_SPLIT: node-parallel kernels (two per step for 8-byte
- * storage, three otherwise) with scratch planes (each EOS evaluated once per node; the faster choice when FP64 arithmetic bounds
- * the step). LBPC_PATH_FUSED: one kernel per step over shared-memory tiles (populations read once
+ * storage, three otherwise) with scratch planes (each EOS evaluated once per node; the faster choice
+ * when FP64 arithmetic bounds the step). LBPC_PATH_FUSED: one kernel per step over shared-memory tiles (populations read once
  * and written once; the faster choice when HBM bounds the step). LBPC_PATH_AUTO (default): split
  * for LBPC_FP64 and LBPC_DF64, fused for LBPC_FP32 and LBPC_FP16DEV. Both compute the same step.
  * The fused step launches one row of CTAs per 8 grid rows, and a launch has at most 65,535 rows of
@@ -188,8 +188,8 @@ lbpc_status lbpc_set_path(lbpc_ctx* c, int32_t path);
  * thread; 1 = 32 x 8, one node per thread (smaller shared-memory footprint, four CTAs per SM, more halo
  * recomputation); 2 = 32 x 16, two nodes per thread; 3 = 32 x 32, two nodes per thread (less halo
  * recomputation per node); 4 = 32 x 8 in persistent CTAs that take tiles in order and start each next
- * tile's staging copy while they finish the current tile (default). Where the rows are not 16-byte
- * multiples (no staging), 4 runs as 1. All compute the same step. LBPC_EINVAL outside 0..4. */
+ * tile's staging copy while they finish the current tile (default). Small grids, and domains of fewer than
+ * 64 columns whose rows are not 16-byte multiples (no staging), run 4 as 1. All compute the same step. LBPC_EINVAL outside 0..4. */
 lbpc_status lbpc_set_fused_tile(lbpc_ctx* c, int32_t tile);
 
 /* Synchronise the stream and check the device status word. */
@@ -256,8 +256,8 @@ void lbpc_destroy(lbpc_ctx* c);
 /* ------------------------------------------------------------------------------------------------
  * Batches: many independent simulations of uneven size advancing together.
  *
- * The per-node arithmetic is the fused step's. A step is a few per-tile launches, one CTA per tile,
- * each holding up to lbpc_batch_per_tile_capacity instances in its kernel parameters (the default),
+ * The per-node arithmetic is the fused step's. A step is a few per-tile launches (one CTA per tile, or
+ * persistent CTAs that walk a launch of many tiles), each holding up to lbpc_batch_per_tile_capacity instances in its kernel parameters (the default),
  * or one launch whose CTAs walk a device-resident work list of (instance, tile) entries (see
  * lbpc_batch_set_config). Steps are replayed through captured CUDA graphs in chunks when the batch
  * has a non-default stream. Instances can join and leave between calls. Their parameters,
@@ -308,7 +308,8 @@ int64_t lbpc_batch_step_count(const lbpc_batch* b, int32_t id);
  * from their index in steps of the grid size. Up to the residency limit of the variant, every CTA is
  * resident (a persistent grid). Above it, up to 64 times that limit, further CTAs start as earlier
  * ones finish, so the hardware balances tiles of uneven cost. A value above that returns LBPC_EINVAL.
- * ctas_per_sm = 0: per-tile launches. A step is a sequence of launches with one CTA per tile, each over
+ * ctas_per_sm = 0: per-tile launches. A step is a sequence of launches with one CTA per tile (variant 0 in
+ * 4- and 2-byte storage: persistent CTAs where a launch has many tiles, most of them interior), each over
  * up to lbpc_batch_per_tile_capacity instances held in its kernel parameters; each launch may start
  * while the previous one drains. A change of instances then captures the step graphs again.
  * A negative value returns LBPC_EINVAL. */

@@ -14,7 +14,10 @@
 // arithmetic the step is bound by the FP64 pipe (84 % busy in both kernels), not by HBM, so its time is its
 // count of FP64 instructions: 229 per node and step (k_macro 85, k_collide_tile 144). Three kernels that
 // pulled f and g twice and rebuilt m* from all nine moments took 283. GB300, droplet evaporation 2048^2: 1.82 ms
-// a step against 2.24 ms; 128^2 17.1 us against 20.6 us. Double-word arithmetic: 0.479 against 0.533 ms.
+// a step against 2.24 ms; 128^2 12 us against 20.6 us (with launch_pdl). Double-word arithmetic: 0.428 against
+// 0.533 ms; there k_macro is at the measured HBM bandwidth (264 B per node in 164 us) and k_collide_tile at 64 % of
+// it (280 B in 271 us) and bound by issue and latency.
+
 #include <type_traits>
 
 #include "lbpc_device.cuh"
@@ -281,8 +284,9 @@ template <class R> __device__ __forceinline__ void gather(const R* __restrict__ 
 }
 
 // Force and collision of the binary64 and double-word steps in one kernel over tiles of CX x CY nodes. The
-// velocities of the tile and its 1-ring go to shared memory (the force of the ring is repeated), so the force,
-// the velocity and the sigma term never visit device memory and the step is two launches. Then the two roles of
+// velocities of the tile and its 1-ring go to shared memory (the force of the ring is repeated: 15 of the 229
+// binary64 instructions, 1.4 times), so the force, the velocity and the sigma term never visit device memory and the
+// step is two launches. Then the two roles of
 // k_collide: the first half of the block relaxes f from the moments that k_macro left in fdst, the second half
 // evaluates the source and relaxes g from T, n4, n6 (or pulls g again where the rates are not all 1).
 //
