@@ -255,11 +255,11 @@ def _dtypes():
 # the entry describes another build and the line reports null.
 MEASURED_TRAFFIC = {
     # one-pass ncu captures (dram__bytes_read.sum + dram__bytes_write.sum) of the bench's own commands
-    ("k_collide", "droplet_evaporation_2048_dT0.1Tc", "fp64"): (1_539_444_224, "51ee3432028044b0"),
-    ("k_collide", "droplet_evaporation_2048_dT0.1Tc", "df64"): (1_640_148_224, "51ee3432028044b0"),
-    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp32"): (2_502_832_640, "51ee3432028044b0"),
-    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp16"): (1_576_405_248, "51ee3432028044b0"),
-    ("k_batch_tiles", "batched_evaporation_256", "fp32"): (3_894_301_184, "51ee3432028044b0"),  # one step: 5 launches
+    ("k_collide", "droplet_evaporation_2048_dT0.1Tc", "fp64"): (1_112_460_288, "cb85eefc95c5856a"),
+    ("k_collide", "droplet_evaporation_2048_dT0.1Tc", "df64"): (1_112_793_856, "cb85eefc95c5856a"),
+    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp32"): (2_511_309_824, "cb85eefc95c5856a"),
+    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp16"): (1_581_058_048, "cb85eefc95c5856a"),
+    ("k_batch_walk", "batched_evaporation_256", "fp32"): (3_967_152_640, "cb85eefc95c5856a"),  # one step: 5 launches
 }
 
 
@@ -413,7 +413,8 @@ def batch_measure(lbpc, workloads, prec, instances, steps, warmup, variant=-1, c
     # per-tile launches (0 CTAs per SM): ceil(instances / capacity) launches and the advance per step;
     # the work-list kernel: one launch and the advance
     per_tile = cfg["ctas_per_sm"] == 0
-    kernel = "k_batch_tiles" if per_tile else "k_batch_step"
+    # per-tile launches of this many tiles are walked by persistent CTAs; smaller ones run k_batch_tiles
+    kernel = "k_batch_walk" if per_tile else "k_batch_step"
     launches_per_step = (-(-len(insts) // lbpc.Batch.per_tile_capacity(prec)) + 1) if per_tile else 2
     bpn = storage_bytes_per_node(prec, lbpc)
     achieved = bpn * nodes / (batch_s / steps) / 1e9
