@@ -389,16 +389,42 @@ __host__ __device__ __forceinline__ long long wall_doubles(int nx) { return 4LL 
 template <class S> struct is_half_t { static constexpr bool value = false; };
 template <> struct is_half_t<__half> { static constexpr bool value = true; };
 
+// double(x) from the bits, exact for every x (NaN stays NaN): a conversion instruction runs at the FP64 pipe's rate,
+// a seventieth of the integer and binary32 ones. A subnormal is scaled into the normal numbers first. A dozen
+// instructions more per value in flight, so it pays where the FP64 pipe and not latency sets the time (launch_sums).
+__host__ __device__ __forceinline__ double widen(float x) {
+  union { float f; unsigned u; } v;
+  v.f = x;
+  const bool tiny = (v.u & 0x7f800000u) == 0;
+  v.f = x * (tiny ? 4294967296.0f : 1.0f);
+  unsigned bias = tiny ? 0x38000000u - (32u << 20) : 0x38000000u;
+  if ((v.u & 0x7f800000u) == 0x7f800000u) bias = 0x70000000u;
+  if ((v.u & 0x7fffffffu) == 0) bias = 0;
+  const unsigned hi = ((unsigned)((int)v.u >> 3) & 0x8fffffffu) + bias;
+  union { unsigned long long u; double d; } r;
+  r.u = ((unsigned long long)hi << 32) | (v.u << 29);
+  return r.d;
+}
+template <class R, bool BITS> __device__ __forceinline__ R widen_to(float x) {
+  if constexpr (BITS) return widen(x);
+  else return R(x);
+}
+
 // IX is the index type: long long in general; int where the caller guarantees that every population
 // index of the buffer (9 N) fits in 31 bits, which turns each address into one 32-bit multiply-add.
-template <class S, class R, class IX = long long>
+// BITS (R = double): narrower storage widened from its bits, see widen.
+template <class S, class R, class IX = long long, bool BITS = false>
 __device__ __forceinline__ R pop_load(const PopBuf<S>& b, IX N, int a, IX idx, const R* w) {
   if constexpr (is_half_t<S>::value) {
-    return R(__half2float(__ldg(b.p + ((IX)a * N + idx)))) + w[a] * R(__ldg(b.ref + idx));
+    return widen_to<R, BITS>(__half2float(__ldg(b.p + ((IX)a * N + idx)))) +
+           w[a] * widen_to<R, BITS>(__ldg(b.ref + idx));
   } else if constexpr (is_dw_t<S>::value) {
-    return R(ldgv(b.p + ((IX)a * N + idx)));
+    const dw v = ldgv(b.p + ((IX)a * N + idx));
+    if constexpr (BITS) return widen(v.hi) + widen(v.lo);
+    else return R(v);
   } else {
-    return R(__ldg(b.p + ((IX)a * N + idx)));
+    if constexpr (BITS && sizeof(S) == 4) return widen(__ldg(b.p + ((IX)a * N + idx)));
+    else return R(__ldg(b.p + ((IX)a * N + idx)));
   }
 }
 
@@ -456,13 +482,13 @@ template <class PT> __device__ __forceinline__ PullSrc pull_src(const PT& P, int
   return s;
 }
 
-template <class S, class R, class IX = long long, class PT = DevParams>
+template <class S, class R, class IX = long long, class PT = DevParams, bool BITS = false>
 __device__ __forceinline__ void pull_from(const PopBuf<S>& src, const R* w, const PT& P, const PullSrc& s,
                                           R v[9]) {
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     const int r = s.row[EY(a) + 1];
-    v[a] = r >= 0 ? pop_load<S, R, IX>(src, (IX)P.N, a, (IX)r * P.pitch + s.col[EX(a) + 1], w) : R(0);
+    v[a] = r >= 0 ? pop_load<S, R, IX, BITS>(src, (IX)P.N, a, (IX)r * P.pitch + s.col[EX(a) + 1], w) : R(0);
   }
 }
 
@@ -585,13 +611,13 @@ template <class R, class PT> __device__ __forceinline__ void heat_closure(R g[9]
 }
 
 // Post-stream, post-boundary f and g at (x, y).
-template <class S, class R, class IX = long long, class PT = DevParams>
+template <class S, class R, class IX = long long, class PT = DevParams, bool BITS = false>
 __device__ __forceinline__ void pull_closed(const PopBuf<S>& fsrc, const PopBuf<S>& gsrc, const PT& P, int x,
                                             int y, R f[9], R g[9]) {
   const Coefs<R>& C = coefs<R>(P);
   const PullSrc src = pull_src(P, x, y);  // f and g read the same nine source nodes
-  pull_from<S, R, IX>(fsrc, C.wf, P, src, f);
-  pull_from<S, R, IX>(gsrc, C.wg, P, src, g);
+  pull_from<S, R, IX, PT, BITS>(fsrc, C.wf, P, src, f);
+  pull_from<S, R, IX, PT, BITS>(gsrc, C.wg, P, src, g);
   flow_closure(f, P, x, y, fsrc.wall);
   heat_closure(g, P, x, y);
 }

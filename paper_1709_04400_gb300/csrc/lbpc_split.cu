@@ -514,13 +514,34 @@ __global__ void __launch_bounds__(BLOCK) k_init(const double* __restrict__ rho_i
   pop_store<S, double>(g, P.N, i, gv, T_in[(long long)y * P.nx + x], P.cd.wg);
 }
 
+// Totals of two values over a block in block_sum's order, with half its additions: lanes 0 to 15 go on with the pairs'
+// sums of a, lanes 16 to 31 with those of b. Valid in thread 0 (a) and thread 16 (b).
+template <int NTH> __device__ __forceinline__ double block_sum_pair(int tid, double a, double b, double* smem) {
+  const int lane = tid & 31, w = tid >> 5;
+  const bool lo = lane < 16;
+  const double other = __shfl_xor_sync(0xffffffffu, lo ? b : a, 16);
+  double v = (lo ? a : b) + other;
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  if ((lane & 15) == 0) smem[(lane >> 4) * (NTH / 32) + w] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (w == 0) {
+    if ((lane & 15) < NTH / 32) s = smem[(lane >> 4) * (NTH / 32) + (lane & 15)];
+#pragma unroll
+    for (int o = NTH / 64; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+  }
+  __syncthreads();
+  return s;
+}
+
 // Sums of rho and T over the current (post-boundary) state into per-block partials. Bound by the FP64 pipe
-// (16 additions per node, and a conversion per population of a narrower storage), so a thread takes K nodes
-// before the block's reduction, whose 30 instructions per warp K = 1 pays for every 32 nodes.
-template <class S, int K>
+// (16 additions per node, and without BITS a conversion per population of a narrower storage), so a thread takes K nodes
+// before the block's reduction, whose 7 instructions per warp K = 1 pays for every 32 nodes.
+template <class S, int K, bool BITS>
 __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, DevParams P,
                                                 double* __restrict__ partials, int stride) {
-  __shared__ double red[BLOCK / 32];
+  __shared__ double red[2 * (BLOCK / 32)];
   const int tid = pdl_wait<BLOCK>();
   double r = 0.0, t = 0.0;
 #pragma unroll 2
@@ -530,14 +551,12 @@ __global__ void __launch_bounds__(BLOCK) k_sums(PopBuf<S> fsrc, PopBuf<S> gsrc, 
     const auto [x, y] = node_at(P, i);
     if (x >= P.nx) continue;
     double f[9], g[9];
-    pull_closed<S, double>(fsrc, gsrc, P, x, y, f, g);
+    pull_closed<S, double, long long, DevParams, BITS>(fsrc, gsrc, P, x, y, f, g);
     r += f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
     t += g[0] + g[1] + g[2] + g[3] + g[4] + g[5] + g[6] + g[7] + g[8];
   }
-  const double sr = block_sum<BLOCK>(r, red);
-  if (tid == 0) partials[blockIdx.x] = sr;
-  const double st = block_sum<BLOCK>(t, red);
-  if (tid == 0) partials[stride + blockIdx.x] = st;
+  const double s = block_sum_pair<BLOCK>(tid, r, t, red);
+  if (tid == 0 || tid == 16) partials[(tid >> 4) * stride + blockIdx.x] = s;
 }
 
 // Post-boundary populations of the current state as FP64 [9][ny][nx] (which = 0: f, 1: g).
@@ -665,15 +684,20 @@ const char* split_kernel_name(int prec, int k) {
 }
 
 // Enqueue k_sums; returns its number of blocks. Four nodes per thread on large grids (2048^2 with k_finish: binary64
-// 264 us, 303 with one node; binary32 399, 436), one where latency counts (256^2: 13.1 us, 15.4 with four).
+// 264 us, 303 with one node), one where latency counts (256^2: 13.1 us, 15.4 with four; 11.7 with the paired reduction).
+// Narrower storage is widened from its bits where the FP64 pipe sets the time. Converted and widened, us with k_finish:
+// binary32 256^2 13.8, 15.2; 512^2 31.5, 27.3; 1000^2 91.9, 78.5; double-word 128^2 8.9, 12.8; 256^2 18.6, 15.7;
+// 2048^2 652, 434; binary16 256^2 17.9, 15.9; 512^2 50.0, 32.0; 2048^2 657, 400.
 template <class S> static int launch_sums(const SplitBuffers& b, const DevParams& P, int k, cudaStream_t st) {
   const int stride = (int)blocks_for(P.N);
-  if (P.N < (1 << 20)) {
-    launch_pdl(k_sums<S, 1>, stride, BLOCK, 0, st, fbuf<S>(b, k), gbuf<S>(b, k), P, b.partials, stride);
-    return stride;
-  }
-  const int nb = (stride + 3) / 4;
-  launch_pdl(k_sums<S, 4>, nb, BLOCK, 0, st, fbuf<S>(b, k), gbuf<S>(b, k), P, b.partials, stride);
+  constexpr bool narrow = !std::is_same<S, double>::value;
+  const int nb = P.N < (1 << 20) ? stride : (stride + 3) / 4;
+  auto* kernel = k_sums<S, 1, false>;
+  if (P.N >= (1 << 20))
+    kernel = k_sums<S, 4, narrow>;
+  else if (narrow && P.N >= (sizeof(S) == 4 ? 1 << 18 : 1 << 16))
+    kernel = k_sums<S, 1, narrow>;
+  launch_pdl(kernel, nb, BLOCK, 0, st, fbuf<S>(b, k), gbuf<S>(b, k), P, b.partials, stride);
   return nb;
 }
 

@@ -149,3 +149,22 @@ def test_sums_to_every_kind_of_memory(prec):
         got = sim.fields()
         assert abs(want[0] / got[0].sum() - 1.0) < 1e-6 and abs(want[1] / got[3].sum() - 1.0) < 1e-6
         sim.close()
+
+
+@pytest.mark.parametrize("prec", [lbpc.FP64, lbpc.FP32, lbpc.FP16DEV, lbpc.DF64], ids=["fp64", "fp32", "fp16", "df64"])
+@pytest.mark.parametrize("n", [11, 363, 600, 1031])
+def test_sums_of_the_populations(prec, n):
+    """The sums against the exported populations: one block that is partly filled (11 x 11), a last block that is, in
+    rows with and without padding (363 x 363), populations widened from their bits in every storage (from 600 x 600
+    on), four nodes per thread (1031 x 1031). Fewer than 100 additions lead to a total of positive numbers, so it is
+    within 100 x 2^-53 = 1.1e-14 of the exact one; numpy's own pairwise sum is as good, and 1e-13 leaves room for
+    both."""
+    case, rho, T = workloads.droplet_evaporation(TC, RV, RL, n=n, radius=0.2 * n, dT_ratio=0.1)
+    sim = lbpc.Simulation(lbpc.params_from_case(case, prec))
+    sim.init(rho, T)
+    sim.step(2)
+    mass, heat = sim.sums()
+    f, g = sim.populations()
+    assert sim.sums() == (mass, heat)
+    sim.close()
+    assert abs(mass / f.sum() - 1.0) < 1e-13 and abs(heat / g.sum() - 1.0) < 1e-13
