@@ -65,6 +65,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
   };
   __shared__ Tile s_tile[2], s_next;
   __shared__ unsigned s_raw;  // number of the next tile
+  __shared__ int s_mapped;    // thread 0's: the instance whose tensor maps it acquired last
   extern __shared__ __align__(128) unsigned char dyn[];
   uint64_t* bar = (uint64_t*)(dyn + B::BYTES - 128);
   auto tile_at = [&](unsigned b) {
@@ -85,11 +86,20 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
     const SegInst<S>& I = L.in[t.k];
     return I.maps && t.x >= 3 && t.x + TX + 3 <= I.P.nx && t.y >= 3 && t.y + TY + 3 <= I.P.ny;
   };
+  auto stage = [&](const Tile& t) {  // thread 0 starts the copy of a staged tile
+    const TmaMaps* maps = L.in[t.k].maps;
+    if (s_mapped != t.k) {  // tiles come in order, so once per instance
+      acquire_maps<S>(maps);
+      s_mapped = t.k;
+    }
+    tma_issue_tile<S, TX, TY>(dyn, bar, *maps, t.x, t.y);
+  };
   auto take = [&]() { return (unsigned)(gridDim.x + atomicAdd(tickets, 1ull)); };
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
+    s_mapped = -1;
     const Tile t0 = tile_at(blockIdx.x);
-    if (staged(t0)) tma_issue_tile<S, TX, TY>(dyn, bar, *L.in[t0.k].maps, t0.x, t0.y);
+    if (staged(t0)) stage(t0);
     s_tile[0] = t0;
     s_raw = take();
   }
@@ -104,7 +114,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
     auto start_next = [&]() {
       if (threadIdx.x != 0) return;
       const Tile next = s_next;
-      if (staged(next)) tma_issue_tile<S, TX, TY>(dyn, bar, *L.in[next.k].maps, next.x, next.y);
+      if (staged(next)) stage(next);
     };
     const int k = __shfl_sync(0xffffffffu, tile.k, 0);
     const int x0 = __shfl_sync(0xffffffffu, tile.x, 0), y0 = __shfl_sync(0xffffffffu, tile.y, 0);
