@@ -89,8 +89,9 @@ struct HostInst {
   lbpc::DevParams dp{};
   long long N = 0;  // nodes
   size_t off = 0, bytes = 0;  // arena block of the instance
-  size_t f[2], g[2], rf[2], rg[2], wall[2], phi, partials, scalars, maps;
-  bool staged = false;        // the device holds tensor maps of both buffers
+  size_t f[2], g[2], rf[2], rg[2], wall[2], phi, partials, scalars;
+  bool staged = false;        // maps holds the tensor maps of both buffers
+  lbpc::TmaMaps maps[2];
   size_t npartials = 0;
   long long step = 0;
   int cur = 0;
@@ -122,7 +123,6 @@ size_t layout_instance(const lbpc_params* p, HostInst* h) {
   h->npartials = std::max(lbpc::fused_max_tiles(p->nx, p->ny), 2 * (size_t)((N + lbpc::split_block() - 1) / lbpc::split_block()));
   h->partials = off; off += a256(h->npartials * sizeof(double));
   h->scalars = off; off += a256(8 * sizeof(double));
-  h->maps = off; off += sb <= 4 ? 2 * sizeof(lbpc::TmaMaps) : 0;
   return off;
 }
 
@@ -303,73 +303,104 @@ unsigned long long* tickets(lbpc_batch* b, int k) {
   return (unsigned long long*)(b->base + b->meta_off + a256(sizeof(lbpc::BatchMeta))) + 2 * k;
 }
 
-// One step as per-tile launches (ctas == 0): the active instances in launches of up to seg_capacity, each
-// instance reading the buffer of parity h.cur ^ rel, then the per-instance advance. Whether the step is
+// An instance's tiles in the batch's tile shape, and those of them that tensor copies can stage: interior ones, 3 nodes
+// from every edge.
+long long tiles_of(const lbpc_batch* b, const HostInst& h, long long* staged = nullptr) {
+  int tx, ty;
+  lbpc::batch_tile_shape(b->variant, tx, ty);
+  if (staged)
+    *staged = h.staged ? (long long)std::max(0, (h.dp.nx - tx - 3) / tx) * std::max(0, (h.dp.ny - ty - 3) / ty) : 0;
+  return (long long)((h.dp.nx + tx - 1) / tx) * ((h.dp.ny + ty - 1) / ty);
+}
+
+// The record of instance k for a launch that reads the buffer of parity h.cur ^ rel.
+template <class S> void fill_seg(const lbpc_batch* b, int k, int rel, lbpc::SegInst<S>& r) {
+  const HostInst& h = b->inst[k];
+  int tx, ty;
+  lbpc::batch_tile_shape(b->variant, tx, ty);
+  char* base = b->base + h.off;
+  const int c = h.cur ^ rel, d = c ^ 1;
+  const bool half = b->prec == LBPC_FP16DEV;
+  r.P = lbpc::params_of<typename lbpc::ArithOf<S>::type>(h.dp);
+  r.fs = lbpc::PopBuf<S>{(S*)(base + h.f[c]), half ? (float*)(base + h.rf[c]) : nullptr, (double*)(base + h.wall[c])};
+  r.gs = lbpc::PopBuf<S>{(S*)(base + h.g[c]), half ? (float*)(base + h.rg[c]) : nullptr, nullptr};
+  r.fd = lbpc::PopBuf<S>{(S*)(base + h.f[d]), half ? (float*)(base + h.rf[d]) : nullptr, (double*)(base + h.wall[d])};
+  r.gd = lbpc::PopBuf<S>{(S*)(base + h.g[d]), half ? (float*)(base + h.rg[d]) : nullptr, nullptr};
+  r.phi_prev = base + h.phi;
+  r.scalars = (double*)(base + h.scalars);
+  r.partials = (double*)(base + h.partials);
+  r.status = (long long*)(b->base + b->status_off) + 8 * k;
+  r.step = (const long long*)(b->base + b->insts_off + (size_t)k * b->inst_struct + offsetof(lbpc::BatchInst<S>, step));
+  r.tiles_x = (h.dp.nx + tx - 1) / tx;
+  r.first = h.step + rel == 0;
+}
+
+// One launch over the n instances of ids, the `launch`-th of its step: L is a SegLaunch or a WalkLaunch.
+template <class S, class L> std::unique_ptr<L> make_launch(const lbpc_batch* b, const int* ids, int n, int rel, int launch) {
+  std::unique_ptr<L> l(new L());
+  memset((void*)l.get(), 0, sizeof(L));
+  l->waits = launch == 0;
+  for (int j = 0; j < n; ++j) {
+    l->first_tile[j] = l->tiles;
+    fill_seg<S>(b, ids[j], rel, l->in[j]);
+    l->tiles += (int)tiles_of(b, b->inst[ids[j]]);
+  }
+  l->n = n;
+  return l;
+}
+template <class S, int CAP> cudaError_t send_tiles(lbpc_batch* b, const int* ids, int n, int rel, int launch) {
+  auto l = make_launch<S, lbpc::SegLaunch<S, CAP>>(b, ids, n, rel, launch);
+  return lbpc::batch_seg_launch(b->prec, b->variant, CAP == lbpc::kSegSmall, l.get(), b->stream);
+}
+template <class S, int CAP> cudaError_t send_walk(lbpc_batch* b, const int* ids, int n, int rel, int launch) {
+  auto l = make_launch<S, lbpc::WalkLaunch<S, CAP>>(b, ids, n, rel, launch);
+  for (int j = 0; j < n; ++j) {
+    const HostInst& h = b->inst[ids[j]];
+    if (!h.staged) continue;
+    const lbpc::TmaMaps& m = h.maps[h.cur ^ rel];
+    l->mapped |= 1ull << j;
+    l->maps[j].f = m.f;
+    l->maps[j].g = m.g;
+    if constexpr (lbpc::is_half_t<S>::value) {
+      l->maps[j].rf = m.rf;
+      l->maps[j].rg = m.rg;
+    }
+  }
+  return lbpc::batch_walk_launch(b->prec, CAP == lbpc::kSegSmall, l.get(), tickets(b, launch), b->stream);
+}
+
+// One step as per-tile launches (ctas == 0): the active instances in launches of as many as the form holds, walked
+// where that is the faster form for the next ones, then the per-instance advance. Whether the step is
 // an instance's first comes from the host's count (h.step + rel), so lbpc_batch_step takes the first
 // step of new instances outside the captured graphs.
 template <class S> cudaError_t seg_step(lbpc_batch* b, int rel) {
-  constexpr int CAP = lbpc::seg_capacity<S>(), SMALL = lbpc::kSegSmall;
-  int tx, ty;
-  lbpc::batch_tile_shape(b->variant, tx, ty);
-  std::unique_ptr<lbpc::SegLaunch<S, CAP>> L(new lbpc::SegLaunch<S, CAP>());
-  std::unique_ptr<lbpc::SegLaunch<S, SMALL>> Ls(new lbpc::SegLaunch<S, SMALL>());
-  memset(L.get(), 0, sizeof(lbpc::SegLaunch<S, CAP>));
-  int launches = 0;
-  auto flush = [&]() -> cudaError_t {
-    if (L->n == 0) return cudaSuccess;
-    cudaError_t e;
-    L->waits = launches == 0;
-    if (L->n <= SMALL) {  // the same records in the kernel with smaller parameters
-      memset(Ls.get(), 0, sizeof(lbpc::SegLaunch<S, SMALL>));
-      Ls->n = L->n;
-      Ls->tiles = L->tiles;
-      Ls->staged = L->staged;
-      Ls->waits = launches == 0;
-      for (int j = 0; j < L->n; ++j) {
-        Ls->first_tile[j] = L->first_tile[j];
-        Ls->in[j] = L->in[j];
+  constexpr int SMALL = lbpc::kSegSmall, CAP = lbpc::seg_capacity<S>();
+  std::vector<int> ids;
+  for (int k = 0; k < (int)b->inst.size(); ++k)
+    if (b->inst[k].used) ids.push_back(k);
+  cudaError_t e = cudaSuccess;
+  for (int at = 0, launch = 0; at < (int)ids.size() && e == cudaSuccess; ++launch) {
+    const int left = (int)ids.size() - at, *p = ids.data() + at;
+    if constexpr (!std::is_same<S, double>::value) {
+      constexpr int WALK = lbpc::walk_capacity<S>();
+      const int n = std::min(left, WALK);
+      long long tiles = 0, staged = 0, s = 0;
+      for (int j = 0; j < n; ++j) {
+        tiles += tiles_of(b, b->inst[p[j]], &s);
+        staged += s;
       }
-      e = lbpc::batch_seg_launch(b->prec, b->variant, true, Ls.get(), tickets(b, launches), b->stream);
-    } else {
-      e = lbpc::batch_seg_launch(b->prec, b->variant, false, L.get(), tickets(b, launches), b->stream);
+      bool walk = false;
+      if (b->variant == 0 && (e = lbpc::batch_walk_wanted(b->prec, n <= SMALL, tiles, staged, &walk)) != cudaSuccess) break;
+      if (walk) {
+        e = n <= SMALL ? send_walk<S, SMALL>(b, p, n, rel, launch) : send_walk<S, WALK>(b, p, n, rel, launch);
+        at += n;
+        continue;
+      }
     }
-    ++launches;
-    L->n = 0;
-    L->tiles = 0;
-    L->staged = 0;
-    return e;
-  };
-  for (int k = 0; k < (int)b->inst.size(); ++k) {
-    const HostInst& h = b->inst[k];
-    if (!h.used) continue;
-    if (L->n == CAP) {
-      const cudaError_t e = flush();
-      if (e != cudaSuccess) return e;
-    }
-    L->first_tile[L->n] = L->tiles;
-    lbpc::SegInst<S>& r = L->in[L->n++];
-    char* base = b->base + h.off;
-    const int c = h.cur ^ rel, d = c ^ 1;
-    const bool half = b->prec == LBPC_FP16DEV;
-    r.P = lbpc::params_of<typename lbpc::ArithOf<S>::type>(h.dp);
-    r.fs = lbpc::PopBuf<S>{(S*)(base + h.f[c]), half ? (float*)(base + h.rf[c]) : nullptr, (double*)(base + h.wall[c])};
-    r.gs = lbpc::PopBuf<S>{(S*)(base + h.g[c]), half ? (float*)(base + h.rg[c]) : nullptr, nullptr};
-    r.fd = lbpc::PopBuf<S>{(S*)(base + h.f[d]), half ? (float*)(base + h.rf[d]) : nullptr, (double*)(base + h.wall[d])};
-    r.gd = lbpc::PopBuf<S>{(S*)(base + h.g[d]), half ? (float*)(base + h.rg[d]) : nullptr, nullptr};
-    r.phi_prev = base + h.phi;
-    r.scalars = (double*)(base + h.scalars);
-    r.partials = (double*)(base + h.partials);
-    r.status = (long long*)(b->base + b->status_off) + 8 * k;
-    if constexpr (!std::is_same<S, double>::value)
-      r.maps = h.staged ? (const lbpc::TmaMaps*)(base + h.maps) + c : nullptr;
-    r.step = (const long long*)(b->base + b->insts_off + (size_t)k * b->inst_struct + offsetof(lbpc::BatchInst<S>, step));
-    r.tiles_x = (h.dp.nx + tx - 1) / tx;
-    r.first = h.step + rel == 0;
-    L->tiles += r.tiles_x * ((h.dp.ny + ty - 1) / ty);
-    if (h.staged && tx == 32 && ty == 8)  // interior tiles: 3 nodes from every edge
-      L->staged += std::max(0, (h.dp.nx - 35) / 32) * std::max(0, (h.dp.ny - 11) / 8);
+    const int n = std::min(left, CAP);
+    e = n <= SMALL ? send_tiles<S, SMALL>(b, p, n, rel, launch) : send_tiles<S, CAP>(b, p, n, rel, launch);
+    at += n;
   }
-  const cudaError_t e = flush();
   if (e != cudaSuccess) return e;
   return lbpc::batch_advance_launch(b->prec, b->base + b->insts_off, (int)b->inst.size(), b->stream);
 }
@@ -543,13 +574,9 @@ LBPC_API lbpc_status lbpc_batch_add(lbpc_batch* b, const lbpc_params* p, const d
   hi.step = 0;
   hi.staged = false;
   if (store_bytes(b->prec) <= 4) {
-    lbpc::TmaMaps maps[2] = {};
     hi.staged = true;
     for (int k = 0; k < 2; ++k)
-      hi.staged &= lbpc::fused_tma_encode(&maps[k], b->prec, 1, s.f[k], s.g[k], s.ref_f[k], s.ref_g[k], hi.dp);
-    // pageable source: the copy is staged before the call returns
-    BCU(b, cudaMemcpyAsync(b->base + hi.off + hi.maps, maps, sizeof maps, cudaMemcpyHostToDevice, b->stream),
-        "lbpc_batch_add tensor maps");
+      hi.staged &= lbpc::fused_tma_encode(&hi.maps[k], b->prec, 1, s.f[k], s.g[k], s.ref_f[k], s.ref_g[k], hi.dp);
   }
   b->dirty = true;
   lbpc_status r = rebuild(b);

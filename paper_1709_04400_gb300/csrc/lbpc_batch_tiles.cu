@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
 // tile being worked on is broadcast from one lane, which lets the compiler keep its parameters in uniform registers.
 template <class S, class R, int TX, int TY, int CAP>
 __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
-    k_batch_walk(const __grid_constant__ SegLaunch<S, CAP> L, unsigned long long* __restrict__ tickets) {
+    k_batch_walk(const __grid_constant__ WalkLaunch<S, CAP> L, unsigned long long* __restrict__ tickets) {
   using B = TmaBox<S, TX, TY>;
   constexpr int NTH = TX * TY;
   if (L.waits) pdl_wait<NTH>();  // every address below depends on shared memory written after it
@@ -65,7 +65,6 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
   };
   __shared__ Tile s_tile[2], s_next;
   __shared__ unsigned s_raw;  // number of the next tile
-  __shared__ int s_mapped;    // thread 0's: the instance whose tensor maps it acquired last
   extern __shared__ __align__(128) unsigned char dyn[];
   uint64_t* bar = (uint64_t*)(dyn + B::BYTES - 128);
   auto tile_at = [&](unsigned b) {
@@ -84,22 +83,13 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
   auto staged = [&](const Tile& t) {
     if (t.k < 0) return false;
     const SegInst<S>& I = L.in[t.k];
-    return I.maps && t.x >= 3 && t.x + TX + 3 <= I.P.nx && t.y >= 3 && t.y + TY + 3 <= I.P.ny;
-  };
-  auto stage = [&](const Tile& t) {  // thread 0 starts the copy of a staged tile
-    const TmaMaps* maps = L.in[t.k].maps;
-    if (s_mapped != t.k) {  // tiles come in order, so once per instance
-      acquire_maps<S>(maps);
-      s_mapped = t.k;
-    }
-    tma_issue_tile<S, TX, TY>(dyn, bar, *maps, t.x, t.y);
+    return ((L.mapped >> t.k) & 1) && t.x >= 3 && t.x + TX + 3 <= I.P.nx && t.y >= 3 && t.y + TY + 3 <= I.P.ny;
   };
   auto take = [&]() { return (unsigned)(gridDim.x + atomicAdd(tickets, 1ull)); };
   if (threadIdx.x == 0) {
     mbar_init(bar, 1);
-    s_mapped = -1;
     const Tile t0 = tile_at(blockIdx.x);
-    if (staged(t0)) stage(t0);
+    if (staged(t0)) tma_issue_tile<S, TX, TY>(dyn, bar, L.maps[t0.k], t0.x, t0.y);
     s_tile[0] = t0;
     s_raw = take();
   }
@@ -114,7 +104,7 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
     auto start_next = [&]() {
       if (threadIdx.x != 0) return;
       const Tile next = s_next;
-      if (staged(next)) stage(next);
+      if (staged(next)) tma_issue_tile<S, TX, TY>(dyn, bar, L.maps[next.k], next.x, next.y);
     };
     const int k = __shfl_sync(0xffffffffu, tile.k, 0);
     const int x0 = __shfl_sync(0xffffffffu, tile.x, 0), y0 = __shfl_sync(0xffffffffu, tile.y, 0);
@@ -147,10 +137,9 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
   if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <class S, class R, int CAP>
-static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, cudaStream_t st, bool* done) {
+// CTAs of the walk that fit on the device at once.
+template <class S, class R, int CAP> static cudaError_t walk_resident(int* out) {
   using B = TmaBox<S, 32, 8>;
-  const SegLaunch<S, CAP>& L = *(const SegLaunch<S, CAP>*)Lh;
   auto* kernel = k_batch_walk<S, R, 32, 8, CAP>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, B::BYTES);
   if (e != cudaSuccess) return e;
@@ -158,25 +147,45 @@ static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, cu
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 256, B::BYTES)) != cudaSuccess) return e;
-  const int resident = sms * (occ > 0 ? occ : 1);  // CTAs of the walk that fit on the device at once
-  // Where the walk is the faster form: enough tiles per CTA, as for one instance, and enough of them staged (an edge
-  // tile's own pulls leave the CTA's next copy waiting). FP32, per-tile launch against walk, instances of one size:
-  // 256^2 (70 % staged) 161, 165 us; 512^2 (85 %) 147, 131; 64 of 64^2 to 512^2 (74 %) 236, 230. FP16: 128^2 (44 %) 274,
-  // 298; 256^2 223, 217; 512^2 196, 166.
+  *out = sms * (occ > 0 ? occ : 1);
+  return cudaSuccess;
+}
+
+// Where the walk is the faster form: enough tiles per CTA, as for one instance, and enough of them staged (an edge
+// tile's own pulls leave the CTA's next copy waiting). FP32, per-tile launch against walk, instances of one size:
+// 256^2 (70 % staged) 161, 165 us; 512^2 (85 %) 147, 131; 64 of 64^2 to 512^2 (74 %) 236, 230. FP16: 128^2 (44 %) 274,
+// 298; 256^2 223, 217; 512^2 196, 166.
+template <class S, class R, int CAP> static cudaError_t walk_wanted_c(long long tiles, long long staged, bool* yes) {
   constexpr bool kHalf = is_half_t<S>::value;
-  *done = (long long)L.tiles > (kHalf ? 12LL : 5LL) * resident && 100LL * L.staged >= (kHalf ? 60LL : 72LL) * L.tiles;
-  if (!*done) return cudaSuccess;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)resident);
-  cfg.blockDim = dim3(256);
-  cfg.dynamicSmemBytes = B::BYTES;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, L, tickets);
+  int resident = 0;
+  const cudaError_t e = walk_resident<S, R, CAP>(&resident);
+  if (e != cudaSuccess) return e;
+  *yes = tiles > (kHalf ? 12LL : 5LL) * resident && 100LL * staged >= (kHalf ? 60LL : 72LL) * tiles;
+  return cudaSuccess;
+}
+cudaError_t batch_walk_wanted(int prec, bool small, long long tiles, long long staged, bool* yes) {
+  if (prec == 1)
+    return small ? walk_wanted_c<float, float, kSegSmall>(tiles, staged, yes)
+                 : walk_wanted_c<float, float, walk_capacity<float>()>(tiles, staged, yes);
+  return small ? walk_wanted_c<__half, float, kSegSmall>(tiles, staged, yes)
+               : walk_wanted_c<__half, float, walk_capacity<__half>()>(tiles, staged, yes);
+}
+
+template <class S, class R, int CAP>
+static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, cudaStream_t st) {
+  using B = TmaBox<S, 32, 8>;
+  const WalkLaunch<S, CAP>& L = *(const WalkLaunch<S, CAP>*)Lh;
+  int resident = 0;
+  const cudaError_t e = walk_resident<S, R, CAP>(&resident);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(k_batch_walk<S, R, 32, 8, CAP>, resident, 256, B::BYTES, st, L, tickets);
+}
+cudaError_t batch_walk_launch(int prec, bool small, const void* L, unsigned long long* tickets, cudaStream_t st) {
+  if (prec == 1)
+    return small ? walk_launch_c<float, float, kSegSmall>(L, tickets, st)
+                 : walk_launch_c<float, float, walk_capacity<float>()>(L, tickets, st);
+  return small ? walk_launch_c<__half, float, kSegSmall>(L, tickets, st)
+               : walk_launch_c<__half, float, walk_capacity<__half>()>(L, tickets, st);
 }
 
 template <class S, class R, int TX, int TY, int NPT, int CAP>
@@ -214,18 +223,7 @@ static cudaError_t seg_launch_p(int variant, bool small, const void* L, cudaStre
                : seg_launch_c<S, R, seg_capacity<S>()>(variant, L, st);
 }
 
-cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, cudaStream_t st) {
-  if (variant == 0 && (prec == 1 || prec == 2)) {
-    bool done = false;
-    cudaError_t e;
-    if (prec == 1)
-      e = small ? walk_launch_c<float, float, kSegSmall>(L, tickets, st, &done)
-                : walk_launch_c<float, float, seg_capacity<float>()>(L, tickets, st, &done);
-    else
-      e = small ? walk_launch_c<__half, float, kSegSmall>(L, tickets, st, &done)
-                : walk_launch_c<__half, float, seg_capacity<__half>()>(L, tickets, st, &done);
-    if (e != cudaSuccess || done) return e;
-  }
+cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, cudaStream_t st) {
   if (prec == 0) return seg_launch_p<double, double>(variant, small, L, st);
   if (prec == 1) return seg_launch_p<float, float>(variant, small, L, st);
   return seg_launch_p<__half, float>(variant, small, L, st);

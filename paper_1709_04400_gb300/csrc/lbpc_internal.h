@@ -57,7 +57,13 @@ template <class S, int TX, int TY> struct TmaBox {
 struct alignas(64) TmaMaps {
   CUtensorMap f, g, rf, rg;  // current buffer's populations (3D) and FP16 reference planes (2D)
 };
-
+// Those that a storage type has, for parameters that hold many.
+template <class S> struct alignas(64) TmaMapsOf {
+  CUtensorMap f, g;
+};
+template <> struct alignas(64) TmaMapsOf<__half> {
+  CUtensorMap f, g, rf, rg;
+};
 
 // Most tiles a fused or batched step launches over an nx x ny domain (the 32 x 8 tile, the smallest
 // shape). A step with the domain-mean buoyancy writes one partial sum per tile, so the partials array
@@ -157,11 +163,7 @@ cudaError_t batch_step_launch(int prec, int variant, int ctas, const BatchMeta* 
 // such launches over the active instances (up to seg_capacity each), then the per-instance advance.
 template <class S> struct ArithOf { using type = float; };  // arithmetic of a storage type in a batch
 template <> struct ArithOf<double> { using type = double; };
-template <class S> struct SegMaps {
-  const TmaMaps* maps;       // tensor maps of the source buffers (device memory), or null
-};
-template <> struct SegMaps<double> {};  // binary64 batches are not staged
-template <class S> struct alignas(16) SegInst : SegMaps<S> {
+template <class S> struct alignas(16) SegInst {
   DevParamsOf<typename ArithOf<S>::type> P;  // header and the one coefficient set the kernel reads
   PopBuf<S> fs, gs, fd, gd;  // this launch's source and destination populations
   void* phi_prev;            // arithmetic type
@@ -181,9 +183,9 @@ template <class S> constexpr int seg_capacity() {
 constexpr int kSegSmall = 16;
 template <class S, int CAP> struct SegLaunch {
   int n;      // instances of this launch
-  int tiles;  // its tiles
-  int staged; // those of them that tensor copies can stage
+  int tiles;  // its CTAs
   int waits;  // the first launch of its step: waits for the step before it
+  int pad_;
   int first_tile[CAP];  // each instance's first CTA, ascending: kept together so that the search of a
                         // CTA's instance reads a few cache lines
   SegInst<S> in[CAP];
@@ -193,9 +195,34 @@ static_assert(sizeof(SegLaunch<double, seg_capacity<double>()>) <= kSegParamByte
               "per-tile launch parameters");
 // Enqueue one per-tile launch over the instances of L, a host SegLaunch<S, CAP> of the batch's storage
 // type with CAP = kSegSmall (small) or seg_capacity<S>(). Unless L waits, the launch may begin while the previous
-// kernel on st drains (its instances are others). tickets: two zeroed words of this launch's own in device memory,
-// left zero.
-cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, unsigned long long* tickets, cudaStream_t st);
+// kernel on st drains (its instances are others).
+cudaError_t batch_seg_launch(int prec, int variant, bool small, const void* L, cudaStream_t st);
+
+// The same launch walked by persistent CTAs (4- and 2-byte storage, 32 x 8 tiles). The tensor maps of the source
+// buffers travel in the parameters beside their instances, which so many fewer fit. Maps in device memory would have to
+// be acquired by each block that uses them, with a system-scope proxy fence per instance: the tiles a block takes are
+// of ever other instances, and 64 uneven FP32 instances took 71.2 ms per 256 steps that way.
+template <class S, int CAP> struct WalkLaunch {
+  int n;      // instances of this launch
+  int tiles;  // its tiles
+  int waits;  // the first launch of its step: waits for the step before it
+  int pad_;
+  unsigned long long mapped;  // bit k: instance k has tensor maps
+  int first_tile[CAP];
+  SegInst<S> in[CAP];
+  TmaMapsOf<S> maps[CAP];
+};
+template <class S> constexpr int walk_capacity() {
+  return (int)((kSegParamBytes - 128) / (sizeof(SegInst<S>) + sizeof(TmaMapsOf<S>) + sizeof(int))) & ~3;
+}
+static_assert(sizeof(WalkLaunch<float, walk_capacity<float>()>) <= kSegParamBytes &&
+                  sizeof(WalkLaunch<__half, walk_capacity<__half>()>) <= kSegParamBytes && walk_capacity<float>() <= 64,
+              "walk launch parameters");
+// Whether a launch of that many tiles, `staged` of which tensor copies can stage, is faster walked.
+cudaError_t batch_walk_wanted(int prec, bool small, long long tiles, long long staged, bool* yes);
+// Enqueue it; L: a host WalkLaunch<S, CAP>, CAP = kSegSmall (small) or walk_capacity<S>(). tickets: two zeroed words of
+// this launch's own in device memory, left zero.
+cudaError_t batch_walk_launch(int prec, bool small, const void* L, unsigned long long* tickets, cudaStream_t st);
 // Enqueue the per-instance advance of a step (rho_ave, buffer parity, step count).
 cudaError_t batch_advance_launch(int prec, void* d_insts, int ninst, cudaStream_t st);
 // Largest resident CTAs per SM of the step kernel for (prec, variant).

@@ -117,26 +117,10 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* tm, in
       : "memory");
 }
 
-// Make tensor maps in device memory that a copy from the host wrote there usable by this block's tensor copies. The
-// copies read descriptors through a proxy of their own, which nothing but this fence brings up to date: the memory may
-// have held another instance's maps before. Maps passed as kernel parameters need none. By the thread that starts the
-// copies, before its first one from these maps in a launch; the scope is the system's because the host wrote them.
-template <class S> __device__ __forceinline__ void acquire_maps(const TmaMaps* m) {
-  static_assert(sizeof(CUtensorMap) == 128, "the fence covers 128 bytes");
-  auto acquire = [](const CUtensorMap* t) {
-    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(t) : "memory");
-  };
-  acquire(&m->f);
-  acquire(&m->g);
-  if (is_half_t<S>::value) {
-    acquire(&m->rf);
-    acquire(&m->rg);
-  }
-}
-
-// Start the copy of a tile's populations (and FP16 reference planes) into its box, by one thread.
-template <class S, int TX, int TY>
-__device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar, const TmaMaps& maps, int x0, int y0) {
+// Start the copy of a tile's populations (and FP16 reference planes) into its box, by one thread. maps: kernel
+// parameters.
+template <class S, int TX, int TY, class M>
+__device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar, const M& maps, int x0, int y0) {
   using B = TmaBox<S, TX, TY>;
   // the box was last read through the generic proxy (stage 1, before a block barrier); order those
   // reads before the copy engine's writes
@@ -144,7 +128,7 @@ __device__ __forceinline__ void tma_issue_tile(unsigned char* dyn, uint64_t* bar
   mbar_expect_tx(bar, (unsigned)(18 * B::BX * B::BY * sizeof(S) + (B::HALF ? 2 * B::REFX * B::BY * 4 : 0)));
   tma_load_3d(dyn, &maps.f, x0 - B::XOFF, y0 - 3, 0, bar);
   tma_load_3d(dyn + B::SET, &maps.g, x0 - B::XOFF, y0 - 3, 0, bar);
-  if (B::HALF) {
+  if constexpr (B::HALF) {
     tma_load_2d(dyn + 2 * B::SET, &maps.rf, x0 - B::XOFF, y0 - 3, bar);
     tma_load_2d(dyn + 2 * B::SET + B::RPLANE, &maps.rg, x0 - B::XOFF, y0 - 3, bar);
   }
