@@ -389,6 +389,16 @@ __host__ __device__ __forceinline__ long long wall_doubles(int nx) { return 4LL 
 template <class S> struct is_half_t { static constexpr bool value = false; };
 template <> struct is_half_t<__half> { static constexpr bool value = true; };
 
+// P.pitch as the index arithmetic of a storage type takes it. A product of signed 32-bit numbers cannot overflow by the
+// language's rules, so the compiler widens a row's nine sources to 64-bit addresses early; unsigned ones stay 32-bit
+// until they are used. The FP16 tiles, which hold a reference's address beside each population's, are short of
+// registers and take the unsigned form: 12 FP16 instances of 60^2 to 77^2 13.97 us a step signed, 10.8 unsigned; 24 of
+// 64^2 to 512^2 119, 110. FP32 is better off with the wide addresses (4096^2 421 us, 434 unsigned; small ones alike).
+template <class S, class PT> __device__ __forceinline__ auto pitch_of(const PT& P) {
+  if constexpr (is_half_t<S>::value) return (unsigned)P.pitch;
+  else return P.pitch;
+}
+
 // double(x) from the bits, exact for every x (NaN stays NaN): a conversion instruction runs at the FP64 pipe's rate,
 // a seventieth of the integer and binary32 ones. A subnormal is scaled into the normal numbers first. A dozen
 // instructions more per value in flight, so it pays where the FP64 pipe and not latency sets the time (launch_sums).
@@ -488,7 +498,7 @@ __device__ __forceinline__ void pull_from(const PopBuf<S>& src, const R* w, cons
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
     const int r = s.row[EY(a) + 1];
-    v[a] = r >= 0 ? pop_load<S, R, IX, BITS>(src, (IX)P.N, a, (IX)r * P.pitch + s.col[EX(a) + 1], w) : R(0);
+    v[a] = r >= 0 ? pop_load<S, R, IX, BITS>(src, (IX)P.N, a, (IX)r * pitch_of<S>(P) + s.col[EX(a) + 1], w) : R(0);
   }
 }
 

@@ -32,8 +32,8 @@ __device__ __forceinline__ int wrap_any(int x, int n) {
 }
 
 // Post-stream populations of an interior node (no wrap, no closure): src[a][i - e_a].
-template <class S, class R, class IX = long long>
-__device__ __forceinline__ void pull_interior(const PopBuf<S>& src, const R* w, IX N, int pitch, IX i, R v[9]) {
+template <class S, class R, class IX = long long, class PI>
+__device__ __forceinline__ void pull_interior(const PopBuf<S>& src, const R* w, IX N, PI pitch, IX i, R v[9]) {
 #pragma unroll
   for (int a = 0; a < 9; ++a) v[a] = pop_load<S, R, IX>(src, N, a, i - (IX)EY(a) * pitch - EX(a), w);
 }
@@ -44,11 +44,11 @@ template <class S, class R, class IX, class PT>
 __device__ __forceinline__ void pull_columns(const PopBuf<S>& fsrc, const PopBuf<S>& gsrc, const PT& P, int x, int y, R f[9],
                                              R g[9]) {
   const Coefs<R>& C = coefs<R>(P);
-  const IX row = (IX)y * P.pitch;
+  const IX row = (IX)y * pitch_of<S>(P);
   const IX at[3] = {row + (x == P.nx - 1 ? 0 : x + 1), row + x, row + (x == 0 ? P.nx - 1 : x - 1)};  // e_x = -1, 0, 1
 #pragma unroll
   for (int a = 0; a < 9; ++a) {
-    const IX i = at[EX(a) + 1] - (IX)EY(a) * P.pitch;
+    const IX i = at[EX(a) + 1] - (IX)EY(a) * pitch_of<S>(P);
     f[a] = pop_load<S, R, IX>(fsrc, (IX)P.N, a, i, C.wf);
     g[a] = pop_load<S, R, IX>(gsrc, (IX)P.N, a, i, C.wg);
   }
@@ -272,9 +272,9 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     const int gx = x0 + tx, gy = y0 + ty;
     active[k] = INTERIOR || (gx < P.nx && (ROWS || gy < P.ny));
     if constexpr (IDX32)
-      pp[k] = (active[k] && P.model == 0 && !first) ? __ldg(phi_prev + ((IX)gy * P.pitch + gx)) : R(0);
+      pp[k] = (active[k] && P.model == 0 && !first) ? __ldg(phi_prev + ((IX)gy * pitch_of<S>(P) + gx)) : R(0);
     else
-      pp[k] = (active[k] && P.model == 0 && !first) ? phi_prev[(long long)gy * P.pitch + gx] : R(0);
+      pp[k] = (active[k] && P.model == 0 && !first) ? phi_prev[(long long)gy * pitch_of<S>(P) + gx] : R(0);
     const int mx = wrap_any(gx, P.nx);
     my[k] = ROWS ? gy : row_of(P, gy);
     if (MODE == 2) {
@@ -283,9 +283,9 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     } else if (MODE == 4) {
       pull_columns<S, R, IX>(fsrc, gsrc, P, mx, gy, f[k], g[k]);
     } else if (INTERIOR) {
-      const IX io = (IX)gy * P.pitch + gx;
-      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.pitch, io, f[k]);
-      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, P.pitch, io, g[k]);
+      const IX io = (IX)gy * pitch_of<S>(P) + gx;
+      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, pitch_of<S>(P), io, f[k]);
+      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, pitch_of<S>(P), io, g[k]);
     } else {
       pull_closed<S, R, IX>(fsrc, gsrc, P, mx, my[k], f[k], g[k]);
     }
@@ -335,9 +335,9 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
     } else if (MODE == 4) {
       pull_columns<S, R, IX>(fsrc, gsrc, P, wrap_any(x0 + hx - 2, P.nx), y0 + hy - 2, fr, gr);
     } else if (INTERIOR) {
-      const IX io = (IX)(y0 + hy - 2) * P.pitch + (x0 + hx - 2);
-      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, P.pitch, io, fr);
-      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, P.pitch, io, gr);
+      const IX io = (IX)(y0 + hy - 2) * pitch_of<S>(P) + (x0 + hx - 2);
+      pull_interior<S, R, IX>(fsrc, C.wf, (IX)P.N, pitch_of<S>(P), io, fr);
+      pull_interior<S, R, IX>(gsrc, C.wg, (IX)P.N, pitch_of<S>(P), io, gr);
     } else {
       const int x = wrap_any(x0 + hx - 2, P.nx), y = row_of(P, y0 + hy - 2);
       pull_closed<S, R, IX>(fsrc, gsrc, P, x, y, fr, gr);
@@ -474,7 +474,7 @@ __device__ __forceinline__ void fused_body(int t, const PopBuf<S>& fsrc, const P
                     (s_rho[hy + 1][hx + 1] + s_rho[hy + 1][hx - 1] - s_rho[hy - 1][hx - 1] - s_rho[hy - 1][hx + 1]) * R(1.0 / 12.0);
       div_lam_gradT = rcv * C.chi * lapT + C.cV_chi * (grx * gTx + gry * gTy);
     }
-    const IX i = (IX)gy * P.pitch + gx;
+    const IX i = (IX)gy * pitch_of<S>(P) + gx;
     const R compress = Tk * (R(1) - dpdT[k] * inv_rcv) * divv;
     R phi, S0, tau_inv = R(0);
     if (P.model == 2) {  // Gong-Cheng: Eq. 13 source, local tau_g (Sec. IV A)
