@@ -14,7 +14,7 @@ ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "liblbpc.so")
 SOURCES = ["lbpc_api.cu", "lbpc_split.cu", "lbpc_fused.cu", "lbpc_batch_kernels.cu", "lbpc_batch_tiles.cu", "lbpc_batch.cu",
            "lbpc_static.cu", "lbpc_probe.cu"]
-HEADERS = ["lbpc_device.cuh", "lbpc_dw.cuh", "lbpc_tile.cuh", "lbpc_internal.h"]
+HEADERS = ["lbpc_device.cuh", "lbpc_dw.cuh", "lbpc_tile.cuh", "lbpc_internal.h", "lbpc_sums_target.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

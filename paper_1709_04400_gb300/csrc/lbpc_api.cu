@@ -7,9 +7,11 @@
 #include <string.h>
 
 #include <cuda_runtime.h>
+#include <cudaTypedefs.h>
 
 #include "../../include/lbpc.h"
 #include "lbpc_internal.h"
+#include "lbpc_sums_target.h"
 
 #define LBPC_API extern "C" __attribute__((visibility("default")))
 
@@ -742,18 +744,25 @@ LBPC_API lbpc_status lbpc_sums(lbpc_ctx* c, double* mass, double* heat) {
   return LBPC_OK;
 }
 
-// The address under which the reduction kernel can write the caller's two doubles itself (memory of the context's
-// device, or pinned host memory mapped for it), or null where a copy is needed. A copy of 16 bytes costs a monitored
-// step its two ordinary stream dependencies besides (binary64 256^2, step and sums: 63 us with it, 53 without).
-static double* device_writable(lbpc_ctx* c, double* out) {
-  cudaPointerAttributes at{};
-  if (((uintptr_t)out & 7) != 0 || cudaPointerGetAttributes(&at, out) != cudaSuccess) {
-    cudaGetLastError();
-    return nullptr;
-  }
-  if (at.type == cudaMemoryTypeDevice && at.device == c->device) return out;
-  if (at.type == cudaMemoryTypeHost) return (double*)at.devicePointer;
+static PFN_cuPointerGetAttribute_v4000 query_pointer_fn() {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &p, 4000, cudaEnableDefault, &q) == cudaSuccess &&
+      q == cudaDriverEntryPointSuccess)
+    return (PFN_cuPointerGetAttribute_v4000)p;
   return nullptr;
+}
+
+static lbpc::AddressInfo address_info(const void* p) {
+  static const PFN_cuPointerGetAttribute_v4000 fn = query_pointer_fn();
+  lbpc::AddressInfo a{};
+  if (cudaPointerGetAttributes(&a.at, p) != cudaSuccess) {
+    cudaGetLastError();
+    a.at = cudaPointerAttributes{};
+  } else if (!fn || fn(&a.access, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) {
+    a.access = 0;
+  }
+  return a;
 }
 
 LBPC_API lbpc_status lbpc_sums_async(lbpc_ctx* c, double* out, int on_device) {
@@ -761,7 +770,9 @@ LBPC_API lbpc_status lbpc_sums_async(lbpc_ctx* c, double* out, int on_device) {
   if (!c || !out) return LBPC_EINVAL;
   if (!c->initialised) return LBPC_ESTATE;
   DeviceGuard g(c->device);
-  double* direct = device_writable(c, out);
+  // A copy of 16 bytes costs a monitored step its two ordinary stream dependencies besides (binary64 256^2, step and
+  // sums: 63 us with it, 53 without), so the reduction writes the caller's memory where it can.
+  double* direct = lbpc::sums_target(out, on_device != 0, c->device, address_info(out), address_info((char*)out + 15));
   CU(c, lbpc::split_sums(c->buf, c->dp, c->p.prec, c->cur, c->stream, direct), "lbpc_sums_async kernels");
   if (!direct)
     CU(c, cudaMemcpyAsync(out, c->buf.scalars + 1, 2 * sizeof(double),
