@@ -255,8 +255,8 @@ def _dtypes():
 # the entry describes another build and the line reports null.
 MEASURED_TRAFFIC = {
     # one-pass ncu captures (dram__bytes_read.sum + dram__bytes_write.sum) of the bench's own commands
-    ("k_collide", "droplet_evaporation_2048_dT0.1Tc", "fp64"): (1_113_285_888, "06556f317e36c813"),
-    ("k_collide", "droplet_evaporation_2048_dT0.1Tc", "df64"): (1_113_380_608, "06556f317e36c813"),
+    ("k_collide_tile", "droplet_evaporation_2048_dT0.1Tc", "fp64"): (1_113_285_888, "06556f317e36c813"),
+    ("k_collide_tile", "droplet_evaporation_2048_dT0.1Tc", "df64"): (1_113_380_608, "06556f317e36c813"),
     ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp32"): (2_511_768_320, "06556f317e36c813"),
     ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp16"): (1_581_142_016, "06556f317e36c813"),
     ("k_batch_walk", "batched_evaporation_256", "fp32"): (3_968_465_920, "06556f317e36c813"),  # one step: 5 launches
@@ -537,15 +537,16 @@ def run_native(args):
            "frac_of_nominal": hbm_step / NOMINAL_HBM_GBS, "of": "whole step", "peak_source": bw_src}
 
     # dominant kernel and its roofline
-    if prec == lbpc.FP64 and "k_collide" in avg:
+    collide = "k_collide_tile" if "k_collide_tile" in avg else "k_collide"  # 8-byte storage, 4- and 2-byte storage
+    if prec == lbpc.FP64 and collide in avg:
         # the binary64 step is bound by the FP64 pipe: its denominator is the FMA rate of this GPU,
         # measured here by a probe kernel, with the clocks seen while it ran
         with ClockSampler(local) as pclk:
             fma64 = lbpc.fma_rate(lbpc.FP64, sim.stream) / 1e12
         fpn = collide_flops(case["lambda_mode"], all(v == 1.0 for v in case["s_g"][1:]))
-        achieved = fpn * N / (avg["k_collide"] / 1e3) / 1e12
-        roof = {"bound": "alu", "kernel": "k_collide", "achieved": achieved, "peak": fma64, "unit": "TFLOP/s",
-                "frac": achieved / fma64, "traffic": measured_traffic("k_collide", case["name"], prec_name),
+        achieved = fpn * N / (avg[collide] / 1e3) / 1e12
+        roof = {"bound": "alu", "kernel": collide, "achieved": achieved, "peak": fma64, "unit": "TFLOP/s",
+                "frac": achieved / fma64, "traffic": measured_traffic(collide, case["name"], prec_name),
                 "peak_source": "binary64 FMA rate measured in this run (lbpc_fma_rate: 8 independent FMA chains per "
                                "thread on every SM)", "probe_clocks": pclk.summary(),
                 "flops_per_node": fpn, "top_kernel": top, "hbm": hbm}
@@ -557,9 +558,9 @@ def run_native(args):
                 "bytes_per_node": bpn, "top_kernel": top, "hbm": hbm}
     else:
         cb = collide_bytes_per_node(pb)
-        achieved = cb * N / (avg["k_collide"] / 1e3) / 1e9
-        roof = {"bound": "hbm", "kernel": "k_collide", "achieved": achieved, "peak": peak_bw, "unit": "GB/s",
-                "frac": achieved / peak_bw, "traffic": measured_traffic("k_collide", case["name"], prec_name),
+        achieved = cb * N / (avg[collide] / 1e3) / 1e9
+        roof = {"bound": "hbm", "kernel": collide, "achieved": achieved, "peak": peak_bw, "unit": "GB/s",
+                "frac": achieved / peak_bw, "traffic": measured_traffic(collide, case["name"], prec_name),
                 "peak_source": bw_src, "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
                 "bytes_per_node": cb, "top_kernel": top, "hbm": hbm}
 

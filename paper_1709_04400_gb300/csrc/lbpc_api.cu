@@ -465,11 +465,11 @@ static cudaError_t launch_step(lbpc_ctx* c, cudaEvent_t* ev) {
 }
 
 static int step_kernel_count(const lbpc_ctx* c) {
-  return use_fused(c) ? 1 : lbpc::split_kernel_count(c->dp, c->p.prec);
+  return use_fused(c) ? lbpc::fused_kernel_count(c->buf, c->dp, c->p.prec, c->cur) : lbpc::split_kernel_count(c->dp, c->p.prec);
 }
 
 static const char* step_kernel_name(const lbpc_ctx* c, int k) {
-  if (use_fused(c)) return k == 0 ? "k_fused" : "";
+  if (use_fused(c)) return k == 0 ? "k_fused" : "k_finish";
   return lbpc::split_kernel_name(c->p.prec, k);
 }
 

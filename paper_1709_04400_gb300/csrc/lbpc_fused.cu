@@ -191,6 +191,17 @@ static cudaError_t loop_residency(int smem, int* out) {
   return cudaSuccess;
 }
 
+// Whether a step's interior tiles are staged by tensor copies.
+// FP32 grids of less than one tile per resident CTA pull straight from L2: nothing is left to overlap the staging
+// with (256^2 5.5 us against 6.2, 150 x 300 9.1 against 9.4; 300 x 400 7.9 against 7.7). FP16 is staged at every size.
+static bool takes_staging(const SplitBuffers& b, const DevParams& P, int prec, int cur) {
+  return (prec == 1 || prec == 2) && b.tma[cur] && (prec == 2 || P.N >= 100000);
+}
+
+int fused_kernel_count(const SplitBuffers& b, const DevParams& P, int prec, int cur) {
+  return P.buoyancy == 1 && takes_staging(b, P, prec, cur) ? 2 : 1;
+}
+
 // ------------------------------------------------------------------------------------------------
 template <class S, class R, int TX, int TY, int NPT = 1, bool LOOP = false>
 static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur, long long step, cudaStream_t st,
@@ -202,9 +213,7 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
   if (ev) cudaEventRecord(ev[0], st);
   bool staged = false;
   if constexpr (sizeof(S) <= 4) {  // the TMA-staged kernel exists for FP32 and FP16 storage
-    // FP32 grids of less than one tile per resident CTA pull straight from L2: nothing is left to overlap the staging
-    // with (256^2 5.5 us against 6.2, 150 x 300 9.1 against 9.4; 300 x 400 7.9 against 7.7). FP16 is staged at every size.
-    if (b.tma[cur] && (is_half_t<S>::value || P.N >= 100000)) {
+    if (takes_staging(b, P, is_half_t<S>::value ? 2 : 1, cur)) {
       using B = TmaBox<S, TX, TY>;
       // The dynamic shared-memory limit is held per device context, so it is set before every launch:
       // the call is cheap, thread-safe, and right after a device reset or on a second device.
@@ -236,7 +245,10 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
           return e;
       }
       // the mean as a kernel of its own: its code in the staged kernels costs every step of theirs 2 to 5 %
-      if (P.buoyancy == 1) fused_finish(b, P, (int)(grid.x * grid.y), st);
+      if (P.buoyancy == 1) {
+        if (ev) cudaEventRecord(ev[1], st);
+        fused_finish(b, P, (int)(grid.x * grid.y), st);
+      }
       staged = true;
     }
   }
@@ -245,7 +257,7 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
                                      P, step, step == 0, mean, b.partials, b.status);
     if (e != cudaSuccess) return e;
   }
-  if (ev) cudaEventRecord(ev[1], st);
+  if (ev) cudaEventRecord(ev[staged && P.buoyancy == 1 ? 2 : 1], st);
   return cudaGetLastError();
 }
 

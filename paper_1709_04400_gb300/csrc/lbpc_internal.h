@@ -228,7 +228,10 @@ cudaError_t batch_advance_launch(int prec, void* d_insts, int ninst, cudaStream_
 // Largest resident CTAs per SM of the step kernel for (prec, variant).
 int batch_max_ctas_per_sm(int prec, int variant);
 
-// Fused single-kernel step (lbpc_fused.cu); same buffers, no scratch planes touched.
+// Fused single-kernel step (lbpc_fused.cu); same buffers, no scratch planes touched. ev: null, or fused_kernel_count + 1
+// events as for split_step. The count is 2 where a staged step (tensor copies) with the domain-mean buoyancy leaves the
+// mean to a kernel of its own.
+int fused_kernel_count(const SplitBuffers& b, const DevParams& P, int prec, int cur);
 cudaError_t fused_step(const SplitBuffers& b, const DevParams& P, int prec, int cur, long long step, cudaStream_t st,
                        cudaEvent_t* ev = nullptr);
 // Encode the tensor maps of one buffer (populations f, g and, for FP16, the reference planes) for the

@@ -678,7 +678,7 @@ int split_kernel_count(const DevParams& P, int prec) { return (is_wide(prec) ? 2
 
 const char* split_kernel_name(int prec, int k) {
   static const char* names[] = {"k_macro", "k_force", "k_collide", "k_finish"};
-  static const char* wide[] = {"k_macro", "k_collide", "k_finish"};
+  static const char* wide[] = {"k_macro", "k_collide_tile", "k_finish"};
   if (k < 0 || k >= (is_wide(prec) ? 3 : 4)) return "";
   return is_wide(prec) ? wide[k] : names[k];
 }
