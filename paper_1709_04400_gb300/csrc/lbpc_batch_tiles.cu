@@ -137,18 +137,9 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
   if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// CTAs of the walk that fit on the device at once.
 template <class S, class R, int CAP> static cudaError_t walk_resident(int* out) {
-  using B = TmaBox<S, 32, 8>;
-  auto* kernel = k_batch_walk<S, R, 32, 8, CAP>;
-  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, B::BYTES);
-  if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0, occ = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, 256, B::BYTES)) != cudaSuccess) return e;
-  *out = sms * (occ > 0 ? occ : 1);
-  return cudaSuccess;
+  static Residency cache;
+  return resident_ctas(cache, k_batch_walk<S, R, 32, 8, CAP>, 256, TmaBox<S, 32, 8>::BYTES, out);
 }
 
 // Where the walk is the faster form: enough tiles per CTA, as for one instance, and enough of them staged (an edge
@@ -176,7 +167,9 @@ static cudaError_t walk_launch_c(const void* Lh, unsigned long long* tickets, cu
   using B = TmaBox<S, 32, 8>;
   const WalkLaunch<S, CAP>& L = *(const WalkLaunch<S, CAP>*)Lh;
   int resident = 0;
-  const cudaError_t e = walk_resident<S, R, CAP>(&resident);
+  cudaError_t e = walk_resident<S, R, CAP>(&resident);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_batch_walk<S, R, 32, 8, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, B::BYTES);
   if (e != cudaSuccess) return e;
   return launch_pdl(k_batch_walk<S, R, 32, 8, CAP>, resident, 256, B::BYTES, st, L, tickets);
 }

@@ -4,7 +4,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "lbpc_tile.cuh"
 
@@ -171,24 +170,9 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
     atomicExch(tickets, 0ull);
 }
 
-// Resident CTAs of the persistent kernel on the current device (SMs x CTAs per SM), queried once per
-// device: the value cannot change while the process runs, so two first calls racing only store the
-// same number twice. The dynamic shared-memory attribute is set before the query.
-template <class S, class R, int TX, int TY, int NPT>
-static cudaError_t loop_residency(int smem, int* out) {
-  static std::atomic<int> cache[64];
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev >= 0 && dev < 64 && (*out = cache[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
-  int sms = 0, occ = 0;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_fused_tma_loop<S, R, TX, TY, NPT>, TX * TY / NPT,
-                                                         (size_t)smem)) != cudaSuccess)
-    return e;
-  *out = std::max(occ, 1) * sms;
-  if (dev >= 0 && dev < 64) cache[dev].store(*out, std::memory_order_relaxed);
-  return cudaSuccess;
+template <class S, class R, int TX, int TY, int NPT> static cudaError_t loop_residency(int smem, int* out) {
+  static Residency cache;
+  return resident_ctas(cache, k_fused_tma_loop<S, R, TX, TY, NPT>, TX * TY / NPT, smem, out);
 }
 
 // Whether a step's interior tiles are staged by tensor copies.

@@ -4,6 +4,8 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include <nvtx3/nvToolsExt.h>
 
 #include "lbpc_device.cuh"
@@ -39,6 +41,26 @@ inline cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// CTAs of a kernel that fit on the current device at once, queried once per device: the value cannot change while the
+// process runs, so two first calls racing only store the same number twice. The dynamic shared-memory limit is set
+// before the query; launches set it themselves (it is held per device context).
+struct Residency {
+  std::atomic<int> of[64];
+};
+template <class K> inline cudaError_t resident_ctas(Residency& cache, K* kernel, int threads, int smem, int* out) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev >= 0 && dev < 64 && (*out = cache.of[dev].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+  int sms = 0, occ = 0;
+  if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, threads, (size_t)smem)) != cudaSuccess) return e;
+  *out = (occ > 0 ? occ : 1) * sms;
+  if (dev >= 0 && dev < 64) cache.of[dev].store(*out, std::memory_order_relaxed);
+  return cudaSuccess;
 }
 
 template <class S, int TX, int TY> struct TmaBox {
