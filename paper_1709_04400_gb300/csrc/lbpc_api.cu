@@ -561,7 +561,9 @@ LBPC_API lbpc_status lbpc_step_timed(lbpc_ctx* c, float* kernel_ms, int32_t max_
 }
 
 LBPC_API const char* lbpc_kernel_name(const lbpc_ctx* c, int32_t k) {
-  if (!c || k < 0 || k >= step_kernel_count(c)) return "";
+  if (!c || k < 0) return "";
+  DeviceGuard g(c->device);
+  if (k >= step_kernel_count(c)) return "";
   return step_kernel_name(c, k);
 }
 

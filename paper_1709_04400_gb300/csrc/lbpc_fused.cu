@@ -175,15 +175,29 @@ template <class S, class R, int TX, int TY, int NPT> static cudaError_t loop_res
   return resident_ctas(cache, k_fused_tma_loop<S, R, TX, TY, NPT>, TX * TY / NPT, smem, out);
 }
 
-// Whether a step's interior tiles are staged by tensor copies.
-// FP32 grids of less than one tile per resident CTA pull straight from L2: nothing is left to overlap the staging
-// with (256^2 5.5 us against 6.2, 150 x 300 9.1 against 9.4; 300 x 400 7.9 against 7.7). FP16 is staged at every size.
-static bool takes_staging(const SplitBuffers& b, const DevParams& P, int prec, int cur) {
-  return (prec == 1 || prec == 2) && b.tma[cur] && (prec == 2 || P.N >= 100000);
-}
-
-int fused_kernel_count(const SplitBuffers& b, const DevParams& P, int prec, int cur) {
-  return P.buoyancy == 1 && takes_staging(b, P, prec, cur) ? 2 : 1;
+// Whether a step's interior tiles are staged by tensor copies: wherever the buffers have tensor maps, but for small FP32
+// grids of 32 x 8 tiles, which pull straight from L2 (below three tiles per four resident CTAs a copy has nothing to
+// overlap with; with the domain-mean buoyancy the unstaged step also takes the mean in its last block, a launch less, and
+// stays ahead up to two tiles per CTA). us a step, unstaged and staged, 608 resident CTAs: 224^2 (196 tiles) 5.3,
+// 5.6; 288 x 352 (396) 6.57, 6.83; 320^2 (400) 6.25, 6.21; 352^2 (484) 7.24, 7.00; 384 x 400 (600) 7.37, 7.05; 512^2 (1024)
+// 11.5, 11.4. Closed pools with the mean: 150 x 300 (190) 8.5, 9.1; 384 x 400 11.0, 11.5; 512^2 16.7, 17.6; 640 x 512 (1280)
+// 20.9, 20.7. The other tile shapes do not differ by more than a few per cent either way, nor does FP16.
+template <class S, class R, int TX, int TY, int NPT>
+static cudaError_t takes_staging(const SplitBuffers& b, const DevParams& P, int cur, bool* yes) {
+  *yes = false;
+  if constexpr (sizeof(S) <= 4) {  // the staged kernels exist for FP32 and FP16 storage
+    *yes = b.tma[cur] != nullptr;
+    if (*yes && !is_half_t<S>::value && TX * TY == 32 * 8) {
+      static Residency cache;
+      int resident = 0;
+      const cudaError_t e =
+          resident_ctas(cache, k_fused_tma<S, R, TX, TY, NPT>, TX * TY / NPT, TmaBox<S, TX, TY>::BYTES, &resident);
+      if (e != cudaSuccess) return e;
+      const long long tiles = (long long)((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY);
+      *yes = 4 * tiles >= (P.buoyancy == 1 ? 8LL : 3LL) * resident;
+    }
+  }
+  return cudaSuccess;
 }
 
 // ------------------------------------------------------------------------------------------------
@@ -196,8 +210,12 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
   const MeanOf mean{b.scalars, (unsigned*)(b.status + 5), grid.x * grid.y, 1.0 / node_count(P)};
   if (ev) cudaEventRecord(ev[0], st);
   bool staged = false;
-  if constexpr (sizeof(S) <= 4) {  // the TMA-staged kernel exists for FP32 and FP16 storage
-    if (takes_staging(b, P, is_half_t<S>::value ? 2 : 1, cur)) {
+  {
+    const cudaError_t e = takes_staging<S, R, TX, TY, NPT>(b, P, cur, &staged);
+    if (e != cudaSuccess) return e;
+  }
+  if constexpr (sizeof(S) <= 4) {
+    if (staged) {
       using B = TmaBox<S, TX, TY>;
       // The dynamic shared-memory limit is held per device context, so it is set before every launch:
       // the call is cheap, thread-safe, and right after a device reset or on a second device.
@@ -233,7 +251,6 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
         if (ev) cudaEventRecord(ev[1], st);
         fused_finish(b, P, (int)(grid.x * grid.y), st);
       }
-      staged = true;
     }
   }
   if (!staged) {
@@ -308,17 +325,41 @@ bool fused_tma_encode(TmaMaps* m, int prec, int tile, void* f, void* g, float* r
 
 // Tile configurations of the FP32 / FP16 fused step: 0 = 32x16, 1 = 32x8, 2 = 32x16 with 2 nodes per
 // thread, 3 = 32x32 with 2 nodes per thread, 4 = 32x8 in persistent CTAs that start each next tile's copy
-// early.
+// early. f is called with the shape.
+template <int TX_, int TY_, int NPT_, bool LOOP_ = false> struct Shape {
+  static constexpr int TX = TX_, TY = TY_, NPT = NPT_;
+  static constexpr bool LOOP = LOOP_;
+};
+template <class F> static cudaError_t with_shape(int fused_tile, F f) {
+  switch (fused_tile) {
+    case 1: return f(Shape<32, 8, 1>());
+    case 2: return f(Shape<32, 16, 2>());
+    case 3: return f(Shape<32, 32, 2>());
+    case 4: return f(Shape<32, 8, 1, true>());
+    default: return f(Shape<32, 16, 1>());
+  }
+}
 template <class S, class R>
 static cudaError_t fused_tiles(const SplitBuffers& b, const DevParams& P, int cur, long long step, cudaStream_t st,
                                cudaEvent_t* ev) {
-  switch (b.fused_tile) {
-    case 1: return fused_impl<S, R, 32, 8, 1>(b, P, cur, step, st, ev);
-    case 2: return fused_impl<S, R, 32, 16, 2>(b, P, cur, step, st, ev);
-    case 3: return fused_impl<S, R, 32, 32, 2>(b, P, cur, step, st, ev);
-    case 4: return fused_impl<S, R, 32, 8, 1, true>(b, P, cur, step, st, ev);
-    default: return fused_impl<S, R, 32, 16, 1>(b, P, cur, step, st, ev);
-  }
+  return with_shape(b.fused_tile, [&](auto s) {
+    using T = decltype(s);
+    return fused_impl<S, R, T::TX, T::TY, T::NPT, T::LOOP>(b, P, cur, step, st, ev);
+  });
+}
+template <class S> static int kernel_count(const SplitBuffers& b, const DevParams& P, int cur) {
+  bool staged = false;
+  with_shape(b.fused_tile, [&](auto s) {
+    using T = decltype(s);
+    return takes_staging<S, float, T::TX, T::TY, T::NPT>(b, P, cur, &staged);
+  });
+  return P.buoyancy == 1 && staged ? 2 : 1;
+}
+
+int fused_kernel_count(const SplitBuffers& b, const DevParams& P, int prec, int cur) {
+  if (prec == 1) return kernel_count<float>(b, P, cur);
+  if (prec == 2) return kernel_count<__half>(b, P, cur);
+  return 1;
 }
 
 cudaError_t fused_step(const SplitBuffers& b, const DevParams& P, int prec, int cur, long long step, cudaStream_t st,

@@ -44,3 +44,35 @@ def test_each_kernel_of_a_step_is_timed(prec, path, n, mean, want):
         got = sim.step_timed()
         assert list(got) == want and all(v > 0.0 for v in got.values())
     sim.close()
+
+
+# FP32 grids of 32 x 8 tiles are staged by tensor copies from 3/4 of a tile per resident CTA on (four CTAs per SM), with
+# the domain-mean buoyancy from two tiles: the grids of 320 and 640 columns on either side of each line.
+@pytest.mark.parametrize("mean,nx,per_sm", [(False, 320, 3), (True, 640, 8)], ids=["plain", "mean"])
+def test_fp32_steps_on_both_sides_of_the_staging_line(mean, nx, per_sm):
+    """The binary32 step against the binary64 one: 30 steps, the parity tests' 1e-4 (u against its largest value)."""
+    import torch
+
+    from .helpers import max_rel, norm_rel
+
+    line = per_sm * torch.cuda.get_device_properties(0).multi_processor_count  # tiles
+    rows = [(line - 1) // (nx // 32) * 8, -(-line // (nx // 32)) * 8]
+    assert rows[0] // 8 * (nx // 32) < line <= rows[1] // 8 * (nx // 32)
+    for ny, names in zip(rows, (["k_fused"], ["k_fused", "k_finish"] if mean else ["k_fused"])):
+        if mean:
+            case, rho, T = workloads.mixed_small(TC, RV, RL, nx=nx, ny=ny)
+        else:
+            case, rho, T = workloads.droplet_evaporation(TC, RV, RL, n=max(nx, ny), radius=60.0, dT_ratio=0.1)
+            case, rho, T = dict(case, nx=nx, ny=ny), rho[:ny, :nx].copy(), T[:ny, :nx].copy()
+        out = []
+        for prec in (lbpc.FP32, lbpc.FP64):
+            sim = lbpc.Simulation(lbpc.params_from_case(case, prec))
+            sim.init(rho, T)
+            sim.step(29)
+            got = sim.step_timed()
+            assert prec == lbpc.FP64 or list(got) == names
+            out.append(sim.fields())
+            sim.close()
+        a, b = out
+        assert max_rel(a[0], b[0]) <= 1e-4 and max_rel(a[3], b[3]) <= 1e-4
+        assert norm_rel(a[1], b[1]) <= 1e-4 and norm_rel(a[2], b[2]) <= 1e-4
