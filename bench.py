@@ -387,7 +387,7 @@ def batch_measure(lbpc, workloads, prec, instances, steps, warmup, variant=-1, c
         clk.__exit__(None, None, None)
     b.check()
     batch_s = ev0.elapsed_time(ev1) / 1e3
-    cfg = b.config()
+    cfg, names = b.config(), b.kernel_names()
     b.close()
     sims = []
     for p, (c, r, t) in zip(params, insts):
@@ -410,12 +410,8 @@ def batch_measure(lbpc, workloads, prec, instances, steps, warmup, variant=-1, c
     value = nodes * steps / batch_s / 1e6
     plain = nodes * steps / plain_s / 1e6
     peak_bw = _peak_hbm()
-    # per-tile launches (0 CTAs per SM): ceil(instances / capacity) launches and the advance per step;
-    # the work-list kernel: one launch and the advance
     per_tile = cfg["ctas_per_sm"] == 0
-    # per-tile launches of this many tiles are walked by persistent CTAs; smaller ones run k_batch_tiles
-    kernel = "k_batch_walk" if per_tile else "k_batch_step"
-    launches_per_step = (-(-len(insts) // lbpc.Batch.per_tile_capacity(prec)) + 1) if per_tile else 2
+    kernel = "+".join(dict.fromkeys(n for n in names if n != "k_batch_advance"))
     bpn = storage_bytes_per_node(prec, lbpc)
     achieved = bpn * nodes / (batch_s / steps) / 1e9
     prec_name = {lbpc.FP64: "fp64", lbpc.FP32: "fp32", lbpc.FP16DEV: "fp16"}[prec]
@@ -432,7 +428,7 @@ def batch_measure(lbpc, workloads, prec, instances, steps, warmup, variant=-1, c
                 "traffic": measured_traffic(kernel, wname, prec_name),
                 "traffic_per": "step (every launch of the step)" if per_tile else "launch"},
         "l2": "working set of %.1f GB exceeds L2" % (nodes * bpn / 1e9),
-        "launches": launches_per_step * steps, "clocks": clk.summary() if clk else None,
+        "launches": len(names) * steps, "clocks": clk.summary() if clk else None,
     }
 
 

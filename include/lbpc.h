@@ -259,7 +259,8 @@ void lbpc_destroy(lbpc_ctx* c);
  * Batches: many independent simulations of uneven size advancing together.
  *
  * The per-node arithmetic is the fused step's. A step is a few per-tile launches (one CTA per tile, or
- * persistent CTAs that walk a launch of many tiles), each holding up to lbpc_batch_per_tile_capacity instances in its kernel parameters (the default),
+ * persistent CTAs that walk a launch of many tiles), each holding up to lbpc_batch_per_tile_capacity instances in its kernel
+ * parameters, a walked one fewer, with their tensor maps (the default),
  * or one launch whose CTAs walk a device-resident work list of (instance, tile) entries (see
  * lbpc_batch_set_config). Steps are replayed through captured CUDA graphs in chunks when the batch
  * has a non-default stream. Instances can join and leave between calls. Their parameters,
@@ -311,7 +312,7 @@ int64_t lbpc_batch_step_count(const lbpc_batch* b, int32_t id);
  * resident (a persistent grid). Above it, up to 64 times that limit, further CTAs start as earlier
  * ones finish, so the hardware balances tiles of uneven cost. A value above that returns LBPC_EINVAL.
  * ctas_per_sm = 0: per-tile launches. A step is a sequence of launches with one CTA per tile (variant 0 in
- * 4- and 2-byte storage: persistent CTAs where a launch has many tiles, most of them interior), each over
+ * 4- and 2-byte storage: persistent CTAs where a launch has many tiles, three in four of them interior), each over
  * up to lbpc_batch_per_tile_capacity instances held in its kernel parameters; each launch may start
  * while the previous one drains. A change of instances then captures the step graphs again.
  * A negative value returns LBPC_EINVAL. */
@@ -332,6 +333,8 @@ lbpc_status lbpc_batch_autotune(lbpc_batch* b, int32_t steps_per_candidate, int3
                                 float* best_ms_per_step);
 
 /* Free bytes left in the arena, the last error message, and teardown (the arena stays the caller's). */
+/* Name of the k-th kernel that a step launches with the present instances and configuration ("" past the last). */
+const char* lbpc_batch_kernel_name(const lbpc_batch* b, int32_t k);
 size_t lbpc_batch_free_bytes(const lbpc_batch* b);
 const char* lbpc_batch_last_error(const lbpc_batch* b);
 void lbpc_batch_destroy(lbpc_batch* b);

@@ -369,40 +369,64 @@ template <class S, int CAP> cudaError_t send_walk(lbpc_batch* b, const int* ids,
   return lbpc::batch_walk_launch(b->prec, CAP == lbpc::kSegSmall, l.get(), tickets(b, launch), b->stream);
 }
 
-// One step as per-tile launches (ctas == 0): the active instances in launches of as many as the form holds, walked
-// where that is the faster form for the next ones, then the per-instance advance. Whether the step is
-// an instance's first comes from the host's count (h.step + rel), so lbpc_batch_step takes the first
-// step of new instances outside the captured graphs.
-template <class S> cudaError_t seg_step(lbpc_batch* b, int rel) {
-  constexpr int SMALL = lbpc::kSegSmall, CAP = lbpc::seg_capacity<S>();
+// The launches of a step as per-tile launches (ctas == 0): the active instances in launches of as many as the form holds,
+// walked where that is the faster form for the next ones. f is called with each: walk, the instances, their number, its
+// index.
+template <class S, class F> cudaError_t plan_step(const lbpc_batch* b, F f) {
   std::vector<int> ids;
   for (int k = 0; k < (int)b->inst.size(); ++k)
     if (b->inst[k].used) ids.push_back(k);
   cudaError_t e = cudaSuccess;
   for (int at = 0, launch = 0; at < (int)ids.size() && e == cudaSuccess; ++launch) {
     const int left = (int)ids.size() - at, *p = ids.data() + at;
+    int n = std::min(left, lbpc::seg_capacity<S>());
+    bool walk = false;
     if constexpr (!std::is_same<S, double>::value) {
-      constexpr int WALK = lbpc::walk_capacity<S>();
-      const int n = std::min(left, WALK);
+      const int m = std::min(left, lbpc::walk_capacity<S>());
       long long tiles = 0, staged = 0, s = 0;
-      for (int j = 0; j < n; ++j) {
+      for (int j = 0; j < m; ++j) {
         tiles += tiles_of(b, b->inst[p[j]], &s);
         staged += s;
       }
-      bool walk = false;
-      if (b->variant == 0 && (e = lbpc::batch_walk_wanted(b->prec, n <= SMALL, tiles, staged, &walk)) != cudaSuccess) break;
-      if (walk) {
-        e = n <= SMALL ? send_walk<S, SMALL>(b, p, n, rel, launch) : send_walk<S, WALK>(b, p, n, rel, launch);
-        at += n;
-        continue;
-      }
+      if (b->variant == 0 && (e = lbpc::batch_walk_wanted(b->prec, m <= lbpc::kSegSmall, tiles, staged, &walk)) != cudaSuccess)
+        break;
+      if (walk) n = m;
     }
-    const int n = std::min(left, CAP);
-    e = n <= SMALL ? send_tiles<S, SMALL>(b, p, n, rel, launch) : send_tiles<S, CAP>(b, p, n, rel, launch);
+    e = f(walk, p, n, launch);
     at += n;
   }
+  return e;
+}
+
+// One such step, then the per-instance advance. Whether the step is
+// an instance's first comes from the host's count (h.step + rel), so lbpc_batch_step takes the first
+// step of new instances outside the captured graphs.
+template <class S> cudaError_t seg_step(lbpc_batch* b, int rel) {
+  constexpr int SMALL = lbpc::kSegSmall;
+  const cudaError_t e = plan_step<S>(b, [&](bool walk, const int* p, int n, int launch) {
+    if constexpr (!std::is_same<S, double>::value)
+      if (walk) return n <= SMALL ? send_walk<S, SMALL>(b, p, n, rel, launch)
+                                  : send_walk<S, lbpc::walk_capacity<S>()>(b, p, n, rel, launch);
+    return n <= SMALL ? send_tiles<S, SMALL>(b, p, n, rel, launch)
+                      : send_tiles<S, lbpc::seg_capacity<S>()>(b, p, n, rel, launch);
+  });
   if (e != cudaSuccess) return e;
   return lbpc::batch_advance_launch(b->prec, b->base + b->insts_off, (int)b->inst.size(), b->stream);
+}
+
+// Names of a step's launches, in order.
+std::vector<const char*> step_names(const lbpc_batch* b) {
+  std::vector<const char*> names;
+  auto add = [&](bool walk, const int*, int, int) {
+    names.push_back(walk ? "k_batch_walk" : "k_batch_tiles");
+    return cudaSuccess;
+  };
+  if (b->ctas > 0) names.push_back("k_batch_step");
+  else if (b->prec == LBPC_FP64) plan_step<double>(b, add);
+  else if (b->prec == LBPC_FP32) plan_step<float>(b, add);
+  else plan_step<__half>(b, add);
+  if (!b->inst.empty()) names.push_back("k_batch_advance");
+  return names;
 }
 
 // One step of the current configuration; rel: parity of this step relative to the instances' h.cur.
@@ -776,6 +800,13 @@ LBPC_API int32_t lbpc_batch_per_tile_capacity(int32_t prec) {
   if (prec == LBPC_FP32) return lbpc::seg_capacity<float>();
   if (prec == LBPC_FP16DEV) return lbpc::seg_capacity<__half>();
   return 0;
+}
+
+LBPC_API const char* lbpc_batch_kernel_name(const lbpc_batch* b, int32_t k) {
+  if (!b || k < 0) return "";
+  DevGuard g(b->device);
+  const std::vector<const char*> names = step_names(b);
+  return k < (int)names.size() ? names[k] : "";
 }
 
 LBPC_API size_t lbpc_batch_free_bytes(const lbpc_batch* b) { return b ? b->arena.free_bytes() : 0; }

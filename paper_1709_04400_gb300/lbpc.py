@@ -32,7 +32,7 @@ EXPORTED = ["lbpc_version", "lbpc_check_params", "lbpc_workspace_bytes", "lbpc_e
             "lbpc_kernel_name", "lbpc_set_path", "lbpc_step_static", "lbpc_batch_instance_bytes", "lbpc_batch_create",
             "lbpc_batch_add", "lbpc_batch_remove", "lbpc_batch_step", "lbpc_batch_check", "lbpc_batch_fields",
             "lbpc_batch_sums", "lbpc_batch_step_count", "lbpc_batch_set_config", "lbpc_batch_config",
-            "lbpc_batch_autotune", "lbpc_batch_free_bytes", "lbpc_batch_last_error", "lbpc_batch_destroy",
+            "lbpc_batch_autotune", "lbpc_batch_kernel_name", "lbpc_batch_free_bytes", "lbpc_batch_last_error", "lbpc_batch_destroy",
             "lbpc_set_fused_tile", "lbpc_checkpoint_bytes", "lbpc_save", "lbpc_load", "lbpc_fma_rate",
             "lbpc_batch_per_tile_capacity"]
 
@@ -115,6 +115,7 @@ def load_library(path: str = LIB_PATH):
         "lbpc_batch_autotune": (ctypes.c_int, [vp, ctypes.c_int32, ctypes.POINTER(ctypes.c_int32),
                                                ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_float)]),
         "lbpc_batch_per_tile_capacity": (ctypes.c_int32, [ctypes.c_int32]),
+        "lbpc_batch_kernel_name": (ctypes.c_char_p, [vp, ctypes.c_int32]),
         "lbpc_batch_free_bytes": (ctypes.c_size_t, [vp]),
         "lbpc_batch_last_error": (ctypes.c_char_p, [vp]),
         "lbpc_batch_destroy": (None, [vp]),
@@ -500,6 +501,13 @@ class Batch:
         self._raise(self.lib.lbpc_batch_autotune(self.h, int(steps_per_candidate), ctypes.byref(bv), ctypes.byref(bc),
                                                  ctypes.byref(ms)), "lbpc_batch_autotune")
         return dict(variant=bv.value, ctas_per_sm=bc.value, ms_per_step=ms.value)
+
+    def kernel_names(self):
+        """Names of the kernels that a step launches with the present instances and configuration, in order."""
+        out = []
+        while name := self.lib.lbpc_batch_kernel_name(self.h, len(out)).decode():
+            out.append(name)
+        return out
 
     def free_bytes(self) -> int:
         return int(self.lib.lbpc_batch_free_bytes(self.h))

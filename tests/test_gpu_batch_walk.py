@@ -1,5 +1,5 @@
 """Batches walked by persistent CTAs, against the same instances in forms that are not walked: an instance in the
-block that another one of other sizes has left."""
+block that another one of other sizes has left, and a step of which a second launch is a walk too."""
 
 import numpy as np
 import pytest
@@ -61,3 +61,21 @@ def test_instance_in_a_freed_block(prec):
     for got, want in zip(b.fields(i), _alone(prec, second, 18)):
         assert np.array_equal(got, want)
     b.close()
+
+
+def test_kernel_names_are_those_launched():
+    """lbpc_batch_kernel_name tells the forms apart: the benchmark names and counts a step's launches by it."""
+    large = [workloads.droplet_evaporation(TC, RV, RL, n=1021, radius=200.0, dT_ratio=d) for d in (0.1, 0.2)]
+    small = [workloads.mixed_small(TC, RV, RL, nx=37, ny=29)]
+    b, _ = _batch(lbpc.FP32, large)
+    assert b.kernel_names() == ["k_batch_walk", "k_batch_advance"]
+    b.set_config(3, 0)
+    assert b.kernel_names() == ["k_batch_tiles", "k_batch_advance"]
+    b.set_config(0, 4)
+    assert b.kernel_names() == ["k_batch_step", "k_batch_advance"]
+    b.close()
+    for prec in (lbpc.FP64, lbpc.FP32, lbpc.FP16DEV):
+        n = lbpc.Batch.per_tile_capacity(prec) + 1
+        b, _ = _batch(prec, small * n)
+        assert b.kernel_names() == ["k_batch_tiles"] * 2 + ["k_batch_advance"]
+        b.close()
