@@ -79,3 +79,27 @@ def test_kernel_names_are_those_launched():
         b, _ = _batch(prec, small * n)
         assert b.kernel_names() == ["k_batch_tiles"] * 2 + ["k_batch_advance"]
         b.close()
+
+
+@PRECS
+def test_second_launch_is_walked(prec):
+    """More instances than a walk holds: the second walk starts while the first one ends and takes its own tickets.
+    Each kind of instance equals, first, middle and last, its run alone by one CTA per tile; 20 steps are one by itself,
+    a captured chunk of 16, and three more."""
+    large = workloads.droplet_evaporation(TC, RV, RL, n=511, radius=100.0, dT_ratio=0.1)
+    kinds = [large, workloads.mixed_small(TC, RV, RL, nx=37, ny=29), workloads.droplet_periodic(TC, RV, RL, n=97, radius=20.0)]
+    cases = kinds * 24  # 24 x (1,024 + 8 + 52) tiles
+    b, ids = _batch(prec, cases)
+    assert b.kernel_names()[:2] == ["k_batch_walk"] * 2
+    b.step(20)
+    b.check()
+    for k, kind in enumerate(kinds):
+        one, (i,) = _batch(prec, [kind])
+        assert one.kernel_names() == ["k_batch_tiles", "k_batch_advance"]
+        one.step(20)
+        want = one.fields(i)
+        one.close()
+        for j in (k, 36 + k, 69 + k):
+            for got, w in zip(b.fields(ids[j]), want):
+                assert np.array_equal(got, w), (kind[0]["name"], j)
+    b.close()
