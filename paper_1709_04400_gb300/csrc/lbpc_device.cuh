@@ -229,10 +229,6 @@ template <class R, class PT> __device__ __forceinline__ void eos(R rho, R T, con
   dpdT = rho * C.R_gas * inv1 - C.a * dtheta * r2 * inv2;
 }
 
-// The same for binary64 and double-word arithmetic, arranged for the fewest operations (their step is bound by
-// the arithmetic pipe): psi^2, (dp/dT)_rho and 1/rho from one reciprocal and one reciprocal square root.
-// With u = rho R / (1 - b rho), A = a rho^2 / (1 + 2 b rho - b^2 rho^2) and h = 1 + kappa (1 - sqrt(T/T_c)):
-// p = u T - A h^2 and dp/dT = u + A h kappa / sqrt(T T_c).
 template <> __device__ __forceinline__ dw inverse_of<dw>(dw x) {  // binary32 reciprocal, corrected once
   x = dw_norm(x);
   const float r = __frcp_rn(x.hi);
@@ -240,11 +236,14 @@ template <> __device__ __forceinline__ dw inverse_of<dw>(dw x) {  // binary32 re
   const float d = __fsub_rn(__fsub_rn(__fsub_rn(1.0f, p.hi), p.lo), __fmul_rn(r, x.lo));  // 1 - r x
   return dw_fast_two_sum(r, __fmul_rn(d, r));
 }
-// Binary64 reciprocal and roots from the hardware's approximations (relative error below 2^-20) by one step
-// of the third-order iteration (Householder 1970; for the reciprocal, r (1 + e + e^2) with e = 1 - x r): the
-// error left is of the order of e^3, below binary64's rounding. 3 and 5 operations of the pipe that bounds the
-// step; the compiler's correctly rounded forms take more. Arguments are normal numbers here (a state outside
-// the equation of state's range is reported by classify, whatever these return for it).
+// Binary64 reciprocal and roots from the hardware's approximations, which see and give the upper 32 bits of a number,
+// by one step of the third-order iteration (Householder 1970; for the reciprocal, r (1 + e + e^2) with
+// e = 1 - x r). |e| is at most 2^-18 by those two truncations (over 2^-1000 to 2^1000 measured 2^-19.98 for the reciprocal,
+// 2^-19.06 for the root's 1 - x y^2), so the step leaves e^3 <= 2^-54, or 5/16 of that for the roots, of a last place of 2^-53
+// or more. With the roundings 1/x is within 1 ulp (measured 0.501), sqrt(x) within 1 (0.744) and 1/sqrt(x) within 1.25
+// (0.922); CUDA states 0.5, 0.5 and 1 for its own, which take more than these 3 and 5 operations of the pipe that bounds
+// the step. Arguments are normal numbers here (a state outside the equation of state's range is reported by classify,
+// whatever these return for it).
 template <> __device__ __forceinline__ double inverse_of<double>(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
@@ -278,6 +277,10 @@ template <> __device__ __forceinline__ double psi_of<double>(double psi2) {
   roots_of(psi2, inv_root, root);
   return b >= 0x0010000000000000LL && b < 0x7ff0000000000000LL ? root : (b == 0x7ff0000000000000LL ? psi2 : 0.0);
 }
+// eos and psi^2 for binary64 and double-word arithmetic, arranged for the fewest operations (their step is bound by
+// the arithmetic pipe): psi^2, (dp/dT)_rho and 1/rho from one reciprocal and one reciprocal square root.
+// With u = rho R / (1 - b rho), A = a rho^2 / (1 + 2 b rho - b^2 rho^2) and h = 1 + kappa (1 - sqrt(T/T_c)):
+// p = u T - A h^2 and dp/dT = u + A h kappa / sqrt(T T_c).
 template <class R, class PT>
 __device__ __forceinline__ R eos_psi_squared(R rho, R T, const PT& P, R& dpdT, R& inv_rho) {
   const Coefs<R>& C = coefs<R>(P);
