@@ -184,14 +184,13 @@ template <class R> __device__ __forceinline__ void from_moments_conserving(const
 // Reciprocal and roots. Binary32 takes the hardware's approximations without the compiler's handling of
 // subnormal and huge arguments (a test, a select and two products each, about 4 % of the fused step's
 // instructions): the same bits for normal arguments, and a state with others is outside the equation of state's range.
-template <class R> __device__ __forceinline__ R inverse_of(R x) { return R(1) / x; }
+template <class R> __device__ R inverse_of(R x);  // float, double and dw
 template <> __device__ __forceinline__ float inverse_of<float>(float x) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-template <class R> __device__ __forceinline__ R inverse_root_of(R x) { return rsqrt(x); }
-template <> __device__ __forceinline__ float inverse_root_of<float>(float x) {
+__device__ __forceinline__ float inverse_root_of(float x) {
   float y;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
@@ -200,7 +199,9 @@ template <> __device__ __forceinline__ float inverse_root_of<float>(float x) {
 // ------------------------------------------------------------------------------------------------
 // Peng-Robinson EOS (Eq. 56) and (dp/dT)_rho
 // ------------------------------------------------------------------------------------------------
+// In binary32 (eos_psi_squared: the wider types).
 template <class R, class PT> __device__ __forceinline__ void eos(R rho, R T, const PT& P, R& p, R& dpdT, R* inv_rho = nullptr) {
+  static_assert(sizeof(R) == 4, "binary32");
   const Coefs<R>& C = coefs<R>(P);
   // theta(T) = [1 + kappa (1 - sqrt(T/T_c))]^2 and d theta/dT = -kappa [..] / sqrt(T T_c); one rsqrt
   // gives both sqrt(T/T_c) = t rsqrt(t) and 1/sqrt(T T_c) = rsqrt(t) / T_c with t = T/T_c.
@@ -311,16 +312,12 @@ __device__ __forceinline__ R eos_psi_squared(R rho, R T, const PT& P, R& dpdT, R
 // g_a = T/18 = g0/10, within a factor 2 of g0/8), and a difference of two binary32 numbers within a
 // factor 2 of each other is exact (Sterbenz). The sums below take every population relative to that ratio first, so
 // the large part is one exact product of the rest population and the rounding falls on small
-// deviations. Binary64 and double-word arithmetic keep the plain sums.
-template <class R> __device__ __forceinline__ R density_of(const R f[9]) {
-  if constexpr (sizeof(R) == 4) {
-    const R q = f[0] * 0.25f;
-    const R A = ((f[1] - q) + (f[2] - q)) + ((f[3] - q) + (f[4] - q));
-    const R B = (fmaf(4.f, f[5], -q) + fmaf(4.f, f[6], -q)) + (fmaf(4.f, f[7], -q) + fmaf(4.f, f[8], -q));
-    return fmaf(2.25f, f[0], A + B * 0.25f);  // rho = 9 f0/4 + A + B/4
-  } else {
-    return f[0] + f[1] + f[2] + f[3] + f[4] + f[5] + f[6] + f[7] + f[8];
-  }
+// deviations. Binary64 and double-word arithmetic keep the plain sums (flow_moments, heat_of).
+__device__ __forceinline__ float density_of(const float f[9]) {
+  const float q = f[0] * 0.25f;
+  const float A = ((f[1] - q) + (f[2] - q)) + ((f[3] - q) + (f[4] - q));
+  const float B = (fmaf(4.f, f[5], -q) + fmaf(4.f, f[6], -q)) + (fmaf(4.f, f[7], -q) + fmaf(4.f, f[8], -q));
+  return fmaf(2.25f, f[0], A + B * 0.25f);  // rho = 9 f0/4 + A + B/4
 }
 
 // Temperature T = sum g. In binary32 also its rounding residual lo (T + lo is the sum of the deviations
@@ -341,12 +338,10 @@ template <class R> __device__ __forceinline__ R heat_of(const R g[9], R& lo) {
   }
 }
 
-// psi^2 = (2/G)(p_EOS - rho c_s^2) (reading of Ref. [48]), with p_EOS first moved by (dp/dT)_rho Tlo
-// for the residual of a binary32 temperature (zero otherwise).
-template <class R>
-__device__ __forceinline__ R psi_squared(R p, R dpdT, R Tlo, R rho, const Coefs<R>& C) {
-  if constexpr (sizeof(R) == 4) return C.psi_scale * ((p + dpdT * Tlo) - rho * R(1.0 / 3.0));
-  else return C.psi_scale * (p - rho * R(1.0 / 3.0));
+// psi^2 = (2/G)(p_EOS - rho c_s^2) (reading of Ref. [48]) in binary32, with p_EOS first moved by (dp/dT)_rho Tlo
+// for the residual of the temperature.
+__device__ __forceinline__ float psi_squared(float p, float dpdT, float Tlo, float rho, const Coefs<float>& C) {
+  return C.psi_scale * ((p + dpdT * Tlo) - rho * float(1.0 / 3.0));
 }
 
 // psi^2 and (dp/dT)_rho of a node in the form its arithmetic takes (Tlo: the residual of a binary32 T).
@@ -716,43 +711,39 @@ __device__ __forceinline__ void relax_flow(const R m[6], R jx, R jy, R rho, R vx
 // times at the scale of the populations, and the roundings of the opposite pair e_a, -e_a differ, which
 // moves momentum at random. The non-equilibrium parts m - m_eq of the energy and stress moments come
 // from the populations' exact deviations from their rest-state ratios (see density_of), not from moments
-// of size about 2 rho that cancel. Binary64 and double-word arithmetic rebuild f* from m* (relax_flow).
+// of size about 2 rho that cancel. This function is binary32's; binary64 and double-word arithmetic rebuild f* from m*
+// (relax_flow).
 template <class R, class PT>
 __device__ __forceinline__ void collide_flow(R f[9], R rho, R vx, R vy, R Fx, R Fy, R Q, const PT& P) {
+  static_assert(sizeof(R) == 4, "binary32");
   const Coefs<R>& C = coefs<R>(P);
-  if constexpr (sizeof(R) == 4) {
-    const R vxx = vx * vx, vyy = vy * vy;
-    const R v2 = vxx + vyy;
-    const R vF = vx * Fx + vy * Fy;
-    const R q = f[0] * 0.25f;
-    const R d1 = f[1] - q, d2 = f[2] - q, d3 = f[3] - q, d4 = f[4] - q;
-    const R d5 = fmaf(4.f, f[5], -q), d6 = fmaf(4.f, f[6], -q), d7 = fmaf(4.f, f[7], -q), d8 = fmaf(4.f, f[8], -q);
-    const R A = (d1 + d2) + (d3 + d4), B = (d5 + d6) + (d7 + d8);
-    const R e_dev = A + B;                       // m1 + 2 rho
-    const R eps_dev = A * -3.f;                  // m2 - rho
-    const R pxx = (d1 + d3) - (d2 + d4);         // m7
-    const R pxy = ((d5 + d7) - (d6 + d8)) * 0.25f;  // m8
-    const R qx = (f[1] - f[3]) * -2.f + ((f[5] - f[6]) + (f[8] - f[7]));  // m4
-    const R qy = (f[2] - f[4]) * -2.f + ((f[5] - f[7]) + (f[6] - f[8]));  // m6
-    const R r3v2 = rho * v2 * 3.f;
-    R dm[9], df[9];
-    dm[0] = R(0);  // S_F,0 = 0 and m0_eq = rho
-    dm[3] = Fx;    // j* = j + F whatever s_j (m_eq,3 = j + F/2)
-    dm[5] = Fy;
-    dm[1] = C.flow.hf[1] * (vF * 6 + Q) - C.flow.s_f[1] * (e_dev - r3v2);  // m1 - m1_eq = (m1 + 2 rho) - 3 rho v^2
-    dm[2] = C.flow.hf[2] * (vF * -6 - Q) - C.flow.s_f[2] * (eps_dev + r3v2);  // m2 - m2_eq = (m2 - rho) + 3 rho v^2
-    dm[4] = C.flow.hf[4] * -Fx - C.flow.s_f[4] * (qx + rho * vx);
-    dm[6] = C.flow.hf[6] * -Fy - C.flow.s_f[6] * (qy + rho * vy);
-    dm[7] = C.flow.hf[7] * ((vx * Fx - vy * Fy) * 2) - C.flow.s_f[7] * (pxx - rho * (vxx - vyy));
-    dm[8] = C.flow.hf[8] * (vx * Fy + vy * Fx) - C.flow.s_f[8] * (pxy - rho * vx * vy);
-    from_moments(dm, df);
+  const R vxx = vx * vx, vyy = vy * vy;
+  const R v2 = vxx + vyy;
+  const R vF = vx * Fx + vy * Fy;
+  const R q = f[0] * 0.25f;
+  const R d1 = f[1] - q, d2 = f[2] - q, d3 = f[3] - q, d4 = f[4] - q;
+  const R d5 = fmaf(4.f, f[5], -q), d6 = fmaf(4.f, f[6], -q), d7 = fmaf(4.f, f[7], -q), d8 = fmaf(4.f, f[8], -q);
+  const R A = (d1 + d2) + (d3 + d4), B = (d5 + d6) + (d7 + d8);
+  const R e_dev = A + B;                       // m1 + 2 rho
+  const R eps_dev = A * -3.f;                  // m2 - rho
+  const R pxx = (d1 + d3) - (d2 + d4);         // m7
+  const R pxy = ((d5 + d7) - (d6 + d8)) * 0.25f;  // m8
+  const R qx = (f[1] - f[3]) * -2.f + ((f[5] - f[6]) + (f[8] - f[7]));  // m4
+  const R qy = (f[2] - f[4]) * -2.f + ((f[5] - f[7]) + (f[6] - f[8]));  // m6
+  const R r3v2 = rho * v2 * 3.f;
+  R dm[9], df[9];
+  dm[0] = R(0);  // S_F,0 = 0 and m0_eq = rho
+  dm[3] = Fx;    // j* = j + F whatever s_j (m_eq,3 = j + F/2)
+  dm[5] = Fy;
+  dm[1] = C.flow.hf[1] * (vF * 6 + Q) - C.flow.s_f[1] * (e_dev - r3v2);  // m1 - m1_eq = (m1 + 2 rho) - 3 rho v^2
+  dm[2] = C.flow.hf[2] * (vF * -6 - Q) - C.flow.s_f[2] * (eps_dev + r3v2);  // m2 - m2_eq = (m2 - rho) + 3 rho v^2
+  dm[4] = C.flow.hf[4] * -Fx - C.flow.s_f[4] * (qx + rho * vx);
+  dm[6] = C.flow.hf[6] * -Fy - C.flow.s_f[6] * (qy + rho * vy);
+  dm[7] = C.flow.hf[7] * ((vx * Fx - vy * Fy) * 2) - C.flow.s_f[7] * (pxx - rho * (vxx - vyy));
+  dm[8] = C.flow.hf[8] * (vx * Fy + vy * Fx) - C.flow.s_f[8] * (pxy - rho * vx * vy);
+  from_moments(dm, df);
 #pragma unroll
-    for (int a = 0; a < 9; ++a) f[a] = f[a] + df[a];
-  } else {
-    R m[6], jx, jy;
-    flow_moments(f, jx, jy, m);
-    relax_flow(m, jx, jy, rho, vx, vy, Fx, Fy, Q, C, f);
-  }
+  for (int a = 0; a < 9; ++a) f[a] = f[a] + df[a];
 }
 
 // The thermal moments n4, n6 (the fluxes qx, qy of g) in binary64 and double-word arithmetic.

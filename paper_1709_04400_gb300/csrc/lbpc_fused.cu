@@ -285,8 +285,8 @@ static bool encode_t(TmaMaps* m, void* f, void* g, float* rf, float* rg, const D
   auto fn = encode_fn();
   if (!fn) return false;
   if (((size_t)P.pitch * sizeof(S)) % 16 != 0) return false;  // row stride must be a multiple of 16 bytes
-  const CUtensorMapDataType dt = sizeof(S) == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
-                                                : (sizeof(S) == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64);
+  static_assert(sizeof(S) <= 4, "FP32 and FP16 storage");
+  const CUtensorMapDataType dt = sizeof(S) == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
   const cuuint64_t dims[3] = {(cuuint64_t)P.nx, (cuuint64_t)P.ny, 9};
   const cuuint64_t strides[2] = {(cuuint64_t)P.pitch * sizeof(S), (cuuint64_t)P.N * sizeof(S)};
   const cuuint32_t box[3] = {(cuuint32_t)B::BX, (cuuint32_t)B::BY, 9};
