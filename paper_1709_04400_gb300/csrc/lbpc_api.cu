@@ -590,6 +590,33 @@ LBPC_API lbpc_status lbpc_fields(lbpc_ctx* c, double* rho, double* ux, double* u
   return LBPC_OK;
 }
 
+static PFN_cuPointerGetAttribute_v4000 query_pointer_fn() {
+  void* p = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &p, 4000, cudaEnableDefault, &q) == cudaSuccess &&
+      q == cudaDriverEntryPointSuccess)
+    return (PFN_cuPointerGetAttribute_v4000)p;
+  return nullptr;
+}
+
+static lbpc::AddressInfo address_info(const void* p) {
+  static const PFN_cuPointerGetAttribute_v4000 fn = query_pointer_fn();
+  lbpc::AddressInfo a{};
+  if (cudaPointerGetAttributes(&a.at, p) != cudaSuccess) {
+    cudaGetLastError();
+    a.at = cudaPointerAttributes{};
+    return a;
+  }
+  const CUdeviceptr q = (CUdeviceptr)(uintptr_t)p;
+  if (!fn || fn(&a.access, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS, q) != CUDA_SUCCESS) a.access = 0;
+  CUdeviceptr start = 0;
+  size_t size = 0;
+  if (fn && fn(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, q) == CUDA_SUCCESS &&
+      fn(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, q) == CUDA_SUCCESS)
+    a.past = (uintptr_t)start + size;
+  return a;
+}
+
 // ---- checkpoint / resume ----
 // Layout: a 512-byte header, then f and g of the current state (storage type, [9][N] each), the FP16
 // reference planes of f and g (FP16 storage only), phi_prev ([N] of the arithmetic type) and the wall
@@ -618,13 +645,95 @@ void ckpt_sizes(const lbpc_ctx* c, size_t& pop, size_t& ref, size_t& phi, size_t
   wall = (size_t)lbpc::wall_doubles(c->p.nx) * sizeof(double);
 }
 
-// Copy rows rows of nx elements between a plane set of the context (rows pitch elements apart) and a buffer without
-// padding.
-cudaError_t copy_rows(const lbpc_ctx* c, void* dst, bool dst_padded, const void* src, size_t elem, size_t rows,
-                      cudaMemcpyKind kind) {
-  const size_t row = (size_t)c->p.nx * elem, pitch = (size_t)c->dp.pitch * elem;
-  if (row == pitch) return cudaMemcpyAsync(dst, src, row * rows, kind, c->stream);
-  return cudaMemcpy2DAsync(dst, dst_padded ? pitch : row, src, dst_padded ? row : pitch, row, rows, kind, c->stream);
+// The address under which the device's kernels reach [p, p + bytes), or null: memory of that device or pinned host memory,
+// as on_device says, all of it to read and write, and aligned for 4-byte elements. Goes through the allocations that it
+// spans, of which there may be several.
+unsigned char* reached(int device, const void* p, size_t bytes, bool on_device) {
+  const uintptr_t begin = (uintptr_t)p, end = begin + bytes;
+  uintptr_t at = 0;
+  for (uintptr_t q = begin; q < end;) {
+    const lbpc::AddressInfo a = address_info((const void*)q);
+    if (a.at.type != (on_device ? cudaMemoryTypeDevice : cudaMemoryTypeHost) || (on_device && a.at.device != device) ||
+        (a.access & 3) != 3 || !a.at.devicePointer || a.past <= q)
+      return nullptr;
+    if (q == begin) at = (uintptr_t)a.at.devicePointer;
+    if ((uintptr_t)a.at.devicePointer != at + (q - begin)) return nullptr;
+    q = a.past;
+  }
+  return (at & 3) == 0 ? (unsigned char*)at : nullptr;
+}
+
+// A section of a checkpoint that holds rows: where it lies in the context and scratch for a copy of it there.
+struct Section {
+  void* rows;
+  void* stage;
+  size_t elem, count, off;  // bytes of an element, rows, offset in the checkpoint
+};
+int sections(const lbpc_ctx* c, int half, Section* s) {
+  const Layout L = layout_of(&c->p);
+  const lbpc::SplitBuffers& b = c->buf;
+  const size_t ny = (size_t)c->p.ny, nx = (size_t)c->p.nx;
+  int n = 0;
+  size_t off = kCkptHeader;
+  auto add = [&](void* rows, void* stage, size_t elem, size_t count) {
+    s[n++] = Section{rows, stage, elem, count, off};
+    off += nx * count * elem;
+  };
+  add(b.f[half], b.f[half ^ 1], L.store, 9 * ny);
+  add(b.g[half], b.g[half ^ 1], L.store, 9 * ny);
+  if (c->p.prec == LBPC_FP16DEV) {
+    add(b.ref_f[half], b.ref_f[half ^ 1], sizeof(float), ny);
+    add(b.ref_g[half], b.ref_g[half ^ 1], sizeof(float), ny);
+  }
+  add(b.phi_prev, b.planes[0], L.real, ny);
+  return n;
+}
+
+// Copy the row sections between half `half` of the context and the checkpoint at buf. Padded rows are packed or unpacked
+// by a kernel, all in one launch: straight from or to memory that it reaches, or through the context's scratch
+// (the other half and a plane) beside plain copies. Pitched copies of rows run at a fraction of HBM, and of the link where the
+// rows are short or it is the host that is read; they are left to what the kernel may not reach and to long rows that go to
+// the host, where they cost nothing and the kernel's writes over the link are slower. us to save and load, by pitched copies
+// and here: 4093^2 FP32 (1.27 GB) in device memory 1287 and 1297, 405 and 410; 1023 x 1025 pinned 457 and 1092, 457 and 428;
+// 99 x 1021 (7.7 MB) pinned 136 and 680, 83 and 76. Copies check what they are given.
+cudaError_t copy_sections(lbpc_ctx* c, int half, unsigned char* buf, size_t bytes, bool on_device, bool save) {
+  Section s[5];
+  const int n = sections(c, half, s);
+  const size_t nx = (size_t)c->p.nx, pitch = (size_t)c->dp.pitch;
+  const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : (save ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice);
+  const bool to_host = save && !on_device;
+  unsigned char* direct = nx == pitch || to_host ? nullptr : reached(c->device, buf, bytes, on_device);
+  const bool pitched = nx != pitch && !direct && (on_device || (to_host && nx * s[0].elem >= 1024));
+  cudaError_t e = cudaSuccess;
+  if (nx == pitch || pitched) {
+    for (int k = 0; k < n && e == cudaSuccess; ++k) {
+      const size_t row = nx * s[k].elem, wide = pitch * s[k].elem;
+      unsigned char* flat = buf + s[k].off;
+      if (!pitched)
+        e = save ? cudaMemcpyAsync(flat, s[k].rows, row * s[k].count, kind, c->stream)
+                 : cudaMemcpyAsync(s[k].rows, flat, row * s[k].count, kind, c->stream);
+      else
+        e = save ? cudaMemcpy2DAsync(flat, row, s[k].rows, wide, row, s[k].count, kind, c->stream)
+                 : cudaMemcpy2DAsync(s[k].rows, wide, flat, row, row, s[k].count, kind, c->stream);
+    }
+    return e;
+  }
+  lbpc::RowSets r{};
+  r.n = n;
+  r.nx = c->p.nx;
+  for (int k = 0; k < n; ++k) {
+    void* flat = direct ? (void*)(direct + s[k].off) : s[k].stage;
+    r.set[k] = save ? lbpc::RowSet{flat, s[k].rows, (long long)nx, (long long)pitch, (long long)s[k].count, (int)s[k].elem}
+                    : lbpc::RowSet{s[k].rows, flat, (long long)pitch, (long long)nx, (long long)s[k].count, (int)s[k].elem};
+  }
+  if (save) e = lbpc::repack_rows(r, c->stream);
+  for (int k = 0; k < n && !direct && e == cudaSuccess; ++k) {
+    const size_t size = nx * s[k].elem * s[k].count;
+    e = save ? cudaMemcpyAsync(buf + s[k].off, s[k].stage, size, kind, c->stream)
+             : cudaMemcpyAsync(s[k].stage, buf + s[k].off, size, kind, c->stream);
+  }
+  if (!save && e == cudaSuccess) e = lbpc::repack_rows(r, c->stream);
+  return e;
 }
 }  // namespace
 
@@ -640,7 +749,8 @@ LBPC_API lbpc_status lbpc_save(lbpc_ctx* c, void* buf, size_t bytes, int on_devi
   if (!c || !buf) return LBPC_EINVAL;
   if (c->err != LBPC_OK) return LBPC_ESTATE;
   if (!c->initialised) return fail(c, LBPC_ESTATE, "lbpc_save before lbpc_init");
-  if (bytes < lbpc_checkpoint_bytes(c)) return LBPC_EINVAL;
+  const size_t need = lbpc_checkpoint_bytes(c);
+  if (bytes < need) return LBPC_EINVAL;
   DeviceGuard g(c->device);
   size_t pop, ref, phi, wall;
   ckpt_sizes(c, pop, ref, phi, wall);
@@ -664,22 +774,8 @@ LBPC_API lbpc_status lbpc_save(lbpc_ctx* c, void* buf, size_t bytes, int on_devi
   CU(c, cudaMemcpyAsync(dst, header, kCkptHeader, on_device ? cudaMemcpyHostToDevice : cudaMemcpyHostToHost,
                         c->stream),
      "lbpc_save header");
-  size_t off = kCkptHeader;
-  const Layout L = layout_of(&c->p);
-  const size_t ny = (size_t)c->p.ny;
-  CU(c, copy_rows(c, dst + off, false, c->buf.f[c->cur], L.store, 9 * ny, d2x), "lbpc_save f");
-  off += pop;
-  CU(c, copy_rows(c, dst + off, false, c->buf.g[c->cur], L.store, 9 * ny, d2x), "lbpc_save g");
-  off += pop;
-  if (ref) {
-    CU(c, copy_rows(c, dst + off, false, c->buf.ref_f[c->cur], sizeof(float), ny, d2x), "lbpc_save ref_f");
-    off += ref;
-    CU(c, copy_rows(c, dst + off, false, c->buf.ref_g[c->cur], sizeof(float), ny, d2x), "lbpc_save ref_g");
-    off += ref;
-  }
-  CU(c, copy_rows(c, dst + off, false, c->buf.phi_prev, L.real, ny, d2x), "lbpc_save phi_prev");
-  off += phi;
-  CU(c, cudaMemcpyAsync(dst + off, c->buf.wall[c->cur], wall, d2x, c->stream), "lbpc_save wall");
+  CU(c, copy_sections(c, c->cur, dst, need, on_device != 0, true), "lbpc_save rows");
+  CU(c, cudaMemcpyAsync(dst + need - wall, c->buf.wall[c->cur], wall, d2x, c->stream), "lbpc_save wall");
   CU(c, cudaStreamSynchronize(c->stream), "lbpc_save sync");
   return LBPC_OK;
 }
@@ -706,22 +802,9 @@ LBPC_API lbpc_status lbpc_load(lbpc_ctx* c, const void* buf, size_t bytes, int o
   if (h.pop_bytes != pop || h.ref_bytes != ref || h.phi_bytes != phi || h.wall_bytes != wall || h.step < 0)
     return fail(c, LBPC_EINVAL, "lbpc_load: section sizes do not match");
   const cudaMemcpyKind x2d = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-  size_t off = kCkptHeader;
-  const Layout L = layout_of(&c->p);
-  const size_t ny = (size_t)c->p.ny;
-  CU(c, copy_rows(c, c->buf.f[0], true, src + off, L.store, 9 * ny, x2d), "lbpc_load f");
-  off += pop;
-  CU(c, copy_rows(c, c->buf.g[0], true, src + off, L.store, 9 * ny, x2d), "lbpc_load g");
-  off += pop;
-  if (ref) {
-    CU(c, copy_rows(c, c->buf.ref_f[0], true, src + off, sizeof(float), ny, x2d), "lbpc_load ref_f");
-    off += ref;
-    CU(c, copy_rows(c, c->buf.ref_g[0], true, src + off, sizeof(float), ny, x2d), "lbpc_load ref_g");
-    off += ref;
-  }
-  CU(c, copy_rows(c, c->buf.phi_prev, true, src + off, L.real, ny, x2d), "lbpc_load phi_prev");
-  off += phi;
-  CU(c, cudaMemcpyAsync(c->buf.wall[0], src + off, wall, x2d, c->stream), "lbpc_load wall");
+  const size_t need = lbpc_checkpoint_bytes(c);
+  CU(c, copy_sections(c, 0, (unsigned char*)buf, need, on_device != 0, false), "lbpc_load rows");
+  CU(c, cudaMemcpyAsync(c->buf.wall[0], src + need - wall, wall, x2d, c->stream), "lbpc_load wall");
   CU(c, cudaMemcpyAsync(c->buf.scalars, &h.rho_ave, sizeof(double), cudaMemcpyHostToDevice, c->stream),
      "lbpc_load rho_ave");
   CU(c, cudaMemsetAsync(c->buf.status, 0, 8 * sizeof(long long), c->stream), "lbpc_load status reset");
@@ -744,27 +827,6 @@ LBPC_API lbpc_status lbpc_sums(lbpc_ctx* c, double* mass, double* heat) {
   if (mass) *mass = s[0];
   if (heat) *heat = s[1];
   return LBPC_OK;
-}
-
-static PFN_cuPointerGetAttribute_v4000 query_pointer_fn() {
-  void* p = nullptr;
-  cudaDriverEntryPointQueryResult q;
-  if (cudaGetDriverEntryPointByVersion("cuPointerGetAttribute", &p, 4000, cudaEnableDefault, &q) == cudaSuccess &&
-      q == cudaDriverEntryPointSuccess)
-    return (PFN_cuPointerGetAttribute_v4000)p;
-  return nullptr;
-}
-
-static lbpc::AddressInfo address_info(const void* p) {
-  static const PFN_cuPointerGetAttribute_v4000 fn = query_pointer_fn();
-  lbpc::AddressInfo a{};
-  if (cudaPointerGetAttributes(&a.at, p) != cudaSuccess) {
-    cudaGetLastError();
-    a.at = cudaPointerAttributes{};
-  } else if (!fn || fn(&a.access, CU_POINTER_ATTRIBUTE_ACCESS_FLAGS, (CUdeviceptr)(uintptr_t)p) != CUDA_SUCCESS) {
-    a.access = 0;
-  }
-  return a;
 }
 
 LBPC_API lbpc_status lbpc_sums_async(lbpc_ctx* c, double* out, int on_device) {

@@ -139,6 +139,19 @@ cudaError_t split_fields(const SplitBuffers& b, const DevParams& P, int prec, in
 // which = 0: f, 1: g; only < 0: all 9 planes [9][ny][nx], else plane `only` into out[ny][nx].
 cudaError_t split_export_pops(const SplitBuffers& b, const DevParams& P, int prec, int cur, int which, int only,
                               double* out, cudaStream_t st);
+// Enqueue copies of rows of nx elements (2 or 4 bytes, at addresses that are multiples of it) from one stride, in
+// elements, to another, between memory that the device reaches: several sets of rows in one launch.
+struct RowSet {
+  void* dst;
+  const void* src;
+  long long dst_stride, src_stride, rows;
+  int elem;
+};
+struct RowSets {
+  int n, nx;
+  RowSet set[5];
+};
+cudaError_t repack_rows(const RowSets& s, cudaStream_t st);
 int split_nplanes();
 int split_block();
 

@@ -18,6 +18,7 @@
 // 0.533 ms; there k_macro is at the measured HBM bandwidth (264 B per node in 164 us) and k_collide_tile at 64 % of
 // it (280 B in 271 us) and bound by issue and latency.
 
+#include <algorithm>
 #include <type_traits>
 
 #include "lbpc_device.cuh"
@@ -593,6 +594,36 @@ __global__ void __launch_bounds__(BLOCK) k_export_fields(Planes<R> pl, DevParams
   if (T) T[o] = (double)pl.p[P_T][i];
 }
 
+// Rows of nx elements from one row stride to another, a warp per row: what packs the rows of a checkpoint and unpacks
+// them. Bound by HBM, or by the link where one side is pinned host memory.
+template <class E>
+__device__ __forceinline__ void repack_row(E* __restrict__ d, const E* __restrict__ s, int lane, int nx) {
+  int x = lane;
+  for (; x + 7 * 32 < nx; x += 8 * 32) {  // eight loads in flight
+    E v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = s[x + 32 * k];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) d[x + 32 * k] = v[k];
+  }
+  for (; x < nx; x += 32) d[x] = s[x];
+}
+__global__ void __launch_bounds__(256) k_repack(const __grid_constant__ RowSets S) {
+  const int t = pdl_wait<256>();
+  long long r = (long long)blockIdx.x * 8 + (t >> 5);
+#pragma unroll 1
+  for (int k = 0; k < S.n; ++k) {
+    const RowSet& q = S.set[k];
+    for (; r < q.rows; r += (long long)gridDim.x * 8) {
+      if (q.elem == 2)
+        repack_row((unsigned short*)q.dst + r * q.dst_stride, (const unsigned short*)q.src + r * q.src_stride, t & 31, S.nx);
+      else
+        repack_row((unsigned*)q.dst + r * q.dst_stride, (const unsigned*)q.src + r * q.src_stride, t & 31, S.nx);
+    }
+    r -= q.rows;
+  }
+}
+
 // ------------------------------------------------------------------------------------------------
 // host launchers
 // ------------------------------------------------------------------------------------------------
@@ -771,6 +802,13 @@ cudaError_t split_export_pops(const SplitBuffers& b, const DevParams& P, int pre
   else
     launch_pdl(k_export_pops<__half>, nb, BLOCK, 0, st, fbuf<__half>(b, cur), gbuf<__half>(b, cur), P, which, only, out);
   return cudaGetLastError();
+}
+
+cudaError_t repack_rows(const RowSets& s, cudaStream_t st) {
+  long long rows = 0;
+  for (int k = 0; k < s.n; ++k) rows += s.set[k].rows;
+  if (rows == 0) return cudaSuccess;
+  return launch_pdl(k_repack, (unsigned)std::min<long long>((rows + 7) / 8, 1 << 20), 256, 0, st, s);
 }
 
 void fused_finish(const SplitBuffers& b, const DevParams& P, int n, cudaStream_t st) {

@@ -10,11 +10,12 @@
 
 namespace lbpc {
 
-// What the runtime and the driver say of one address: its attributes, and the access of the current device
-// (CU_POINTER_ATTRIBUTE_ACCESS_FLAGS; 3: reads and writes).
+// What the runtime and the driver say of one address: its attributes, the access of the current device
+// (CU_POINTER_ATTRIBUTE_ACCESS_FLAGS; 3: reads and writes), and the end of its allocation (0 if unknown).
 struct AddressInfo {
   cudaPointerAttributes at;
   unsigned long long access;
+  uintptr_t past;
 };
 
 // The address under which a kernel on `device` writes out[0] and out[1], or null where a copy must do it, which checks
