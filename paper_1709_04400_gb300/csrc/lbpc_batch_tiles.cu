@@ -112,8 +112,11 @@ __global__ void __launch_bounds__(TX* TY, fused_min_blocks<S, TX * TY, 1>())
     const bool st = __shfl_sync(0xffffffffu, (int)staged(tile), 0) != 0;
     if (st) {
       if (!mbar_wait_bounded(bar, parity)) {
-        if (threadIdx.x == 0) report(I.status, *I.step, x0, y0, ST_TIMEOUT);
+        report(I.status, *I.step, x0, y0, ST_TIMEOUT);
         mbar_wait_bounded(bar, parity);  // let the copy in flight land before the block's shared memory goes away
+        // no tile is left for the threads whose wait did end, with or without thread 0
+        s_tile[0].k = s_tile[1].k = s_next.k = -1;
+        __threadfence();  // this tile's ticket is counted before the CTA's end is
         break;
       }
       parity ^= 1u;

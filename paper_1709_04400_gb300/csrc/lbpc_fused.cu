@@ -142,8 +142,11 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
     };
     if (inside(tile)) {
       if (!mbar_wait_bounded(bar, parity)) {
-        if (threadIdx.x == 0) report(status, step, tile.x, tile.y, ST_TIMEOUT);
+        report(status, step, tile.x, tile.y, ST_TIMEOUT);
         mbar_wait_bounded(bar, parity);  // let the copy in flight land before the block's shared memory goes away
+        // no tile is left for the threads whose wait did end, with or without thread 0
+        s_tile[0].x = s_tile[1].x = s_next[0].x = s_next[1].x = -1;
+        __threadfence();  // this tile's ticket is counted before the CTA's end is
         break;
       }
       parity ^= 1u;
