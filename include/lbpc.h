@@ -312,7 +312,7 @@ int64_t lbpc_batch_step_count(const lbpc_batch* b, int32_t id);
  * resident (a persistent grid). Above it, up to 64 times that limit, further CTAs start as earlier
  * ones finish, so the hardware balances tiles of uneven cost. A value above that returns LBPC_EINVAL.
  * ctas_per_sm = 0: per-tile launches. A step is a sequence of launches with one CTA per tile (variant 0 in
- * 4- and 2-byte storage: persistent CTAs where a launch has many tiles, three in four of them interior), each over
+ * 4- and 2-byte storage: persistent CTAs where a launch has enough tiles, and few enough of them at an edge), each over
  * up to lbpc_batch_per_tile_capacity instances held in its kernel parameters; each launch may start
  * while the previous one drains. A change of instances then captures the step graphs again.
  * A negative value returns LBPC_EINVAL. */

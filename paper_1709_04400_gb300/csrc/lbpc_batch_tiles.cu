@@ -145,21 +145,21 @@ template <class S, class R, int CAP> static cudaError_t walk_resident(int* out) 
   return resident_ctas(cache, k_batch_walk<S, R, 32, 8, CAP>, 256, TmaBox<S, 32, 8>::BYTES, out);
 }
 
-// Where the walk is the faster form: enough tiles per CTA, as for one instance, and enough of them staged, because an
-// edge tile's own pulls leave the CTA's next copy waiting. Measured over 52 batches per storage type, of one size or of
-// mixed ones, evaporation alone or half pools, us a step by one CTA per tile and walked. FP32: 36 of 256^2 (70 % staged) 91.7,
-// 95.9; 40 of 128^2 to 384^2 (72 %) 104.7, 108.2; 20 of 200^2 to 400^2 (77 %) 85.2, 86.5, with pools 96.7, 95.8; 19 of 352^2 (78 %)
-// 87.6, 86.4; 40 of 256^2 to 512^2 (79 %) 191, 184; 9 of 512^2 (85 %) 85.3, 78.8. Every batch below 74 % but one was slower
-// walked and every one above 78 % faster; between them ten batches of one launch take 0.984 to 1.015 times as long by tiles
-// (1.004 in the mean) and one of two launches (64 of 64^2 to 512^2, half pools) 1.037 times, so the line is at 75 %.
-// FP16: 28 of 224^2 (66 %) 76.6, 80.0; 28 of 256^2 (70 %) 94.5, 94.8; 28 of 128^2 to 384^2
-// (73 %) 114, 110; below 12 tiles per CTA 14 of 128^2 to 384^2 (73 %) 58.9, 61.0.
+// Where the walk is the faster form. Against one CTA per tile it gains on a staged tile, loses on an edge tile, whose own
+// pulls leave the CTA's next copy waiting, and pays once per CTA for its first copy and the last, ragged wave: an
+// edge tile costs what 2.3 staged tiles bring in FP32 and 1.9 in FP16, a CTA what 2.4 and 2.0 bring. The numbers are
+// fitted to 240 batches of one launch, 1 to 40 instances of one size or of mixed ones, evaporation alone and half pools,
+// 2.6 to 59 tiles per CTA, 44 to 92 % of them staged; the rule takes the slower form by more than 1 % in 4 of them, by
+// 1.9 % at most. us a step by one CTA per tile and walked, FP32: 36 of 256^2 (15 tiles per CTA, 70 %) 91.7, 95.9;
+// 12 of 64^2 to 512^2 (7.4, 78 %) 46.7, 49.5; 13 of 384^2 (12, 80 %) 72.9, 71.6; 4 of 512^2 (6.7, 85 %) 43.0, 42.1; 40 of
+// 256^2 to 512^2 (35, 79 %) 191, 184. FP16: 28 of 256^2 (12, 70 %) 94.5, 94.8; 5 of 384^2 (4.7, 80 %) 37.9, 39.8; 7 of 384^2 (6.6)
+// 53.1, 51.6; 6 of 512^2 (10, 85 %) 75.4, 66.0.
 template <class S, class R, int CAP> static cudaError_t walk_wanted_c(long long tiles, long long staged, bool* yes) {
   constexpr bool kHalf = is_half_t<S>::value;
   int resident = 0;
   const cudaError_t e = walk_resident<S, R, CAP>(&resident);
   if (e != cudaSuccess) return e;
-  *yes = tiles > (kHalf ? 12LL : 5LL) * resident && 100LL * staged >= (kHalf ? 71LL : 75LL) * tiles;
+  *yes = 10 * staged - (kHalf ? 19LL : 23LL) * (tiles - staged) >= (kHalf ? 20LL : 24LL) * resident;
   return cudaSuccess;
 }
 cudaError_t batch_walk_wanted(int prec, bool small, long long tiles, long long staged, bool* yes) {
