@@ -90,7 +90,8 @@ __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NP
 //
 // Bound by HBM in FP32 (4096^2: 413 us, 91 % of the measured copy bandwidth at 152 B per node) and by issue in
 // FP16. What the walk itself costs counts: with each ticket awaited where the next copy starts, one tensor copy
-// per population plane, and tile origins divided out by every thread, 4096^2 took 469 us (FP16 528, now 470).
+// per population plane, and tile origins divided out by every thread, 4096^2 took 469 us (FP16 528, then 470; now 455,
+// see pitch_of).
 template <class S, class R, int TX, int TY, int NPT>
 __global__ void __launch_bounds__(TX* TY / NPT, fused_min_blocks<S, TX * TY / NPT, NPT>())
     k_fused_tma_loop(PopBuf<S> fsrc, PopBuf<S> gsrc, PopBuf<S> fdst, PopBuf<S> gdst, R* __restrict__ phi_prev,
@@ -229,10 +230,10 @@ static cudaError_t fused_impl(const SplitBuffers& b, const DevParams& P, int cur
         if (e != cudaSuccess) return e;
         int resident = 0;  // CTAs of the persistent kernel that fit on the device at once
         if ((e = loop_residency<S, R, TX, TY, NPT>(B::BYTES, &resident)) != cudaSuccess) return e;
-        // Persistent CTAs pay off where each walks many tiles, more of them in FP16, whose tiles are shorter of
-        // memory time to hide. FP32, one CTA per tile against persistent: 768^2 (3.8 tiles per CTA) 21.6, 23.0 us;
-        // 1024^2 (6.7) 38.3, 36.6; 2048^2 131, 113. FP16: 1024^2 45.1, 48.8; 1536^2 (15) 85.5, 85.6; 2048^2 138, 135.
-        if ((long long)grid.x * grid.y > (is_half_t<S>::value ? 12LL : 5LL) * resident) {
+        // Persistent CTAs pay off where each walks several tiles. us, one CTA per tile against persistent, FP32: 768^2
+        // (3.8 tiles per CTA) 21.6, 23.1; 896^2 (5.2) 30.7, 30.3; 1024^2 (6.7) 38.5, 36.6; 2048^2 130, 112. FP16: 25.3, 26.4;
+        // 32.3, 32.2; 41.5, 40.1; 133, 124.
+        if ((long long)grid.x * grid.y > 5LL * resident) {
           unsigned long long* tickets = (unsigned long long*)(b.status + 6);
           if ((e = launch_pdl(k_fused_tma_loop<S, R, TX, TY, NPT>, resident, TX * TY / NPT, B::BYTES, st, fs, gs, fd, gd,
                               (R*)b.phi_prev, P, step, step == 0, b.scalars, b.partials, b.status, tickets,

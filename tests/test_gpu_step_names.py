@@ -76,3 +76,24 @@ def test_fp32_steps_on_both_sides_of_the_staging_line(mean, nx, per_sm):
         a, b = out
         assert max_rel(a[0], b[0]) <= 1e-4 and max_rel(a[3], b[3]) <= 1e-4
         assert norm_rel(a[1], b[1]) <= 1e-4 and norm_rel(a[2], b[2]) <= 1e-4
+
+
+@pytest.mark.parametrize("prec", [lbpc.FP32, lbpc.FP16DEV], ids=["fp32", "fp16"])
+def test_persistent_just_above_its_line(prec):
+    """More than five tiles per resident CTA (four CTAs per SM) run persistent: the first such grid of 1001 columns
+    (padded rows) gives the bits of one CTA per tile."""
+    import numpy as np
+    import torch
+
+    rows = 5 * 4 * torch.cuda.get_device_properties(0).multi_processor_count // 32 + 1
+    case, rho, T = workloads.mixed_small(TC, RV, RL, nx=1001, ny=8 * rows - 3)
+    out = []
+    for tile in (4, 1):
+        sim = lbpc.Simulation(lbpc.params_from_case(case, prec))
+        sim.set_fused_tile(tile)
+        sim.init(rho, T)
+        sim.step(8)
+        out.append(sim.fields())
+        sim.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
