@@ -255,11 +255,11 @@ def _dtypes():
 # the entry describes another build and the line reports null.
 MEASURED_TRAFFIC = {
     # one-pass ncu captures (dram__bytes_read.sum + dram__bytes_write.sum) of the bench's own commands
-    ("k_collide_tile", "droplet_evaporation_2048_dT0.1Tc", "fp64"): (1_113_285_888, "06556f317e36c813"),
-    ("k_collide_tile", "droplet_evaporation_2048_dT0.1Tc", "df64"): (1_113_380_608, "06556f317e36c813"),
-    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp32"): (2_511_768_320, "06556f317e36c813"),
-    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp16"): (1_581_142_016, "06556f317e36c813"),
-    ("k_batch_walk", "batched_evaporation_256", "fp32"): (3_968_465_920, "06556f317e36c813"),  # one step: 5 launches
+    ("k_collide_tile", "droplet_evaporation_2048_dT0.1Tc", "fp64"): (1_112_562_176, "13cc4fc37ac49967"),
+    ("k_collide_tile", "droplet_evaporation_2048_dT0.1Tc", "df64"): (1_112_871_424, "13cc4fc37ac49967"),
+    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp32"): (2_511_107_584, "13cc4fc37ac49967"),
+    ("k_fused", "droplet_evaporation_4096_dT0.1Tc", "fp16"): (1_583_139_072, "13cc4fc37ac49967"),
+    ("k_batch_walk", "batched_evaporation_256", "fp32"): (3_869_779_712, "13cc4fc37ac49967"),  # one step: 7 launches
 }
 
 
